@@ -107,6 +107,39 @@ struct lbmbt_ctx {
     int tuned_oz = 0;             // 0: untuned, else the own-z form the tuner chose (2 staged, 3 z-marching)
     struct Tuned { int kernel, block, spt, variant, stages, oz; };
     std::map<std::string, Tuned> tune_cache;
+    // two-step sweep (auto kernel choice): work items, per-member item prefix
+    bool pair_ok = false;
+    int multi_opt = 0;            // steps of a pass: 0 auto, 1 one, 2 two, 3 resident
+    bool general = false;         // the run has a waveform value other than 0, +-1
+    // resident sweep (auto kernel choice, small grids)
+    bool res_ok = false;
+    std::vector<ResBlock> res_blocks;
+    ResBlock* d_res_blocks = nullptr;
+    size_t cap_rb = 0;
+    int res_sites = 0, res_recv = 0;          // the largest block's sites and received values
+    size_t res_smem = 0;
+    uint4* d_packets = nullptr;
+    size_t cap_pk = 0;
+    unsigned res_stamp = 1;       // next unused stamp
+    float2* d_mout = nullptr;
+    size_t cap_mo = 0;
+    bool has_mout = false;        // the members have mout: the signal is summed from it
+    int sig_parts = 0;            // parts of a member's signal
+    long long* d_idx = nullptr;   // 0 .. n_members
+    size_t cap_ix = 0;
+    int* d_res_start = nullptr;   // [n + 1] blocks of a member
+    size_t cap_rs = 0;
+    double2* d_zpart = nullptr;
+    size_t cap_zp = 0;
+    PairMap* d_pair_maps = nullptr;
+    size_t cap_pm = 0;
+    std::vector<PairItem> pair_items;
+    PairItem* d_pair_items = nullptr;
+    size_t cap_pi = 0;
+    std::vector<long long> pair_start;
+    long long* d_pair_start = nullptr;
+    size_t cap_ps = 0;
+    long long slot_base = 0;      // two-step launches so far: level of step k is (k - slot_base) % 2
     int tma_grid = 0;
     int sm_count = 0;
     int tile_block = 0, tile_spt = 0;
@@ -141,6 +174,7 @@ struct lbmbt_ctx {
     void* field_req = nullptr;    // lbmbt_set_field: field buffer for the next lbmbt_prepare
     cudaGraphExec_t graph = nullptr;
     int graph_series = -1;
+    bool graph_pair = false;
     // adjoint buffers
     float2* d_ck = nullptr;
     size_t cap_ck = 0;
@@ -272,7 +306,10 @@ extern "C" int lbmbt_destroy(lbmbt_ctx* c)
     cudaFree(c->d_desc); cudaFree(c->d_tile_start); cudaFree(c->d_partial); cudaFree(c->d_Z);
     cudaFree(c->d_series); cudaFree(c->d_state); cudaFree(c->d_ctl); cudaFree(c->d_err);
     cudaFree(c->d_ftab); cudaFree(c->d_unit_start); cudaFree(c->d_etab); cudaFree(c->d_cc_start);
-    cudaFree(c->d_adj_unit_start); cudaFree(c->d_halo);
+    cudaFree(c->d_adj_unit_start); cudaFree(c->d_halo); cudaFree(c->d_pair_items); cudaFree(c->d_pair_start);
+    cudaFree(c->d_pair_maps);
+    cudaFree(c->d_res_blocks); cudaFree(c->d_packets); cudaFree(c->d_mout); cudaFree(c->d_idx);
+    cudaFree(c->d_res_start); cudaFree(c->d_zpart);
     cudaFree(c->d_ck); cudaFree(c->d_seg); cudaFree(c->d_gacc); cudaFree(c->d_gout); cudaFree(c->d_laminit);
     if (c->owned_stream) cudaStreamDestroy(c->owned_stream);
     delete c;
@@ -854,6 +891,251 @@ static SweepArgs sweep_args(lbmbt_ctx* c)
 }
 
 
+static bool any_slab(const lbmbt_ctx* c);
+
+// Whether a run of these members takes the resident sweep, and its blocks: the
+// smallest blocks (the same bound for every member) that do not outnumber the
+// SMs.  Where they fit it is the fastest sweep at every size measured (us a step,
+// one-step / two-step / resident): 16^3 5.7 / 8.0 / 1.5, 32^3 6.8 / 8.5 / 1.5, 48^3
+// 9.4 / 8.6 / 2.8, 64^3 12.8 / 10.3 / 4.5, eight members of 24^3 8.6 / 8.7 / 2.7.
+static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
+{
+    c->res_ok = false;
+    if (c->kernel_opt != 0 || c->scheme != 0 || c->test_wait_ns > 0 || any_slab(c) || c->n_steps < 2) return LBMBT_OK;
+    if (!c->sm_count) CU(c, cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
+    long long total = 0;
+    for (auto& d : descs) {
+        if (d.dlt) return LBMBT_OK;
+        total += d.N;
+    }
+    if (total > (long long)c->sm_count * resident_max_sites() || (int)descs.size() > c->sm_count) return LBMBT_OK;
+    int limit = 0;
+    CU(c, cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+    limit -= 2048;   // the kernel's static arrays
+    // fewest blocks of at most `cap` sites for one grid, then the fewest received values
+    struct Cut { int cy, cz, recv; };
+    auto cut = [](const MemberDesc& d, int cap) {
+        Cut best = {0, 0, 0};
+        for (int cz = 1; cz <= d.nz; ++cz) {
+            const int hz = (d.nz + cz - 1) / cz;
+            if ((d.nz + hz - 1) / hz != cz) continue;
+            const long long rows = cap / ((long long)d.nx * hz);
+            if (rows < 1) continue;
+            const int cy = (int)((d.ny + std::min<long long>(rows, d.ny) - 1) / std::min<long long>(rows, d.ny));
+            const int hy = (d.ny + cy - 1) / cy;
+            const int recv = 2 * d.nx * ((cy > 1 ? hz : 0) + (cz > 1 ? hy : 0));
+            const long long n = (long long)cy * cz, nb = (long long)best.cy * best.cz;
+            if (!best.cy || n < nb || (n == nb && recv < best.recv)) best = {cy, cz, recv};
+        }
+        return best;
+    };
+    int cap = 0;
+    std::vector<Cut> cuts(descs.size());
+    for (int t = 64; t <= resident_max_sites(); t += t < 1024 ? 64 : 128) {
+        long long n = 0;
+        int recv = 0;
+        bool ok = true;
+        for (size_t m = 0; m < descs.size() && ok; ++m) {
+            cuts[m] = cut(descs[m], t);
+            ok = cuts[m].cy > 0;
+            n += (long long)cuts[m].cy * cuts[m].cz;
+            recv = std::max(recv, cuts[m].recv);
+        }
+        if (ok && n <= c->sm_count && resident_smem(t, recv, c->lattice == 1) <= (size_t)limit) { cap = t; break; }
+    }
+    if (!cap) return LBMBT_OK;
+    c->res_blocks.clear();
+    c->res_sites = c->res_recv = 0;
+    for (size_t m = 0; m < descs.size(); ++m) {
+        const MemberDesc& d = descs[m];
+        const int cy = cuts[m].cy, cz = cuts[m].cz, first = (int)c->res_blocks.size();
+        auto at = [&](int y, int z) { return first + (z + cz) % cz * cy + (y + cy) % cy; };
+        for (int z = 0; z < cz; ++z)
+            for (int y = 0; y < cy; ++y) {
+                ResBlock b = {};
+                b.m = (int)m;
+                b.y0 = (int)((long long)d.ny * y / cy);
+                b.hy = (int)((long long)d.ny * (y + 1) / cy) - b.y0;
+                b.z0 = (int)((long long)d.nz * z / cz);
+                b.hz = (int)((long long)d.nz * (z + 1) / cz) - b.z0;
+                auto face = [&](bool end, int bc, int n, int nb) {
+                    return end && bc != BC_PER ? RES_MIRROR : n == 1 ? RES_SELF : nb;
+                };
+                b.nbr[0] = face(y == 0, d.bc[1], cy, at(y - 1, z));
+                b.nbr[1] = face(y == cy - 1, d.bc[1], cy, at(y + 1, z));
+                b.nbr[2] = face(z == 0, d.bc[2], cz, at(y, z - 1));
+                b.nbr[3] = face(z == cz - 1, d.bc[2], cz, at(y, z + 1));
+                for (int f = 0; f < 4; ++f) {
+                    b.recv[f] = b.n_recv;
+                    if (b.nbr[f] >= 0) b.n_recv += d.nx * (f < 2 ? b.hz : b.hy);
+                }
+                c->res_sites = std::max(c->res_sites, d.nx * b.hy * b.hz);
+                c->res_recv = std::max(c->res_recv, b.n_recv);
+                c->res_blocks.push_back(b);
+            }
+    }
+    for (auto& b : c->res_blocks)
+        for (int f = 0; f < 4; ++f)
+            if (b.nbr[f] >= 0) b.dest[f] = c->res_blocks[b.nbr[f]].recv[f ^ 1];
+    c->res_smem = resident_smem(c->res_sites, c->res_recv, c->lattice == 1);
+    c->res_ok = true;
+    return LBMBT_OK;
+}
+
+// Device side of the plan.
+static int build_resident(lbmbt_ctx* c)
+{
+    if (!c->res_ok) return LBMBT_OK;
+    c->res_ok = false;   // until it stands
+    const int n = c->n_members, nb = (int)c->res_blocks.size();
+    std::vector<int> start(n + 1, 0);
+    for (auto& b : c->res_blocks) start[b.m + 1]++;
+    for (int m = 0; m < n; ++m) start[m + 1] += start[m];
+    const size_t pk = sizeof(uint4) * 4 * (size_t)std::max(c->res_recv, 1) * nb;
+    const bool fresh = c->cap_pk < pk;
+    int rc = grow(c, &c->d_res_blocks, &c->cap_rb, sizeof(ResBlock) * nb);
+    if (!rc) rc = grow(c, &c->d_packets, &c->cap_pk, pk);
+    if (!rc) rc = grow(c, &c->d_res_start, &c->cap_rs, sizeof(int) * start.size());
+    if (rc) return rc;
+    if (fresh) {   // no packet there carries a stamp to come
+        CU(c, cudaMemsetAsync(c->d_packets, 0, c->cap_pk, c->stream));
+        c->res_stamp = 1;
+    }
+    CU(c, cudaMemcpyAsync(c->d_res_blocks, c->res_blocks.data(), sizeof(ResBlock) * nb, cudaMemcpyHostToDevice, c->stream));
+    CU(c, cudaMemcpyAsync(c->d_res_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, c->stream));
+    CU(c, cudaStreamSynchronize(c->stream));   // the host buffers are given back
+    c->res_ok = true;
+    return LBMBT_OK;
+}
+
+// Plan of the two-step sweep for one grid: tx x ty tiles of w x h columns (w
+// even, so that rows start on 16-byte words) that leave few of a block's
+// threads to halo columns and ragged edges.  A row of the grown tile takes w / 2
+// + 2 threads.  Narrow rows waste sectors at their ends.
+struct PairTiles { int tx, ty, w, h; };
+
+static PairTiles pair_tiles(int nx, int ny, int nt)
+{
+    PairTiles best = {0, 0, 0, 0};
+    double bc = 1e300;
+    for (int tx = 1; tx <= nx; ++tx) {
+        int w = (nx + tx - 1) / tx;
+        w += w & 1;
+        const int ex = w / 2 + 2;
+        if (ex * 3 > nt || ex > pair_max_row()) continue;
+        if (w < 8 && best.tx) break;
+        const int hm = std::min(ny, nt / ex - 2);
+        const int ty = (ny + hm - 1) / hm, n = (nx + w - 1) / w;
+        const double cost = (double)n * ty * (1.0 + 3.0 / (w + 2));
+        if (cost < bc) { bc = cost; best = {n, ty, w, (ny + ty - 1) / ty}; }
+    }
+    return best;
+}
+
+// Whether a run of these members takes the two-step sweep: the automatic
+// kernel choice, hybrid scheme, D3Q7, half-link membranes, whole grids.  Beyond
+// the resident sweep's grids it was the faster one at every size measured (us a
+// step, one-step / two-step): 65^3 13.0 / 12.8, 72^3 17.0 / 10.3, 4 x 300 x 300 16.1
+// / 9.8, 96^3 22.1 / 16.6, 128^3 46.5 / 36.2, 40 members of 30^3 43.7 / 28.1.
+static bool pair_eligible(const lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
+{
+    if (c->kernel_opt != 0 || c->scheme != 0 || c->lattice != 0 || c->test_wait_ns > 0 || any_slab(c)) return false;
+    for (auto& d : descs)
+        if (d.dlt || d.nz < 4 || d.nx < 4 || d.ny < 4) return false;   // a column is near one face of an axis only
+    return c->n_steps >= 2;
+}
+
+// Work items of the two-step sweep for the prepared members, balanced over
+// `slots` resident blocks: a chunk of zc planes costs about zc + 3.5 plane
+// times (two planes of step 1 beyond the chunk, and the first loads).
+static int build_pair(lbmbt_ctx* c)
+{
+    if (!c->pair_ok) return LBMBT_OK;
+    c->pair_ok = false;   // until the plan stands
+    if (!c->sm_count) CU(c, cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
+    int per_sm = 0;
+    CU(c, pair_prepare(c->general, &per_sm));
+    if (per_sm < 1) return fail(c, LBMBT_EINVAL, "two-step sweep does not fit on an SM");
+    const long long slots = (long long)c->sm_count * per_sm;
+    const int nt = pair_threads();
+    std::vector<PairTiles> tl(c->n_members);
+    std::map<std::pair<int, int>, PairTiles> seen;
+    int nz_max = 0;
+    for (int m = 0; m < c->n_members; ++m) {
+        const MemberDesc& d = c->descs[m];
+        auto it = seen.find({d.nx, d.ny});
+        if (it == seen.end()) it = seen.emplace(std::make_pair(d.nx, d.ny), pair_tiles(d.nx, d.ny, nt)).first;
+        tl[m] = it->second;
+        nz_max = std::max(nz_max, d.nz);
+    }
+    auto chunks = [&](int nz, int zc) { return std::max(1, (nz + zc - 1) / zc); };
+    int best_zc = nz_max;
+    double best = 1e300;
+    for (int q = 1; q <= nz_max / 4; ++q) {
+        const int zc = (nz_max + q - 1) / q;
+        double total = 0, longest = 0;
+        long long n = 0;
+        for (int m = 0; m < c->n_members; ++m) {
+            const int nc = chunks(c->descs[m].nz, zc);
+            const double cost = (double)((c->descs[m].nz + nc - 1) / nc) + 3.5;
+            const long long k = (long long)tl[m].tx * tl[m].ty * nc;
+            n += k;
+            total += k * cost;
+            longest = std::max(longest, cost);
+        }
+        const double est = n <= slots ? longest : std::max(longest, total / slots + 0.5 * longest);
+        if (est < best) { best = est; best_zc = zc; }
+        if (n > 64 * slots) break;
+    }
+    c->pair_items.clear();
+    c->pair_start.assign(c->n_members + 1, 0);
+    for (int m = 0; m < c->n_members; ++m) {
+        const MemberDesc& d = c->descs[m];
+        const int nc = chunks(d.nz, best_zc);
+        for (int q = 0; q < nc; ++q) {
+            const int z0 = (int)((long long)d.nz * q / nc), z1 = (int)((long long)d.nz * (q + 1) / nc);
+            for (int b = 0; b < tl[m].ty; ++b)
+                for (int e = 0; e < tl[m].tx; ++e) {
+                    PairItem p = {};
+                    p.m = m;
+                    p.x0 = e * tl[m].w;
+                    p.w = std::min(tl[m].w, d.nx - p.x0);
+                    p.y0 = (int)((long long)d.ny * b / tl[m].ty);
+                    p.h = (int)((long long)d.ny * (b + 1) / tl[m].ty) - p.y0;
+                    p.z0 = z0;
+                    p.z1 = z1;
+                    p.ex = tl[m].w / 2 + 2;
+                    p.hb = tl[m].h;
+                    c->pair_items.push_back(p);
+                }
+        }
+        c->pair_start[m + 1] = (long long)c->pair_items.size();
+    }
+    const size_t n = c->pair_items.size();
+    if (n > 0x3fffffff) return fail(c, LBMBT_EINVAL, "work list too long");
+    int rc = grow(c, &c->d_pair_items, &c->cap_pi, sizeof(PairItem) * n);
+    if (!rc) rc = grow(c, &c->d_pair_start, &c->cap_ps, sizeof(long long) * (c->n_members + 1));
+    if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * 2 * n);
+    if (rc) return rc;
+    std::vector<PairMap> maps(4 * (size_t)c->n_members);
+    rc = grow(c, &c->d_pair_maps, &c->cap_pm, sizeof(PairMap) * maps.size());
+    if (rc) return rc;
+    for (int m = 0; m < c->n_members; ++m) {
+        const MemberDesc& d = c->descs[m];
+        for (int more = 0; more < 2; ++more)
+            for (int lvl = 0; lvl < 2; ++lvl)
+                CU(c, pair_encode_map(&maps[2 * ((size_t)more * c->n_members + m) + lvl],
+                                      d.state + (size_t)lvl * 7 * d.plane, d, tl[m].w / 2 + 2, tl[m].h + 2 + more));
+    }
+    CU(c, cudaMemcpyAsync(c->d_pair_maps, maps.data(), sizeof(PairMap) * maps.size(), cudaMemcpyHostToDevice, c->stream));
+    CU(c, cudaMemcpyAsync(c->d_pair_items, c->pair_items.data(), sizeof(PairItem) * n, cudaMemcpyHostToDevice, c->stream));
+    CU(c, cudaMemcpyAsync(c->d_pair_start, c->pair_start.data(), sizeof(long long) * (c->n_members + 1),
+                          cudaMemcpyHostToDevice, c->stream));
+    CU(c, cudaStreamSynchronize(c->stream));   // the host buffers are given back
+    c->pair_ok = true;
+    return LBMBT_OK;
+}
+
 static int write_ctl(lbmbt_ctx* c, int sig_step, int field_step, int slot_base = 0, int slot_mod = 2)
 {
     StepCtl h;
@@ -874,9 +1156,16 @@ static int write_ctl(lbmbt_ctx* c, int sig_step, int field_step, int slot_base =
 static int init_state(lbmbt_ctx* c)
 {
     SweepArgs a = sweep_args(c);
-    CU(c, launch_init(a, c->n_tiles, c->tile_block, c->tile_spt, 0, c->stream));
+    if (c->pair_ok) {
+        long long mp = 0;
+        for (auto& d : c->descs) mp = std::max(mp, d.plane);
+        CU(c, launch_pair_init(c->d_desc, c->n_members, mp, c->stream));
+    } else {
+        CU(c, launch_init(a, c->n_tiles, c->tile_block, c->tile_spt, 0, c->stream));
+    }
     c->launches++;
     c->k_cur = 0;
+    c->slot_base = 0;
     return LBMBT_OK;
 }
 
@@ -896,6 +1185,22 @@ static int issue_step(lbmbt_ctx* c)
     if (c->series_mode) {
         CU(c, launch_reduce(c->d_partial, part_start(c), part_per(c), c->n_members, c->d_Z, c->d_series, c->n_steps, c->d_ctl,
                             c->stream));
+        c->launches++;
+    }
+    return LBMBT_OK;
+}
+
+// Issue two steps as one launch of the two-step sweep (steps = 1: the odd
+// step of a run, by the same items so that the signal partials agree).
+static int issue_pair(lbmbt_ctx* c, int steps)
+{
+    const SweepArgs a = sweep_args(c);
+    const int n = (int)c->pair_items.size();
+    CU(c, launch_sweep_pair(a, c->d_pair_items, c->d_pair_maps, n, c->general, steps, c->stream));
+    c->launches++;
+    if (c->series_mode) {
+        CU(c, launch_reduce(c->d_partial, c->d_pair_start, 1, c->n_members, c->d_Z, c->d_series, c->n_steps, c->d_ctl,
+                            c->stream, steps, n));
         c->launches++;
     }
     return LBMBT_OK;
@@ -993,12 +1298,10 @@ static int autotune(lbmbt_ctx* c)
     return LBMBT_OK;
 }
 
-static bool any_slab(const lbmbt_ctx* c);
-
 // ex (optional, [n_members]): each member's own waveform (f, n_steps; f NULL
 // for the run's) and field output.
 static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool series, void* field_dev,
-                   const lbmbt_member_ex* ex = nullptr)
+                   const lbmbt_member_ex* ex = nullptr, bool whole_run = true, bool to_end = true)
 {
     if (c->geoms.empty()) return fail(c, LBMBT_ESTATE, "no geometry set");
     if (c->n_phases == 0) return fail(c, LBMBT_ESTATE, "phases not set");
@@ -1111,15 +1414,41 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
         }
     }
     invalidate_run(c);
+    c->general = false;
+    auto general = [](double f) { return f != 0.0 && f != 1.0 && f != -1.0; };
+    for (double f : c->f) c->general = c->general || general(f);
+    if (ex)
+        for (int m = 0; m < n_members; ++m)
+            for (long long k = 0; ex[m].f && k < ex[m].n_steps; ++k) c->general = c->general || general(ex[m].f[k]);
+    c->res_ok = false;
+    if (whole_run && (c->multi_opt == 0 || c->multi_opt == 3)) {
+        rc = plan_resident(c, descs);
+        if (rc) return rc;
+    }
+    c->pair_ok = whole_run && (c->multi_opt == 0 || c->multi_opt == 2) && !c->res_ok && pair_eligible(c, descs);
     c->n_members = n_members;
     c->members.assign(mem, mem + n_members);
     c->descs = descs;
     c->series_mode = series;
     c->n_slots = 2;
     // state: n_slots * 7 planes per member
-    size_t total = 0;
-    for (auto& d : c->descs) total += (size_t)c->n_slots * 7 * d.plane * sizeof(float2);
-    rc = grow(c, &c->d_state, &c->cap_state, total);
+    for (;;) {
+        size_t total = 0;
+        for (auto& d : c->descs) {
+            d.pitch = d.nx;
+            d.plane = (d.N + 63) / 64 * 64;
+            if (c->pair_ok) {   // rows with ghost columns, of even length
+                d.pitch = (d.nx + 2 * pair_ghost() + 1) / 2 * 2;
+                d.plane = ((long long)d.pitch * (d.ny + 2 * pair_ghost()) * d.nz + 63) / 64 * 64;
+            }
+            total += (size_t)c->n_slots * 7 * d.plane * sizeof(float2);
+        }
+        rc = grow(c, &c->d_state, &c->cap_state, total);
+        if (rc != LBMBT_ENOMEM || !c->pair_ok) break;
+        cudaGetLastError();   // no room for the ghosts: the one-step sweeps need none
+        c->err.clear();
+        c->pair_ok = false;
+    }
     if (rc) return rc;
     size_t off = 0;
     for (auto& d : c->descs) {
@@ -1127,6 +1456,46 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
         off += (size_t)c->n_slots * 7 * d.plane * sizeof(float2);
     }
     if (field_dev) c->descs[0].field = (float2*)field_dev;
+    if (ex)
+        for (int m = 0; m < n_members; ++m) c->descs[m].field = static_cast<float2*>(ex[m].field_dev);
+    c->has_mout = false;
+    if (c->res_ok || c->pair_ok) {
+        // M at the signal step: the field, where a run to the end writes it at
+        // that step, else a buffer
+        std::vector<std::pair<const float2*, const float2*>> fl;
+        for (auto& d : c->descs)
+            if (d.field) fl.push_back({d.field, d.field + d.N});
+        std::sort(fl.begin(), fl.end());
+        bool own = to_end;   // each member's field is its own
+        for (size_t i = 1; i < fl.size(); ++i) own = own && fl[i - 1].second <= fl[i].first;
+        size_t need = 0;
+        for (auto& d : c->descs)
+            if (!own || !d.field) need += sizeof(float2) * (size_t)d.N;
+        rc = grow(c, &c->d_mout, &c->cap_mo, need);
+        if (rc && (rc != LBMBT_ENOMEM || c->res_ok)) return rc;
+        c->has_mout = rc == LBMBT_OK;
+        if (rc) {   // no room: the two-step sweep sums M itself
+            cudaGetLastError();
+            c->err.clear();
+        }
+        size_t at = 0;
+        for (auto& d : c->descs) {
+            d.mout = nullptr;
+            if (!c->has_mout) continue;
+            if (own && d.field) d.mout = d.field;
+            else { d.mout = c->d_mout + at; at += (size_t)d.N; }
+        }
+        long long biggest = 0;
+        for (auto& d : c->descs) biggest = std::max(biggest, d.N);
+        c->sig_parts = (int)std::max<long long>(16, std::min<long long>(biggest >> 14, 1024));
+        std::vector<long long> idx(n_members + 1);
+        std::iota(idx.begin(), idx.end(), 0LL);
+        rc = grow(c, &c->d_idx, &c->cap_ix, sizeof(long long) * idx.size());
+        if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n_members * c->sig_parts);
+        if (rc) return rc;
+        CU(c, cudaMemcpyAsync(c->d_idx, idx.data(), sizeof(long long) * idx.size(), cudaMemcpyHostToDevice, c->stream));
+        CU(c, cudaStreamSynchronize(c->stream));
+    }
     if (ex) {
         // members' own waveforms: f_k (zero past the member's end, one entry
         // past the run's) and F_k = sum_{m<k} f_m dt, as lbmbt_set_sequence
@@ -1162,7 +1531,6 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
             CU(c, cudaMemcpyAsync(c->d_wF, wF.data(), sizeof(double) * wF.size(), cudaMemcpyHostToDevice, c->stream));
             CU(c, cudaStreamSynchronize(c->stream));
         }
-        for (int m = 0; m < n_members; ++m) c->descs[m].field = static_cast<float2*>(ex[m].field_dev);
     }
     {   // slab halo planes: two of nx*ny complex values per slab member
         c->halo_off.assign(n_members, 0);
@@ -1207,6 +1575,8 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
         if (rc) return rc;
     }
     rc = build_worklist(c, c->block, c->spt);
+    if (!rc) rc = build_resident(c);
+    if (!rc) rc = build_pair(c);
     if (rc) return rc;
     rc = init_state(c);
     if (rc) return rc;
@@ -1215,14 +1585,69 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
     return LBMBT_OK;
 }
 
-static int capture_graph(lbmbt_ctx* c)
+// Z of every member from its mout, with the one-step sweep's thread sums.
+static int sum_signal(lbmbt_ctx* c)
+{
+    CU(c, launch_signal(c->d_desc, c->n_members, c->use_tma, c->use_tma ? tma_consumers(c->tma_variant) : c->tile_block,
+                        c->use_tma ? tma_sites_per_thread(c->tma_variant) : c->tile_spt, c->sig_parts, c->d_partial,
+                        c->stream));
+    CU(c, launch_reduce(c->d_partial, c->d_idx, c->sig_parts, c->n_members, c->d_Z, nullptr, 0, c->d_ctl, c->stream));
+    c->launches += 2;
+    return LBMBT_OK;
+}
+
+// n steps by the resident sweep.  A launch takes at most RES_CHUNK steps (in
+// series mode fewer: the parts of Z of every step wait in memory for their sum).
+constexpr long long RES_CHUNK = 1 << 15, RES_SERIES_CHUNK = 1 << 12;
+
+static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_step)
+{
+    const SweepArgs a = sweep_args(c);
+    const int nb = (int)c->res_blocks.size();
+    const long long chunk = c->series_mode ? RES_SERIES_CHUNK : RES_CHUNK;
+    if (c->series_mode) {
+        int rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * nb * std::min(n, chunk));
+        if (rc) return rc;
+    }
+    for (long long k = c->k_cur, end = c->k_cur + n; k < end;) {
+        ResArgs r;
+        r.blocks = c->d_res_blocks;
+        r.packets = c->d_packets;
+        r.recv_max = std::max(c->res_recv, 1);
+        r.k0 = (int)k;
+        r.n_steps = (int)std::min(chunk, end - k);
+        r.lsrc = (int)((k - c->slot_base) & 1);
+        r.ldst = (int)((k + r.n_steps - c->slot_base) & 1);
+        if (c->res_stamp > 0xffffffffu - (unsigned)r.n_steps) {   // stamps used up: start over on clean buffers
+            CU(c, cudaMemsetAsync(c->d_packets, 0, c->cap_pk, c->stream));
+            c->res_stamp = 1;
+        }
+        r.stamp0 = c->res_stamp;
+        c->res_stamp += (unsigned)r.n_steps;
+        r.sig_step = sig_step;
+        r.field_step = field_step;
+        r.series = c->series_mode ? 1 : 0;
+        r.zpart = c->d_zpart;
+        CU(c, launch_resident(a, r, nb, c->res_sites, c->res_smem, c->lattice == 1, c->general, c->stream));
+        c->launches++;
+        if (c->series_mode) {
+            CU(c, launch_resident_series(c->d_zpart, c->d_res_start, c->n_members, nb, r.n_steps, k, c->n_steps, c->d_series,
+                                         c->stream));
+            c->launches++;
+        }
+        k += r.n_steps;
+    }
+    return LBMBT_OK;
+}
+
+static int capture_graph(lbmbt_ctx* c, bool pair)
 {
     drop_graph(c);
     cudaGraph_t g;
     CU(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     const long long before = c->launches;
-    for (int i = 0; i < GRAPH_CHUNK; ++i) {
-        int rc = issue_step(c);
+    for (int i = 0; i < GRAPH_CHUNK; i += pair ? 2 : 1) {
+        int rc = pair ? issue_pair(c, 2) : issue_step(c);
         if (rc) {
             cudaStreamEndCapture(c->stream, &g);
             return rc;
@@ -1234,6 +1659,7 @@ static int capture_graph(lbmbt_ctx* c)
     cudaGraphDestroy(g);
     if (e != cudaSuccess) { c->graph = nullptr; return fail(c, LBMBT_ECUDA, "graph instantiate: %s", cudaGetErrorString(e)); }
     c->graph_series = c->series_mode ? 1 : 0;
+    c->graph_pair = pair;
     return LBMBT_OK;
 }
 
@@ -1255,29 +1681,47 @@ static int advance(lbmbt_ctx* c, long long n, bool want_signal)
     if (n > 1 && any_slab(c))
         return fail(c, LBMBT_EINVAL, "a slab advances one step at a time, with a halo exchange between steps");
     const long long last = c->k_cur + n - 1;
-    int rc = write_ctl(c, want_signal ? (int)last : -1, (c->field_dev && last == c->n_steps - 1) ? (int)last : -1);
+    int rc = write_ctl(c, want_signal ? (int)last : -1, (c->field_dev && last == c->n_steps - 1) ? (int)last : -1,
+                       (int)c->slot_base);
     if (rc) return rc;
+    const bool pair = c->pair_ok;   // its state has a layout of its own
     long long left = n;
-    if (c->use_graph && n >= GRAPH_CHUNK) {
-        if (!c->graph || c->graph_series != (c->series_mode ? 1 : 0)) {
-            rc = capture_graph(c);
+    const bool res = c->res_ok && n >= 2;
+    if (res) {
+        rc = issue_resident(c, n, want_signal ? (int)last : -1,
+                            (c->field_dev && last == c->n_steps - 1) ? (int)last : -1);
+        if (rc) return rc;
+        c->k_cur += n;
+        return want_signal ? sum_signal(c) : LBMBT_OK;
+    }
+    if (pair && (n & 1)) {   // the odd step first: the last launch is of two steps
+        rc = issue_pair(c, 1);
+        if (rc) return rc;
+        --left;
+    }
+    if (c->use_graph && left >= GRAPH_CHUNK) {
+        if (!c->graph || c->graph_series != (c->series_mode ? 1 : 0) || c->graph_pair != pair) {
+            rc = capture_graph(c, pair);
             if (rc) return rc;
         }
-        const int per = (c->use_tma ? 1 : 2) + (c->series_mode ? 1 : 0);
+        const int per = pair ? 1 + (c->series_mode ? 1 : 0) : (c->use_tma ? 1 : 2) + (c->series_mode ? 1 : 0);
         while (left >= GRAPH_CHUNK) {
             CU(c, cudaGraphLaunch(c->graph, c->stream));
-            c->launches += GRAPH_CHUNK * per;
+            c->launches += (pair ? GRAPH_CHUNK / 2 : GRAPH_CHUNK) * per;
             left -= GRAPH_CHUNK;
         }
     }
     while (left > 0) {
-        rc = issue_step(c);
+        rc = pair ? issue_pair(c, 2) : issue_step(c);
         if (rc) return rc;
-        --left;
+        left -= pair ? 2 : 1;
     }
     c->k_cur += n;
+    if (pair) c->slot_base += n / 2;   // a launch of two steps writes the other level once
+    if (want_signal && pair && c->has_mout) return sum_signal(c);
     if (want_signal && !c->series_mode) {
-        CU(c, launch_reduce(c->d_partial, part_start(c), part_per(c), c->n_members, c->d_Z, nullptr, 0, c->d_ctl, c->stream));
+        CU(c, launch_reduce(c->d_partial, pair ? c->d_pair_start : part_start(c), pair ? 1 : part_per(c), c->n_members,
+                            c->d_Z, nullptr, 0, c->d_ctl, c->stream));
         c->launches++;
     }
     return LBMBT_OK;
@@ -1307,6 +1751,11 @@ static int fetch_signal(lbmbt_ctx* c, double* signal_out, double* series_out)
     }
     int rc = sync(c);
     if (rc) return rc;
+    if ((c->res_ok || c->pair_ok) && c->has_mout && !ser.empty())   // the signal is summed apart from the series
+        for (int m = 0; m < c->n_members; ++m) {
+            const int es = c->descs[m].end_step;
+            ser[(size_t)m * c->n_steps + (es >= 0 ? es : c->n_steps - 1)] = Z[m];
+        }
     for (int m = 0; m < c->n_members; ++m) {
         const double N = (double)c->descs[m].N;
         if (signal_out) {
@@ -1390,11 +1839,11 @@ extern "C" int lbmbt_prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* me
     if (!c) return LBMBT_EINVAL;
     if (n_members == 0) {
         lbmbt_member m = plain_member(c);
-        int rc = prepare(c, 1, &m, false, c->field_req);
+        int rc = prepare(c, 1, &m, false, c->field_req, nullptr, true, false);
         return rc ? rc : sync(c);
     }
     if (!members) return fail(c, LBMBT_EINVAL, "members is NULL");
-    int rc = prepare(c, n_members, members, false, c->field_req);
+    int rc = prepare(c, n_members, members, false, c->field_req, nullptr, true, false);
     return rc ? rc : sync(c);
 }
 
@@ -1513,6 +1962,10 @@ extern "C" int lbmbt_set_option(lbmbt_ctx* c, int opt, int64_t v)
             return fail(c, LBMBT_EINVAL, "column planes must be 0 (auto) or a power of two <= 64");
         c->zc_opt = (int)v;
         break;
+    case LBMBT_OPT_MULTI_STEP:
+        if (v < 0 || v > 3) return fail(c, LBMBT_EINVAL, "steps of a pass must be 0 (auto), 1, 2 or 3 (resident)");
+        c->multi_opt = (int)v;
+        break;
     default: return fail(c, LBMBT_EINVAL, "unknown option %d", opt);
     }
     invalidate_run(c);
@@ -1538,6 +1991,8 @@ extern "C" int lbmbt_get_option(lbmbt_ctx* c, int opt, int64_t* v)
     case LBMBT_OPT_GRAD_GROUPS: *v = c->grad_groups; break;
     case LBMBT_OPT_TEST_WAIT_NS: *v = c->test_wait_ns; break;
     case LBMBT_OPT_COLUMN_PLANES: *v = c->zc_opt; break;
+    case LBMBT_OPT_MULTI_STEP: *v = c->multi_opt; break;
+    case LBMBT_OPT_MULTI_STEP_USED: *v = !c->prepared ? 0 : c->res_ok ? 3 : c->pair_ok ? 2 : 1; break;
     case LBMBT_OPT_STAGE_OWN_Z_USED: *v = c->prepared && c->use_tma ? c->tma_form + 1 : 0; break;
     case LBMBT_OPT_KERNEL_USED: *v = c->prepared ? (c->use_tma ? 2 : 1) : 0; break;
     default: return fail(c, LBMBT_EINVAL, "unknown option %d", opt);
@@ -1567,7 +2022,7 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
 {
     const int saved_block = c->block;
     if (c->block > 256) c->block = 256;
-    int rc = prepare(c, n, mem, false, nullptr);
+    int rc = prepare(c, n, mem, false, nullptr, nullptr, false);   // the adjoint reads every level
     c->block = saved_block;
     if (rc) return rc;
     const long long K = c->n_steps;

@@ -47,6 +47,8 @@ struct MemberDesc {
     int rpu_adj;          // x-rows per unit of the bulk-copy adjoint sweep
     long long unit0_adj;  // first row-unit of this member (bulk-copy adjoint)
     int nx, ny, nz;
+    int pitch;            // two-step sweep: length of the state's rows, with ghost columns
+                          // (the other sweeps' rows are nx long)
     int bc[3];            // BcMode per axis
     double gG[3];         // gamma*G0, rad/(um ms)
     double dx;            // um
@@ -84,6 +86,10 @@ struct MemberDesc {
     // run's shared tables unless the member has a waveform of its own
     const float* fw;
     const double* Fw;
+    // resident and two-step sweeps: where M goes at the signal step, for
+    // launch_signal to sum (the field buffer, if it is written at that step
+    // too); nullptr (two-step only): the sweep sums M itself
+    float2* mout;
     // step whose end signal partials (and field, if any) are this member's
     // own: its echo when it is shorter than the run; -1: the step control's
     int end_step;
@@ -153,10 +159,12 @@ cudaError_t launch_init(const SweepArgs& a, long long n_tiles, int block, int sp
 // Register sweep (one block per tile), then the one-thread step advance.
 cudaError_t launch_sweep(const SweepArgs& a, long long n_tiles, int block, int spt, cudaStream_t st);
 cudaError_t links_prepare();   // dynamic shared memory of the membrane-position sweeps
-// Sums partial[tile_start[m]*per .. tile_start[m+1]*per) per member.
+// Sums partial[tile_start[m]*per .. tile_start[m+1]*per) per member.  steps =
+// 2 (series after a two-step launch): the second step's partials follow at
+// `stride`, and both steps enter the series.
 cudaError_t launch_reduce(const double2* partial, const long long* tile_start, int per, int n_members,
                           double2* out, double2* series, long long series_stride,
-                          const StepCtl* ctl, cudaStream_t st);
+                          const StepCtl* ctl, cudaStream_t st, int steps = 1, long long stride = 0);
 
 // ---- bulk-copy sweep (sweep_tma.cu) --------------------------------------
 // oz: the own rows of planes 5 and 6 go through the stage (wanted where
@@ -164,9 +172,68 @@ cudaError_t launch_reduce(const double2* partial, const long long* tile_start, i
 // later); without it they are prefetched into registers with planes 3 and 4.
 size_t tma_smem_bytes(int cap, int capx, int nst, int form);
 int tma_partials_per_unit(int variant);
+int tma_consumers(int variant);           // threads that have sites
+int tma_sites_per_thread(int variant);
 cudaError_t tma_prepare(int cap, int capx, int nst, int variant, int form, int* ctas_per_sm);
 cudaError_t launch_sweep_tma(const SweepArgs& a, long long n_units, int cap, int capx, int nst, int variant, int form,
                              int grid, cudaStream_t st);
+
+// ---- two-step sweep (sweep_pair.cu) --------------------------------------
+// The state of a run on it has pair_ghost() ghost columns and rows on each side
+// of every plane and rows of `pitch` columns, so all its steps are its own.
+// One work item: columns [x0, x0 + w) x [y0, y0 + h), planes [z0, z1) of
+// member m; x0 even.  The items of a member are consecutive, members in order;
+// ex (pairs of columns in a row of a block, >= (w + 5) / 2) and hb (>= h) are the
+// member's, those of its tensor maps' boxes.
+struct PairItem {
+    int m, x0, w, y0, h, z0, z1, ex, hb;
+};
+int pair_threads();            // threads of a block: ex (hb + 2) may not exceed them,
+int pair_max_row();            // nor ex this
+int pair_ghost();
+struct alignas(128) PairMap {   // a tensor map (CUtensorMap)
+    unsigned char b[128];
+};
+// Maps of a run: [2][n_members][2 levels], boxes of hb + 2 and of hb + 3 rows.
+cudaError_t pair_encode_map(PairMap* out, const void* level, const MemberDesc& d, int ex, int rows);
+// general: the waveform may take values other than 0 and +-1.
+cudaError_t pair_prepare(bool general, int* ctas_per_sm);
+// steps = 2: k -> k + 2, or 1: k -> k + 1 (the odd step of a run).  Signal
+// partials (members without mout): one per item; in series mode always, and the
+// second step's follow at n_items.
+cudaError_t launch_sweep_pair(const SweepArgs& a, const PairItem* items, const PairMap* maps, int n_items, bool general,
+                              int steps, cudaStream_t st);
+cudaError_t launch_pair_init(const MemberDesc* members, int n_members, long long max_plane, cudaStream_t st);
+
+// ---- resident sweep (sweep_resident.cu) -----------------------------------
+// One block of a small grid: all of x, rows [y0, y0 + hy), planes [z0, z0 + hz)
+// of member m; nbr: the blocks across its -y, +y, -z, +z faces, or what is there
+// instead; recv: where a face's values start among the n_recv it receives;
+// dest: where they start among the neighbour's.
+constexpr int RES_SELF = -1, RES_MIRROR = -2;
+struct ResBlock {
+    int m, y0, hy, z0, hz, nbr[4], recv[4], dest[4], n_recv;
+};
+struct ResArgs {
+    const ResBlock* blocks;
+    uint4* packets;               // [n_blocks][4 turns][recv_max]
+    int recv_max;
+    int k0, n_steps;              // steps k0 .. k0 + n_steps - 1
+    int lsrc, ldst;               // time levels read and written
+    unsigned stamp0;              // stamp of step k0's packets
+    int sig_step, field_step;     // as in StepCtl; a member's own end step goes before them
+    int series;                   // 1: zpart[n][block] = the block's part of Z after each step
+    double2* zpart;
+};
+int resident_max_sites();         // sites of a block
+size_t resident_smem(int sites, int recv, bool d2);
+cudaError_t launch_resident(const SweepArgs& a, const ResArgs& r, int n_blocks, int max_sites, size_t smem, bool d2,
+                            bool general, cudaStream_t st);
+// out[m][parts], to be summed; rows: the thread sums of the bulk-copy sweep
+cudaError_t launch_signal(const MemberDesc* members, int n_members, bool rows, int block, int spt, int parts, double2* out,
+                          cudaStream_t st);
+cudaError_t launch_resident_series(const double2* zpart, const int* block_start, int n_members, int n_blocks, int n_steps,
+                                   long long k0, long long stride, double2* series, cudaStream_t st);
 
 // ---- adjoint (adjoint.cu) -------------------------------------------------
 // Per-tile gradient accumulators: [0..3] sum <lambda, w M - g> per phase

@@ -372,10 +372,12 @@ __global__ void factor_table_kernel(const MemberDesc* __restrict__ members, int 
 // ---------------------------------------------------------------- reduce
 __global__ void reduce_kernel(const double2* __restrict__ partial, const long long* __restrict__ tile_start,
                               int per, double2* __restrict__ out, double2* __restrict__ series,
-                              long long series_stride, const StepCtl* ctl)
+                              long long series_stride, const StepCtl* ctl, long long stride)
 {
     __shared__ double2 sh[256];
     const int m = blockIdx.x;
+    const int back = gridDim.y - blockIdx.y;   // this block's step ends at step word k - back + 1
+    partial += blockIdx.y * stride;
     const long long t0 = tile_start[m] * per, t1 = tile_start[m + 1] * per;
     double2 v = make_double2(0.0, 0.0);
     for (long long t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
@@ -392,8 +394,8 @@ __global__ void reduce_kernel(const double2* __restrict__ partial, const long lo
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        out[m] = sh[0];
-        if (series) series[m * series_stride + (__ldcg(&ctl->k) - 1)] = sh[0];
+        if (back == 1) out[m] = sh[0];
+        if (series) series[m * series_stride + (__ldcg(&ctl->k) - back)] = sh[0];
     }
 }
 
@@ -492,9 +494,11 @@ static cudaError_t launch_sweep_blocks(const SweepArgs& a, long long n_tiles, in
 }
 
 cudaError_t launch_reduce(const double2* partial, const long long* tile_start, int per, int n_members, double2* out,
-                          double2* series, long long series_stride, const StepCtl* ctl, cudaStream_t st)
+                          double2* series, long long series_stride, const StepCtl* ctl, cudaStream_t st, int steps,
+                          long long stride)
 {
-    reduce_kernel<<<n_members, 256, 0, st>>>(partial, tile_start, per, out, series, series_stride, ctl);
+    reduce_kernel<<<dim3(n_members, steps), 256, 0, st>>>(partial, tile_start, per, out, series, series_stride, ctl,
+                                                          stride);
     return cudaGetLastError();
 }
 

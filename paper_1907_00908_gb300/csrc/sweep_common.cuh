@@ -243,7 +243,11 @@ __device__ __forceinline__ float2 source_dtRM(float ep, float th, float mr, floa
 // 7 ns each, measured: a register sweep has ~10^5 blocks a step): block b
 // counts on shard b % CTL_SHARDS, and the last block of each shard counts on
 // `done`.
-__device__ __forceinline__ void step_done(StepCtl* ctl, int k, unsigned nblocks, bool fence)
+// `steps` = time steps of the launch; `dbase` is added to slot_base: a launch
+// of two steps writes the other time level, so the level of step k + 2 is
+// (k + 2 - (slot_base + 1)) % slot_mod.
+__device__ __forceinline__ void step_done(StepCtl* ctl, int k, unsigned nblocks, bool fence, int steps = 1,
+                                          int dbase = 0)
 {
     if (fence) __threadfence();
     const unsigned s = blockIdx.x % CTL_SHARDS;
@@ -253,7 +257,8 @@ __device__ __forceinline__ void step_done(StepCtl* ctl, int k, unsigned nblocks,
     const unsigned shards = nblocks < CTL_SHARDS ? nblocks : CTL_SHARDS;
     if (atomicAdd(&ctl->done, 1u) == shards - 1u) {
         ctl->done = 0u;
-        ctl->k = k + 1;
+        ctl->k = k + steps;
+        if (dbase) ctl->slot_base = ctl->slot_base + dbase;
     }
 }
 

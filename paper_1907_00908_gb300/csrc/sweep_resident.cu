@@ -1,0 +1,417 @@
+// sweep_resident.cu -- many time steps in one launch for grids that fit on chip.
+//
+// A step of a small grid is latency, not work: one launch per step took 6.5 us
+// at 32^3, of which the launch, the first copies and the drain are nearly all,
+// on 32 of 152 SMs.  Here one cooperative launch runs every step.  The grid is
+// cut into blocks of nx x hy x hz sites, one per CTA and SM, whose populations
+// stay in shared memory (two time levels of populations 1-6; the rest population
+// in registers).  Only the faces travel: per step a block sends one population
+// of one layer of sites through each of its four faces.
+//
+// A face value is one 16-byte packet {re, stamp, im, stamp} in a buffer of the
+// receiving block, and the receiver polls the packet itself: there is no grid
+// barrier, no flag and no fence, so a step costs one store-to-load trip through
+// L2.  Each 8-byte half carries its stamp, so a half that arrived alone is not
+// taken.  Stamps count the steps of all launches on the context and never
+// repeat, so what an earlier launch left in the buffers is never taken either.
+// Four buffers take turns (step modulo 4).  A block overwrites the packet of
+// step k at step k + 4, after it has received the neighbour's packet of step
+// k + 3; the neighbour sent that after its block barrier of step k + 2, and all
+// its threads had read step k before its barrier of step k + 1.
+//
+// Every poll is bounded (2 s); one that runs out sets the error word of the step
+// control, and the block goes on without waiting.
+//
+// Arithmetic and order per site are those of the register sweep (same bits).
+#include <algorithm>
+
+#include "lbmbt_internal.cuh"
+#include "sweep_common.cuh"
+#include "tma_common.cuh"
+
+namespace lbmbt {
+namespace {
+
+constexpr int RES_NT = 512;           // threads of a block
+constexpr int RES_MAX_SITES = 2048;   // sites of a block: 13 x 8 B each in shared memory
+
+__device__ __forceinline__ void send(uint4* to, float2 v, unsigned stamp)
+{
+    asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(to), "r"(__float_as_uint(v.x)), "r"(stamp),
+                 "r"(__float_as_uint(v.y)), "r"(stamp)
+                 : "memory");
+}
+
+__device__ __forceinline__ uint4 peek(const uint4* from)
+{
+    uint4 p;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(p.x), "=r"(p.y), "=r"(p.z), "=r"(p.w)
+                 : "l"(from)
+                 : "memory");
+    return p;
+}
+
+// Polls a packet until both halves carry the stamp; `dead` once the limit has passed.
+__device__ __noinline__ uint4 await(const uint4* from, unsigned stamp, bool& dead)
+{
+    uint4 p = peek(from);
+    const unsigned long long t0 = globaltimer();
+    for (unsigned n = 1; !dead && !(p.y == stamp && p.w == stamp); ++n) {
+        if ((n & 63u) == 0 && globaltimer() - t0 > WAIT_NS) dead = true;
+        p = peek(from);
+    }
+    return p;
+}
+
+// Site flags: bits 0..5 at a face of the grid, 6..9 on a face of the block (-y, +y,
+// -z, +z), 10 a site at all, 16..21 the membrane links, 22..23 the phase.
+enum : unsigned { S_GRID = 63u, S_SEND = 0x3c0u, S_ON = 1024u };
+
+// SPT sites a thread; D2: the D2Q5 lattice (no z populations, weights of a);
+// GEN: the waveform may take values other than 0 and +-1.
+template <int SPT, bool D2, bool GEN>
+__global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepArgs a, const ResArgs r)
+{
+    extern __shared__ __align__(16) unsigned char res_smem[];
+    __shared__ float2 s_fac[2][6];   // boundary factors of this step and of the next
+    __shared__ float s_f[2];
+    __shared__ float2 s_phase[4];    // (omega, eps) per phase
+    __shared__ double2 s_red[RES_NT / 32];
+
+    constexpr int NP = D2 ? 4 : 6;   // populations in shared memory: 1 .. NP
+    const int t = threadIdx.x;
+    const ResBlock b = r.blocks[blockIdx.x];
+    const MemberDesc* __restrict__ d = a.members + b.m;
+    const int nx = d->nx, ny = d->ny, nz = d->nz;
+    const int S = nx * b.hy * b.hz, layer = nx * b.hy;
+    // two time levels of [NP][S] and the received face values after each; the rotations
+    const int lsz = NP * S + b.n_recv;
+    float2* const lev = reinterpret_cast<float2*>(res_smem);
+    float2* const rots = lev + 2 * lsz;
+    const unsigned P = (unsigned)d->plane, sxy = (unsigned)nx * ny;
+    const float2* __restrict__ src = d->state + (size_t)r.lsrc * 7 * P;
+    const int bc[3] = {d->bc[0], d->bc[1], d->bc[2]};
+    const float sh = d->s_share;
+    const int es = d->end_step;
+    const int sig = es >= 0 ? es : r.sig_step, fstep = es >= 0 ? es : r.field_step;
+    float2* const field = d->field;
+    float2* const mout = d->mout;
+    if (t < 4) s_phase[t] = make_float2(d->omega[t], d->eps[t]);
+
+    // this thread's sites: element in the grid, flags, place in a z face (low
+    // half) and in a y face, and where the y and z pulls come from (element of a
+    // level, 16 bits each: -y, +y and -z, +z)
+    unsigned gs[SPT], fl[SPT], pl[SPT], oy[SPT], oz[SPT];
+    float2 p0[SPT];
+    float thg[SPT];
+#pragma unroll
+    for (int j = 0; j < SPT; ++j) {
+        const int l = t + j * RES_NT;
+        gs[j] = fl[j] = pl[j] = oy[j] = oz[j] = 0u;
+        p0[j] = make_float2(0.f, 0.f);
+        thg[j] = 0.f;
+        if (l < S) {
+            const int z = l / layer, in = l - z * layer, row = in / nx, x = in - row * nx;
+            const int gy = b.y0 + row, gz = b.z0 + z;
+            const unsigned s = (unsigned)gz * sxy + (unsigned)gy * nx + x;
+            gs[j] = s;
+            const unsigned mk = d->mask[s];
+            const bool yl = row == 0, yh = row == b.hy - 1, zl = z == 0, zh = z == b.hz - 1;
+            fl[j] = S_ON | (mk << 16) | (x == 0 ? 1u : 0u) | (x == nx - 1 ? 2u : 0u) | (gy == 0 ? 4u : 0u) |
+                    (gy == ny - 1 ? 8u : 0u) | (gz == 0 ? 16u : 0u) | (gz == nz - 1 ? 32u : 0u) |
+                    (yl && b.nbr[0] >= 0 ? 64u : 0u) | (yh && b.nbr[1] >= 0 ? 128u : 0u) |
+                    (zl && b.nbr[2] >= 0 ? 256u : 0u) | (zh && b.nbr[3] >= 0 ? 512u : 0u);
+            const int ez = z * nx + x;
+            pl[j] = (unsigned)in | ((unsigned)ez << 16);
+            // the neighbour's site, a received value, the far side of this block, or
+            // (mirror) the own opposite population
+            auto from = [&](bool face, int nb, int step, int wrap, int pop, int opp, int recv) -> unsigned {
+                if (!face) return (unsigned)((pop - 1) * S + l + step);
+                if (nb >= 0) return (unsigned)(NP * S + recv);
+                return (unsigned)(nb == RES_SELF ? (pop - 1) * S + l + wrap : (opp - 1) * S + l);
+            };
+            const int wy = (b.hy - 1) * nx, wz = (b.hz - 1) * layer;
+            oy[j] = from(yl, b.nbr[0], -nx, wy, 3, 4, b.recv[0] + ez) | (from(yh, b.nbr[1], nx, -wy, 4, 3, b.recv[1] + ez) << 16);
+            if (!D2)
+                oz[j] = from(zl, b.nbr[2], -layer, wz, 5, 6, b.recv[2] + in) |
+                        (from(zh, b.nbr[3], layer, -wz, 6, 5, b.recv[3] + in) << 16);
+            rots[l] = rotation_m1(d, 1.f, x, gy, gz);
+            if (GEN) thg[j] = __fmaf_rn(d->ctheta[2], (float)(gz + d->z0),
+                                        __fmaf_rn(d->ctheta[1], (float)gy, __fmul_rn(d->ctheta[0], (float)x)));
+            p0[j] = __ldcg(src + s);
+#pragma unroll
+            for (int i = 1; i <= NP; ++i) lev[(i - 1) * S + l] = __ldcg(src + (size_t)i * P + s);
+        }
+    }
+    if (t < 6) s_fac[0][t] = __ldg(a.fac + ((size_t)r.k0 * a.n_members + b.m) * 6 + t);
+    if (t == 6) s_f[0] = __ldg(d->fw + r.k0);
+
+    bool dead = false;
+    const uint4* const mine = r.packets + (size_t)blockIdx.x * 4 * r.recv_max;
+    // sends the populations that leave the block at a site on its faces, with the stamp of step n
+    auto send_faces = [&](unsigned f, unsigned place, int n, float2 v3, float2 v4, float2 v5, float2 v6) {
+        const unsigned stamp = r.stamp0 + (unsigned)n;
+        const size_t turn = (size_t)(n & 3) * r.recv_max;
+        const int in = (int)(place & 0xffffu), ez = (int)(place >> 16);
+        auto to = [&](int face, int e) {
+            return r.packets + ((size_t)b.nbr[face] * 4 * r.recv_max + turn + b.dest[face] + e);
+        };
+        if (f & 64u) send(to(0, ez), v4, stamp);
+        if (f & 128u) send(to(1, ez), v3, stamp);
+        if (f & 256u) send(to(2, in), v6, stamp);
+        if (f & 512u) send(to(3, in), v5, stamp);
+    };
+#pragma unroll
+    for (int j = 0; j < SPT; ++j)
+        if (fl[j] & S_SEND) {   // the values that the first step pulls
+            const float2* v = lev + t + j * RES_NT;
+            send_faces(fl[j], pl[j], 0, v[2 * S], v[3 * S], D2 ? v[0] : v[4 * S], D2 ? v[0] : v[5 * S]);
+        }
+
+    for (int n = 0; n < r.n_steps; ++n) {
+        const int k = r.k0 + n;
+        float2* const cur = lev + (n & 1) * lsz;
+        float2* const nxt = lev + ((n & 1) ^ 1) * lsz;
+        // the next step's factors and waveform value
+        float2 fnext = make_float2(0.f, 0.f);
+        if (n + 1 < r.n_steps) {
+            if (t < 6) fnext = __ldg(a.fac + ((size_t)(k + 1) * a.n_members + b.m) * 6 + t);
+            if (t == 6) fnext.x = __ldg(d->fw + k + 1);
+        }
+        // the neighbours' face values, two polls in flight a thread
+        {
+            const unsigned stamp = r.stamp0 + (unsigned)n;
+            const uint4* box = mine + (size_t)(n & 3) * r.recv_max;
+            for (int e = t; e < b.n_recv; e += 2 * RES_NT) {
+                const bool two = e + RES_NT < b.n_recv;
+                uint4 p = peek(box + e), q = two ? peek(box + e + RES_NT) : p;
+                if (!(p.y == stamp && p.w == stamp)) p = await(box + e, stamp, dead);
+                cur[NP * S + e] = make_float2(__uint_as_float(p.x), __uint_as_float(p.z));
+                if (two) {
+                    if (!(q.y == stamp && q.w == stamp)) q = await(box + e + RES_NT, stamp, dead);
+                    cur[NP * S + e + RES_NT] = make_float2(__uint_as_float(q.x), __uint_as_float(q.z));
+                }
+            }
+        }
+        __syncthreads();   // the level, its face values and the factors are complete
+        const float2* fac = s_fac[n & 1];
+        const float f = s_f[n & 1];
+        const bool do_sig = k == sig, do_fld = field != nullptr && k == fstep;
+        double zr = 0.0, zi = 0.0;
+#pragma unroll
+        for (int j = 0; j < SPT; ++j) {
+            const int l = t + j * RES_NT;
+            const unsigned F = fl[j];
+            if (!(F & S_ON)) continue;
+            const float2* c = cur + l;
+            float2 g[Q];
+            g[0] = p0[j];
+            // x: the block spans the axis
+            g[1] = (F & 1u) ? (bc[0] == BC_PER ? c[nx - 1] : c[S]) : c[-1];
+            g[2] = (F & 2u) ? (bc[0] == BC_PER ? c[S - (nx - 1)] : c[0]) : c[S + 1];
+            g[3] = cur[oy[j] & 0xffffu];
+            g[4] = cur[oy[j] >> 16];
+            if (!D2) {
+                g[5] = cur[oz[j] & 0xffffu];
+                g[6] = cur[oz[j] >> 16];
+            } else {
+                g[5] = g[6] = make_float2(0.f, 0.f);
+            }
+            if (F & S_GRID) {
+                if (F & 1u) g[1] = face_fix(g[1], bc[0], fac[0]);
+                if (F & 2u) g[2] = face_fix(g[2], bc[0], fac[1]);
+                if (F & 4u) g[3] = face_fix(g[3], bc[1], fac[2]);
+                if (F & 8u) g[4] = face_fix(g[4], bc[1], fac[3]);
+                if (!D2) {
+                    if (F & 16u) g[5] = face_fix(g[5], bc[2], fac[4]);
+                    if (F & 32u) g[6] = face_fix(g[6], bc[2], fac[5]);
+                }
+            }
+            if (F & 0x3f0000u) {   // half-link membranes (Eq. B5)
+                if (F & 0x20000u) g[1] = mix(c[S], g[1], sh);
+                if (F & 0x10000u) g[2] = mix(c[0], g[2], sh);
+                if (F & 0x80000u) g[3] = mix(c[3 * S], g[3], sh);
+                if (F & 0x40000u) g[4] = mix(c[2 * S], g[4], sh);
+                if (!D2) {
+                    if (F & 0x200000u) g[5] = mix(c[5 * S], g[5], sh);
+                    if (F & 0x100000u) g[6] = mix(c[4 * S], g[6], sh);
+                }
+            }
+            float2 q;
+            if (GEN && f != 0.f && f != 1.f && f != -1.f) {   // rotation_m1's general form
+                float sn, cs;
+                sincosf(0.5f * __fmul_rn(f, thg[j]), &sn, &cs);
+                q = make_float2(__fmul_rn(-2.f, __fmul_rn(sn, sn)), __fmul_rn(2.f, __fmul_rn(sn, cs)));
+            } else {
+                const float2 v = rots[l];
+                q = make_float2(__fmul_rn(v.x, fabsf(f)), __fmul_rn(v.y, f));
+            }
+            const float2 pe = s_phase[F >> 22 & 3u];
+            float mr, mi;
+            react(g, reaction_q(q, pe.y), mr, mi);
+            collide_w(g, pe.x, mr, mi, a.w0, a.wxy, a.wz);
+            p0[j] = g[0];
+            // the faces first: a neighbour waits for them (nobody after the last step)
+            if ((F & S_SEND) && n + 1 < r.n_steps) send_faces(F, pl[j], n + 1, g[3], g[4], g[5], g[6]);
+#pragma unroll
+            for (int i = 1; i <= NP; ++i) nxt[(i - 1) * S + l] = g[i];
+            if (do_sig) mout[gs[j]] = make_float2(mr, mi);
+            if (do_fld) field[gs[j]] = make_float2(mr, mi);
+            if (r.series) {
+                zr += mr;
+                zi += mi;
+            }
+        }
+        if (t < 6) s_fac[(n & 1) ^ 1][t] = fnext;
+        if (t == 6) s_f[(n & 1) ^ 1] = fnext.x;
+        if (r.series) {   // this block's part of Z after the step
+            for (int o = 16; o > 0; o >>= 1) {
+                zr += __shfl_down_sync(0xffffffffu, zr, o);
+                zi += __shfl_down_sync(0xffffffffu, zi, o);
+            }
+            if ((t & 31) == 0) s_red[t >> 5] = make_double2(zr, zi);
+            __syncthreads();
+            if (t == 0) {
+                double2 v = make_double2(0.0, 0.0);
+                for (int w = 0; w < RES_NT / 32; ++w) {
+                    v.x += s_red[w].x;
+                    v.y += s_red[w].y;
+                }
+                r.zpart[(size_t)n * gridDim.x + blockIdx.x] = v;
+            }
+        }
+    }
+
+    // each site's values are this thread's own
+    float2* __restrict__ dst = d->state + (size_t)r.ldst * 7 * P;
+    const float2* __restrict__ end = lev + (r.n_steps & 1) * lsz;
+#pragma unroll
+    for (int j = 0; j < SPT; ++j) {
+        const int l = t + j * RES_NT;
+        if (!(fl[j] & S_ON)) continue;
+        dst[gs[j]] = p0[j];
+#pragma unroll
+        for (int i = 1; i <= NP; ++i) dst[(size_t)i * P + gs[j]] = end[(i - 1) * S + l];
+        if (D2)
+            for (int i = 5; i < Q; ++i) dst[(size_t)i * P + gs[j]] = make_float2(0.f, 0.f);
+    }
+    if (dead) atomicOr(&a.ctl->err, 1);
+}
+
+// Parts of Z per member (out[m][parts]) from the magnetisation M of its sites,
+// with the thread sums of the one-step sweep that the grid would otherwise take
+// (FP32 over a thread's few sites, FP64 above), so that a signal does not
+// depend on which sweep ran: the register sweep's thread has sites s, s + block,
+// .. of a tile of block x spt, the bulk-copy sweep's l, l + block, .. of a unit of
+// rpu rows.
+__global__ void signal_kernel(const MemberDesc* __restrict__ members, int rows, int block, int spt,
+                              double2* __restrict__ out)
+{
+    __shared__ double2 sh[256];
+    const MemberDesc& d = members[blockIdx.x];
+    const float2* __restrict__ M = d.mout;
+    const long long N = d.N;
+    // units of a plane (rows != 0) or tiles of the whole grid
+    const long long span = rows ? (long long)d.nx * d.ny : N;
+    const int unit = rows ? d.rpu * d.nx : block * spt;
+    const long long per = (span + unit - 1) / unit, n_units = per * (N / span);
+    double2 v = make_double2(0.0, 0.0);
+    for (long long u = blockIdx.y; u < n_units; u += gridDim.y) {
+        const long long s0 = (u / per) * span + (u % per) * unit, s1 = min(s0 + unit, (u / per + 1) * span);
+        for (int t = threadIdx.x; t < block; t += 256) {
+            float zr = 0.f, zi = 0.f;
+            for (int j = 0; j < spt; ++j) {
+                const long long s = s0 + t + (long long)j * block;
+                if (s < s1) {
+                    const float2 m = M[s];
+                    zr += m.x;
+                    zi += m.y;
+                }
+            }
+            v.x += zr;
+            v.y += zi;
+        }
+    }
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (threadIdx.x < o) {
+            sh[threadIdx.x].x += sh[threadIdx.x + o].x;
+            sh[threadIdx.x].y += sh[threadIdx.x + o].y;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) out[(size_t)blockIdx.x * gridDim.y + blockIdx.y] = sh[0];
+}
+
+// series[m][k0 + n] = sum of the member's blocks' parts of step n (one warp each).
+__global__ void resident_series_kernel(const double2* __restrict__ zpart, const int* __restrict__ block_start,
+                                       int n_members, int n_blocks, int n_steps, long long k0, long long stride,
+                                       double2* __restrict__ series)
+{
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (w >= n_members * n_steps) return;
+    const int m = w / n_steps, n = w - m * n_steps;
+    double2 v = make_double2(0.0, 0.0);
+    for (int b = block_start[m] + lane; b < block_start[m + 1]; b += 32) {
+        const double2 p = zpart[(size_t)n * n_blocks + b];
+        v.x += p.x;
+        v.y += p.y;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+    }
+    if (lane == 0) series[m * stride + k0 + n] = v;
+}
+
+using ResFn = void (*)(const SweepArgs, const ResArgs);
+
+template <bool D2, bool GEN>
+ResFn res_spt(int spt)
+{
+    return spt <= 1 ? sweep_resident_kernel<1, D2, GEN>
+           : spt <= 2 ? sweep_resident_kernel<2, D2, GEN> : sweep_resident_kernel<4, D2, GEN>;
+}
+ResFn res_kernel(int spt, bool d2, bool gen)
+{
+    if (d2) return gen ? res_spt<true, true>(spt) : res_spt<true, false>(spt);
+    return gen ? res_spt<false, true>(spt) : res_spt<false, false>(spt);
+}
+
+}  // namespace
+
+int resident_max_sites() { return RES_MAX_SITES; }
+
+size_t resident_smem(int sites, int recv, bool d2) { return ((size_t)(d2 ? 9 : 13) * sites + 2 * recv) * sizeof(float2); }
+
+cudaError_t launch_resident(const SweepArgs& a, const ResArgs& r, int n_blocks, int max_sites, size_t smem, bool d2,
+                            bool general, cudaStream_t st)
+{
+    const void* fn = (const void*)res_kernel((max_sites + RES_NT - 1) / RES_NT, d2, general);
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    SweepArgs aa = a;
+    ResArgs rr = r;
+    void* args[2] = {&aa, &rr};
+    return cudaLaunchCooperativeKernel(fn, dim3(n_blocks), dim3(RES_NT), args, smem, st);
+}
+
+cudaError_t launch_signal(const MemberDesc* members, int n_members, bool rows, int block, int spt, int parts, double2* out,
+                          cudaStream_t st)
+{
+    signal_kernel<<<dim3(n_members, parts), 256, 0, st>>>(members, rows ? 1 : 0, block, spt, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_resident_series(const double2* zpart, const int* block_start, int n_members, int n_blocks, int n_steps,
+                                   long long k0, long long stride, double2* series, cudaStream_t st)
+{
+    const long long warps = (long long)n_members * n_steps;
+    resident_series_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(zpart, block_start, n_members, n_blocks, n_steps,
+                                                                        k0, stride, series);
+    return cudaGetLastError();
+}
+
+}  // namespace lbmbt

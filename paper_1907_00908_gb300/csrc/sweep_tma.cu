@@ -530,6 +530,9 @@ size_t tma_smem_bytes(int cap, int capx, int nst, int form) { return stage_bytes
 // signal partial slots per unit: one per consumer warp of the variant
 int tma_partials_per_unit(int variant) { return variant == 1 ? 12 : variant == 2 ? 8 : variant == 3 ? 11 : 16; }
 
+int tma_consumers(int variant) { return tma_partials_per_unit(variant) * 32; }
+int tma_sites_per_thread(int variant) { return variant == 0 ? 2 : variant == 2 ? 4 : 3; }
+
 // variant 0: 16 consumer warps x 2 sites, 1: 12 x 3, 2: 8 x 4, 3 (default):
 // 11 x 3 (units <= 1024 sites).  The register file is split over the SM's 4
 // sub-partitions: with the producer warp, 9 to 12 warps per CTA allow 168

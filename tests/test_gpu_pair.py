@@ -1,0 +1,126 @@
+"""The two-step sweep (LBMBT_OPT_MULTI_STEP = 2) against the one-step register
+sweep: the same bits in the field; the signal is summed from the same FP32
+thread sums as the one-step sweep that the grid would take otherwise, which
+for an nx not a multiple of 16 is the register sweep (FP64 rounding only, 1e-13
+of the sum of |M|), else the bulk-copy one (two or three sites a thread: 2^-22
+of the sum of |M|); the series within that."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_1907_00908_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+INF = math.inf
+
+
+@pytest.fixture(scope="module")
+def lb():
+    from paper_1907_00908_gb300 import lbmbt
+    lbmbt.lib()
+    return lbmbt
+
+
+def _geom(shape, seed, n_labels=3):
+    rng = np.random.default_rng(seed)
+    coarse = rng.integers(0, n_labels, size=[(n + 2) // 3 for n in shape])
+    lab = np.kron(coarse, np.ones((3, 3, 3), int))[:shape[0], :shape[1], :shape[2]]
+    return synth.Geometry(np.ascontiguousarray(lab, np.int32), np.arange(n_labels).astype(np.uint8) % 3, 0.5)
+
+
+def _solver(lb, kernel, geoms, bc, gG, f, kap=0.03):
+    s = lb.Solver(0)
+    s.set_option(lb.OPT_KERNEL, kernel)
+    s.set_option(lb.OPT_MULTI_STEP, 2)
+    for i, g in enumerate(geoms):
+        (s.add_geometry if i else s.set_geometry)(g.labels, g.phase_of_label, g.dx, bc)
+    s.set_phases([2.0, 1.0, 1.5], [80.0, 50.0, INF])
+    s.set_permeability(kap)
+    s.set_sequence(0.01, f, gG)
+    return s
+
+
+def _wave(kind, n):
+    if kind == "pgse":
+        f = np.zeros(n)
+        f[:max(1, n // 3)] = 1.0
+        f[n - max(1, n // 3):] = -1.0
+        return f
+    return np.cos(np.arange(n) * 0.7)
+
+
+# tile edges and remainders: one column, one tile, several ragged tiles; the
+# smallest nz; faces of every kind
+CASES = [
+    ((4, 1, 1), (0, 0, 0), (0.3, 0.2, 0.1), "pgse", 7),
+    ((4, 5, 3), (0, 0, 0), (0.0, 0.2, 0.4), "pgse", 2),
+    ((5, 2, 40), (0, 0, 0), (0.3, 0.0, 0.1), "cos", 9),
+    ((37, 23, 31), (0, 0, 0), (0.2, 0.1, -0.3), "pgse", 18),
+    ((20, 34, 70), (1, 0, 0), (0.4, 0.0, 0.0), "pgse", 16),
+    ((21, 33, 17), (1, 1, 1), (0.0, 0.3, 0.0), "pgse", 33),
+    ((40, 12, 64), (1, 1, 1), (0.0, 0.0, 0.5), "cos", 8),
+    ((33, 40, 35), (0, 1, 1), (0.3, 0.0, 0.0), "cos", 21),
+    ((64, 64, 96), (0, 0, 0), (0.0, 0.0, 0.0), "pgse", 5),
+    ((150, 18, 48), (0, 0, 1), (0.2, -0.1, 0.0), "pgse", 34),
+]
+
+
+@pytest.mark.parametrize("shape,bc,gG,wave,n", CASES)
+@pytest.mark.parametrize("kap", [0.03, 0.0, INF])
+def test_two_step_sweep_gives_the_one_step_bits(lb, shape, bc, gG, wave, n, kap):
+    g = _geom(shape, sum(shape))
+    f = _wave(wave, n)
+    out = []
+    for kernel in (0, 1):
+        with _solver(lb, kernel, [g], bc, gG, f, kap) as s:
+            fld = torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda")
+            r = s.run(field=fld, series=True)
+            q = s.run(field=fld)
+            torch.cuda.synchronize()
+            used = 2 if kernel == 0 and min(shape) >= 4 else 1
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == used
+            out.append((fld.cpu().numpy(), r, q))
+    assert np.array_equal(out[0][0], out[1][0])
+    tol = (1e-13 if shape[2] % 16 else 2.0 ** -22) * np.abs(out[0][0]).sum() + 1e-30
+    assert abs(out[0][2]["Z"] - out[1][2]["Z"]) <= tol
+    assert out[0][1]["Z"] == out[0][2]["Z"]
+    assert np.abs(out[0][1]["series"] - out[1][1]["series"]).max() <= 2.0 ** -22 * g.n_sites
+
+
+def test_batch_members_end_on_either_step_and_runs_continue_in_any_split(lb):
+    geoms = [_geom((24, 20, 33), 5), _geom((9, 41, 16), 6), _geom((48, 16, 16), 7)]
+    n = 21
+    f = _wave("pgse", n)
+    waves = [None, _wave("pgse", 10), _wave("cos", 11), _wave("pgse", 1), None, _wave("pgse", 20)]
+    gs = [(0.2, 0.1, 0.0), (0.0, 0.3, 0.1), (0.1, 0.1, 0.1), (0.3, 0.0, 0.0), (0.0, 0.0, 0.4), (0.2, 0.0, 0.2)]
+    geo = [0, 1, 2, 0, 2, 1]
+    res = []
+    for kernel in (0, 1):
+        with _solver(lb, kernel, geoms, (0, 0, 0), gs[0], f) as s:
+            fields = [torch.zeros(geoms[i].n_sites, dtype=torch.complex64, device="cuda") for i in geo]
+            m = lb.Solver.members(gs, geo, [0.03, 0.0, INF, 0.1, 0.03, 0.2])
+            r = s.run_batch(m, waveforms=waves, fields=fields)
+            q = s.run_batch(m, waveforms=waves, fields=fields, series=True)
+            torch.cuda.synchronize()
+            sums = [float(v.abs().sum()) for v in fields]
+            res.append(([v.cpu().numpy() for v in fields], r["Z"], q["Z"], sums))
+    for a, b in zip(res[0][0], res[1][0]):
+        assert np.array_equal(a, b)
+    assert np.all(np.abs(res[0][1] - res[1][1]) <= 2.0 ** -22 * np.array(res[0][3]))
+    assert np.array_equal(res[0][1], res[0][2])
+    # the same run stepped by hand
+    g = geoms[0]
+    ref = None
+    for split in ([21], [1, 1, 19], [2, 17, 2], [3, 16, 1, 1], [20, 1]):
+        with _solver(lb, 0, [g], (0, 0, 0), gs[0], f) as s:
+            fld = torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda")
+            s.set_field(fld)
+            s.prepare()
+            for k in split:
+                s.advance(k)
+            torch.cuda.synchronize()
+            v = fld.cpu().numpy()
+        ref = v if ref is None else ref
+        assert np.abs(ref).max() > 0 and np.array_equal(ref, v)

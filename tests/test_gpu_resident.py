@@ -1,0 +1,118 @@
+"""The resident sweep (all steps of a run in one launch) against the one-step
+sweeps: the same bits in the field; the signal is summed from the same FP32
+thread sums, so it differs by FP64 rounding only (1e-13 of the sum of |M|);
+the series is summed in FP64 throughout, so it differs by the FP32 rounding of
+the one-step sweep's thread sums (three sites at most: 2^-22 of the sum)."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_1907_00908_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+INF = math.inf
+
+
+@pytest.fixture(scope="module")
+def lb():
+    from paper_1907_00908_gb300 import lbmbt
+    lbmbt.lib()
+    return lbmbt
+
+
+def _geom(shape, seed):
+    rng = np.random.default_rng(seed)
+    coarse = rng.integers(0, 3, size=[(n + 2) // 3 for n in shape])
+    lab = np.kron(coarse, np.ones((3, 3, 3), int))[:shape[0], :shape[1], :shape[2]]
+    return synth.Geometry(np.ascontiguousarray(lab, np.int32), np.arange(3, dtype=np.uint8), 0.5)
+
+
+def _solver(lb, multi, geoms, bc, gG, f, kap, lattice):
+    s = lb.Solver(0)
+    s.set_option(lb.OPT_MULTI_STEP, multi)
+    s.set_option(lb.OPT_LATTICE, lattice)
+    for i, g in enumerate(geoms):
+        (s.add_geometry if i else s.set_geometry)(g.labels, g.phase_of_label, g.dx, bc)
+    s.set_phases([2.0, 1.0, 1.5], [80.0, 50.0, INF])
+    s.set_permeability(kap)
+    s.set_sequence(0.01, f, gG)
+    return s
+
+
+def _wave(kind, n):
+    f = np.zeros(n)
+    f[:max(1, n // 3)] = 1.0
+    f[n - max(1, n // 3):] = -1.0
+    return f if kind == "pgse" else np.cos(np.arange(n) * 0.7)
+
+
+# one block, one row or plane a block, ragged cuts, faces of every kind, the
+# largest blocks (2048 sites), both lattices
+CASES = [
+    ((1, 1, 1), (0, 0, 0), (0.3, 0.2, 0.1), "pgse", 7, 0),
+    ((2, 1, 9), (0, 0, 0), (0.3, 0.0, 0.1), "cos", 5, 0),
+    ((7, 5, 3), (1, 1, 1), (0.0, 0.2, 0.0), "pgse", 6, 0),
+    ((32, 32, 32), (0, 0, 0), (0.2, 0.1, -0.3), "pgse", 40, 0),
+    ((31, 29, 33), (1, 0, 0), (0.4, 0.0, 0.0), "cos", 17, 0),
+    ((23, 41, 16), (0, 1, 1), (0.3, 0.0, 0.0), "pgse", 20, 0),
+    ((57, 57, 57), (0, 0, 0), (0.1, -0.2, 0.1), "pgse", 12, 0),
+    ((64, 64, 64), (1, 1, 1), (0.0, 0.0, 0.3), "pgse", 9, 0),
+    ((1, 200, 200), (0, 0, 0), (0.3, 0.2, 0.0), "pgse", 30, 1),
+    ((1, 61, 500), (1, 1, 0), (0.0, 0.2, 0.0), "cos", 11, 1),
+    ((1, 3, 1024), (0, 1, 0), (0.1, 0.0, 0.0), "pgse", 4, 1),
+]
+
+
+@pytest.mark.parametrize("shape,bc,gG,wave,n,lattice", CASES)
+@pytest.mark.parametrize("kap", [0.03, 0.0, INF])
+def test_resident_sweep_gives_the_one_step_bits(lb, shape, bc, gG, wave, n, lattice, kap):
+    g = _geom(shape, sum(shape))
+    f = _wave(wave, n)
+    out = []
+    for multi in (0, 1):
+        with _solver(lb, multi, [g], bc, gG, f, kap, lattice) as s:
+            fld = torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda")
+            r = s.run(field=fld, series=True)
+            q = s.run(field=fld)
+            torch.cuda.synchronize()
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == (1 if multi else 3)
+            out.append((fld.cpu().numpy(), r, q))
+    assert np.array_equal(out[0][0], out[1][0])
+    total = np.abs(out[0][0]).sum()
+    assert abs(out[0][2]["Z"] - out[1][2]["Z"]) <= 1e-13 * total
+    assert np.abs(out[0][1]["series"] - out[1][1]["series"]).max() <= 2.0 ** -22 * g.n_sites
+
+
+def test_resident_batch_with_own_echoes_and_any_split(lb):
+    geoms = [_geom((24, 20, 33), 5), _geom((9, 41, 16), 6), _geom((12, 16, 16), 7)]
+    n = 21
+    f = _wave("pgse", n)
+    waves = [None, _wave("pgse", 10), _wave("cos", 11), _wave("pgse", 1), None]
+    gs = [(0.2, 0.1, 0.0), (0.0, 0.3, 0.1), (0.1, 0.1, 0.1), (0.3, 0.0, 0.0), (0.0, 0.0, 0.4)]
+    geo = [0, 1, 2, 0, 2]
+    res = []
+    for multi in (0, 1):
+        with _solver(lb, multi, geoms, (0, 0, 0), gs[0], f, 0.03, 0) as s:
+            fields = [torch.zeros(geoms[i].n_sites, dtype=torch.complex64, device="cuda") for i in geo]
+            r = s.run_batch(lb.Solver.members(gs, geo, [0.03, 0.0, INF, 0.1, 0.03]), waveforms=waves, fields=fields)
+            torch.cuda.synchronize()
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == (1 if multi else 3)
+            res.append(([v.cpu().numpy() for v in fields], r["Z"], np.array([float(v.abs().sum()) for v in fields])))
+    for a, b in zip(res[0][0], res[1][0]):
+        assert np.array_equal(a, b)
+    assert np.all(np.abs(res[0][1] - res[1][1]) <= 1e-13 * res[0][2])
+    g = geoms[0]
+    ref = None
+    for split in ([21], [1, 1, 19], [2, 17, 2], [20, 1]):   # one step by itself: the one-step sweep
+        with _solver(lb, 0, [g], (0, 0, 0), gs[0], f, 0.03, 0) as s:
+            fld = torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda")
+            s.set_field(fld)
+            s.prepare()
+            for k in split:
+                s.advance(k)
+            torch.cuda.synchronize()
+            v = fld.cpu().numpy()
+        ref = v if ref is None else ref
+        assert np.abs(ref).max() > 0 and np.array_equal(ref, v)
