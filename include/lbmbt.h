@@ -384,15 +384,14 @@ enum {
                                 LBMBT_EINVAL when it does not divide every
                                 member's nz                                  */
     LBMBT_OPT_MULTI_STEP = 18, /* runs with LBMBT_OPT_KERNEL = 0, the hybrid
-                                scheme, half-link membranes and no slabs: how
+                                scheme, no slabs and no membrane angles: how
                                 many steps a pass over the state makes.  0
                                 (default) auto: all of them in one launch
                                 (resident sweep) where the grids fit on chip,
-                                else two (two-step sweep, D3Q7) where the
-                                grids are large enough to gain, else one.  1
-                                one; 2 two where nx, ny, nz >= 4 on D3Q7; 3
-                                resident where the grids fit.  The fields are
-                                the same bits                                */
+                                else two (two-step sweep) where nx, ny, nz >= 4
+                                on D3Q7 with half-link membranes, else one.  1
+                                one; 2 two where it can run; 3 resident where
+                                the grids fit.  The fields are the same bits */
     LBMBT_OPT_MULTI_STEP_USED = 19 /* read-only: 1, 2 or 3 for the prepared
                                 run, else 0                                  */
 };

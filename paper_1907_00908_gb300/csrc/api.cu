@@ -117,6 +117,8 @@ struct lbmbt_ctx {
     ResBlock* d_res_blocks = nullptr;
     size_t cap_rb = 0;
     int res_sites = 0, res_recv = 0;          // the largest block's sites and received values
+    bool res_links = false;       // a member has membrane positions
+    int res_max_links = 0;
     size_t res_smem = 0;
     uint4* d_packets = nullptr;
     size_t cap_pk = 0;
@@ -904,17 +906,20 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
     if (c->kernel_opt != 0 || c->scheme != 0 || c->test_wait_ns > 0 || any_slab(c) || c->n_steps < 2) return LBMBT_OK;
     if (!c->sm_count) CU(c, cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
     long long total = 0;
+    bool links = false;
     for (auto& d : descs) {
-        if (d.dlt) return LBMBT_OK;
+        if (d.dth) return LBMBT_OK;   // the angle rule's stencil leaves the axis
+        links = links || d.dlt;
         total += d.N;
     }
+    const int width = links ? 3 : 1, least = links ? 2 : 1;   // values a face site, layers of a block
     if (total > (long long)c->sm_count * resident_max_sites() || (int)descs.size() > c->sm_count) return LBMBT_OK;
     int limit = 0;
     CU(c, cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
     limit -= 2048;   // the kernel's static arrays
     // fewest blocks of at most `cap` sites for one grid, then the fewest received values
     struct Cut { int cy, cz, recv; };
-    auto cut = [](const MemberDesc& d, int cap) {
+    auto cut = [&](const MemberDesc& d, int cap) {
         Cut best = {0, 0, 0};
         for (int cz = 1; cz <= d.nz; ++cz) {
             const int hz = (d.nz + cz - 1) / cz;
@@ -922,8 +927,9 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
             const long long rows = cap / ((long long)d.nx * hz);
             if (rows < 1) continue;
             const int cy = (int)((d.ny + std::min<long long>(rows, d.ny) - 1) / std::min<long long>(rows, d.ny));
+            if ((cz > 1 && d.nz / cz < least) || (cy > 1 && d.ny / cy < least)) continue;
             const int hy = (d.ny + cy - 1) / cy;
-            const int recv = 2 * d.nx * ((cy > 1 ? hz : 0) + (cz > 1 ? hy : 0));
+            const int recv = 2 * width * d.nx * ((cy > 1 ? hz : 0) + (cz > 1 ? hy : 0));
             const long long n = (long long)cy * cz, nb = (long long)best.cy * best.cz;
             if (!best.cy || n < nb || (n == nb && recv < best.recv)) best = {cy, cz, recv};
         }
@@ -967,7 +973,7 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
                 b.nbr[3] = face(z == cz - 1, d.bc[2], cz, at(y, z + 1));
                 for (int f = 0; f < 4; ++f) {
                     b.recv[f] = b.n_recv;
-                    if (b.nbr[f] >= 0) b.n_recv += d.nx * (f < 2 ? b.hz : b.hy);
+                    if (b.nbr[f] >= 0) b.n_recv += width * d.nx * (f < 2 ? b.hz : b.hy);
                 }
                 c->res_sites = std::max(c->res_sites, d.nx * b.hy * b.hz);
                 c->res_recv = std::max(c->res_recv, b.n_recv);
@@ -978,6 +984,7 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
         for (int f = 0; f < 4; ++f)
             if (b.nbr[f] >= 0) b.dest[f] = c->res_blocks[b.nbr[f]].recv[f ^ 1];
     c->res_smem = resident_smem(c->res_sites, c->res_recv, c->lattice == 1);
+    c->res_links = links;
     c->res_ok = true;
     return LBMBT_OK;
 }
@@ -1003,6 +1010,20 @@ static int build_resident(lbmbt_ctx* c)
     }
     CU(c, cudaMemcpyAsync(c->d_res_blocks, c->res_blocks.data(), sizeof(ResBlock) * nb, cudaMemcpyHostToDevice, c->stream));
     CU(c, cudaMemcpyAsync(c->d_res_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, c->stream));
+    c->res_max_links = 0;
+    if (c->res_links) {   // the lists lie in shared memory too
+        int n_links = 0;
+        CU(c, cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
+        CU(c, launch_resident_links(c->d_desc, c->d_res_blocks, nb, c->lattice == 1, c->d_err, c->stream));
+        c->launches++;
+        CU(c, cudaMemcpyAsync(&n_links, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        CU(c, cudaStreamSynchronize(c->stream));
+        c->res_max_links = (n_links + 1) / 2 * 2;
+        c->res_smem += resident_link_bytes() * c->res_max_links;
+        int limit = 0;
+        CU(c, cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+        if (c->res_smem + 2048 > (size_t)limit || n_links > 0xffff) return LBMBT_OK;   // one step a launch
+    }
     CU(c, cudaStreamSynchronize(c->stream));   // the host buffers are given back
     c->res_ok = true;
     return LBMBT_OK;
@@ -1628,6 +1649,8 @@ static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_ste
         r.field_step = field_step;
         r.series = c->series_mode ? 1 : 0;
         r.zpart = c->d_zpart;
+        r.links = c->res_links ? 1 : 0;
+        r.max_links = c->res_max_links;
         CU(c, launch_resident(a, r, nb, c->res_sites, c->res_smem, c->lattice == 1, c->general, c->stream));
         c->launches++;
         if (c->series_mode) {

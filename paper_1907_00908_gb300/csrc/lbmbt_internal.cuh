@@ -208,7 +208,8 @@ cudaError_t launch_pair_init(const MemberDesc* members, int n_members, long long
 // ---- resident sweep (sweep_resident.cu) -----------------------------------
 // One block of a small grid: all of x, rows [y0, y0 + hy), planes [z0, z0 + hz)
 // of member m; nbr: the blocks across its -y, +y, -z, +z faces, or what is there
-// instead; recv: where a face's values start among the n_recv it receives;
+// instead; recv: where a face's values start among the n_recv it receives (one
+// per site of the face; with membrane positions three);
 // dest: where they start among the neighbour's.
 constexpr int RES_SELF = -1, RES_MIRROR = -2;
 struct ResBlock {
@@ -222,11 +223,18 @@ struct ResArgs {
     int lsrc, ldst;               // time levels read and written
     unsigned stamp0;              // stamp of step k0's packets
     int sig_step, field_step;     // as in StepCtl; a member's own end step goes before them
+    int links;                    // 1: a member has membrane positions
+    int max_links;                // listed links of a block at most (rounded up to even)
     int series;                   // 1: zpart[n][block] = the block's part of Z after each step
     double2* zpart;
 };
 int resident_max_sites();         // sites of a block
 size_t resident_smem(int sites, int recv, bool d2);
+// Membrane positions: shared memory per listed link, and the most a block lists
+// (*out, zeroed before).
+size_t resident_link_bytes();
+cudaError_t launch_resident_links(const MemberDesc* members, const ResBlock* blocks, int n_blocks, bool d2, int* out,
+                                  cudaStream_t st);
 cudaError_t launch_resident(const SweepArgs& a, const ResArgs& r, int n_blocks, int max_sites, size_t smem, bool d2,
                             bool general, cudaStream_t st);
 // out[m][parts], to be summed; rows: the thread sums of the bulk-copy sweep

@@ -3,7 +3,7 @@
 // D2Q5 grids, at given angles (the general-angle rule of Appendix B):
 // second-neighbour reads with the outer-face transforms, the combinations,
 // and the arriving population of one listed link.  Used by the register
-// sweep only.
+// sweep; the resident sweep takes the coefficients and the sum.
 #pragma once
 #include "sweep_common.cuh"
 
@@ -46,8 +46,7 @@ __device__ __forceinline__ float2 read_along(const float2* __restrict__ src, uns
 // (Eq. c_d) coefficients of dl and 1 - dl and rho = kappa dt / (eps_D dx).
 // Used only when s + e_i lies in s's compartment and y - e_i in y's, and
 // kappa is finite.
-__device__ __forceinline__ float2 link_combine(float dl, float rho, float2 own_ib, float2 v_behind, float2 own_i,
-                                               float2 v1, float2 v_far, float2 w_y)
+__device__ __forceinline__ void link_coefficients(float dl, float rho, float (&A)[3], float (&B)[3])
 {
     float cn[4], cd[4], cns[4], cds[4];
     const float ds = 1.f - dl;
@@ -58,16 +57,28 @@ __device__ __forceinline__ float2 link_combine(float dl, float rho, float2 own_i
     cns[0] = 1.f; cns[1] = -us * qs; cns[2] = us * qs; cns[3] = 2.f * qs;
     cds[0] = 2.f * (ds - 1.f); cds[1] = -us * us * qs; cds[2] = 2.f * us * qs; cds[3] = (3.f - 2.f * ds) * qs;
     const float invF = __frcp_rn(cd[3] * cds[3] + (cd[3] * cns[3] + cn[3] * cds[3]) * rho);
-    float A[3], B[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
         A[j] = (cd[3] * cds[3] * cn[j] + (cds[3] * cn[3] * cd[j] + cns[3] * cd[3] * cn[j]) * rho) * invF;
         B[j] = cd[3] * cn[3] * (cns[j] - cds[j]) * rho * invF;
     }
+}
+
+__device__ __forceinline__ float2 link_sum(const float (&A)[3], const float (&B)[3], float2 own_ib, float2 v_behind,
+                                           float2 own_i, float2 v1, float2 v_far, float2 w_y)
+{
     float2 r;
     r.x = A[0] * own_ib.x + A[1] * v_behind.x + A[2] * own_i.x + B[0] * v1.x + B[1] * v_far.x + B[2] * w_y.x;
     r.y = A[0] * own_ib.y + A[1] * v_behind.y + A[2] * own_i.y + B[0] * v1.y + B[1] * v_far.y + B[2] * w_y.y;
     return r;
+}
+
+__device__ __forceinline__ float2 link_combine(float dl, float rho, float2 own_ib, float2 v_behind, float2 own_i,
+                                               float2 v1, float2 v_far, float2 w_y)
+{
+    float A[3], B[3];
+    link_coefficients(dl, rho, A, B);
+    return link_sum(A, B, own_ib, v_behind, own_i, v1, v_far, w_y);
 }
 
 // Arriving population i at site so (coordinates xo, yo, zo) across the

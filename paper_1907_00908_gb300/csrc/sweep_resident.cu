@@ -23,10 +23,18 @@
 // control, and the block goes on without waiting.
 //
 // Arithmetic and order per site are those of the register sweep (same bits).
+//
+// Membranes at given positions (theta = 0 rule): where each of a link's six
+// values lies and its six coefficients do not change over a run, so every launch
+// lists the block's links once in shared memory and a step gathers and sums,
+// one link a thread, before the sites take the results.  A face then carries
+// three values a column: both populations of its axis in the outer layer and
+// the outgoing one of the layer behind.
 #include <algorithm>
 
 #include "lbmbt_internal.cuh"
 #include "sweep_common.cuh"
+#include "links.cuh"
 #include "tma_common.cuh"
 
 namespace lbmbt {
@@ -65,12 +73,68 @@ __device__ __noinline__ uint4 await(const uint4* from, unsigned stamp, bool& dea
 }
 
 // Site flags: bits 0..5 at a face of the grid, 6..9 on a face of the block (-y, +y,
-// -z, +z), 10 a site at all, 16..21 the membrane links, 22..23 the phase.
-enum : unsigned { S_GRID = 63u, S_SEND = 0x3c0u, S_ON = 1024u };
+// -z, +z), 10 a site at all, 11..14 in the layer behind a face of the block, 16..21
+// the membrane links (of the half-link rule), 22..23 the phase.
+enum : unsigned { S_GRID = 63u, S_SEND = 0x3c0u, S_SEND2 = 0x7800u, S_ON = 1024u };
+
+// A listed link: elements of a level of own g_ib, g_ib behind, own g_i, g_i(y),
+// g_i behind y, g_ib(y); per value 4 bits, 1 + the boundary factor it takes and
+// 8 if conjugated first; the coefficients.
+struct LinkEntry {
+    uint16_t at[6];
+    uint32_t face;
+    float A[3], B[3];
+};
+static_assert(sizeof(LinkEntry) == 40, "link entry");
+
+// cmul() with its roundings written out: as the register sweep's reads beyond a
+// face come out of the compiler, so that the fields are the same bits.
+__device__ __forceinline__ float2 turn(float2 a, float2 b)
+{
+    return make_float2(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)), __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+
+// Directions (bits 1..6) in which site s takes the position rule: a membrane
+// behind it, none ahead, none behind the far node.
+__device__ __forceinline__ unsigned rule_links(const MemberDesc* __restrict__ d, unsigned mk, int x, int y, int z, int np)
+{
+    unsigned rule = 0;
+    const int c[3] = {x, y, z}, n[3] = {d->nx, d->ny, d->nz};
+    for (int i = 1; i <= np; ++i) {
+        const int ib = (i & 1) ? i + 1 : i - 1, a = (i - 1) >> 1;
+        if (!(mk & (1u << (ib - 1))) || (mk & (1u << (i - 1)))) continue;
+        int v[3] = {c[0], c[1], c[2]};
+        v[a] = (v[a] + ((i & 1) ? n[a] - 1 : 1)) % n[a];   // a membrane never crosses a mirror face
+        const unsigned mky = d->mask[((unsigned)v[2] * d->ny + v[1]) * d->nx + v[0]];
+        if (!(mky & (1u << (ib - 1)))) rule |= 1u << i;
+    }
+    return rule;
+}
+
+// Largest number of listed links of a block.
+__global__ void resident_links_kernel(const MemberDesc* __restrict__ members, const ResBlock* __restrict__ blocks, int np,
+                                      int* out)
+{
+    __shared__ int n;
+    if (threadIdx.x == 0) n = 0;
+    __syncthreads();
+    const ResBlock b = blocks[blockIdx.x];
+    const MemberDesc* __restrict__ d = members + b.m;
+    const int nx = d->nx, S = nx * b.hy * b.hz;
+    if (d->dlt)
+        for (int l = threadIdx.x; l < S; l += blockDim.x) {
+            const int z = l / (nx * b.hy), row = l / nx - z * b.hy, x = l % nx, gy = b.y0 + row, gz = b.z0 + z;
+            const unsigned rule = rule_links(d, d->mask[((unsigned)gz * d->ny + gy) * nx + x], x, gy, gz, np);
+            if (rule) atomicAdd(&n, __popc(rule));
+        }
+    __syncthreads();
+    if (threadIdx.x == 0) atomicMax(out, n);
+}
 
 // SPT sites a thread; D2: the D2Q5 lattice (no z populations, weights of a);
-// GEN: the waveform may take values other than 0 and +-1.
-template <int SPT, bool D2, bool GEN>
+// GEN: the waveform may take values other than 0 and +-1; LK: a member has
+// membrane positions.
+template <int SPT, bool D2, bool GEN, bool LK>
 __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepArgs a, const ResArgs r)
 {
     extern __shared__ __align__(16) unsigned char res_smem[];
@@ -89,6 +153,13 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
     const int lsz = NP * S + b.n_recv;
     float2* const lev = reinterpret_cast<float2*>(res_smem);
     float2* const rots = lev + 2 * lsz;
+    float2* const lres = rots + S;                                       // results of the listed links
+    LinkEntry* const lent = reinterpret_cast<LinkEntry*>(lres + r.max_links);
+    __shared__ int s_links;
+    if (LK) {
+        if (threadIdx.x == 0) s_links = 0;
+        __syncthreads();
+    }
     const unsigned P = (unsigned)d->plane, sxy = (unsigned)nx * ny;
     const float2* __restrict__ src = d->state + (size_t)r.lsrc * 7 * P;
     const int bc[3] = {d->bc[0], d->bc[1], d->bc[2]};
@@ -103,12 +174,13 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
     // half) and in a y face, and where the y and z pulls come from (element of a
     // level, 16 bits each: -y, +y and -z, +z)
     unsigned gs[SPT], fl[SPT], pl[SPT], oy[SPT], oz[SPT];
+    unsigned lk[SPT];   // LK: first result of the site's listed links, their directions << 16
     float2 p0[SPT];
     float thg[SPT];
 #pragma unroll
     for (int j = 0; j < SPT; ++j) {
         const int l = t + j * RES_NT;
-        gs[j] = fl[j] = pl[j] = oy[j] = oz[j] = 0u;
+        gs[j] = fl[j] = pl[j] = oy[j] = oz[j] = lk[j] = 0u;
         p0[j] = make_float2(0.f, 0.f);
         thg[j] = 0.f;
         if (l < S) {
@@ -136,6 +208,59 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
             if (!D2)
                 oz[j] = from(zl, b.nbr[2], -layer, wz, 5, 6, b.recv[2] + in) |
                         (from(zh, b.nbr[3], layer, -wz, 6, 5, b.recv[3] + in) << 16);
+            if (LK) {
+                fl[j] |= (row == 1 && b.nbr[0] >= 0 ? 0x800u : 0u) | (row == b.hy - 2 && b.nbr[1] >= 0 ? 0x1000u : 0u) |
+                         (z == 1 && b.nbr[2] >= 0 ? 0x2000u : 0u) | (z == b.hz - 2 && b.nbr[3] >= 0 ? 0x4000u : 0u);
+                const unsigned rule = d->dlt ? rule_links(d, mk, x, gy, gz, NP) : 0u;
+                if (rule) {
+                    int e = atomicAdd(&s_links, __popc(rule));
+                    lk[j] = (unsigned)e | rule << 16;
+                    for (int i = 1; i <= NP; ++i) {
+                        if (!(rule & (1u << i))) continue;
+                        const int ib = (i & 1) ? i + 1 : i - 1, a3 = (i - 1) >> 1, dir = (i & 1) ? 1 : -1;
+                        fl[j] &= ~(1u << (16 + ib - 1));   // not the half-link rule
+                        LinkEntry L;
+                        L.face = 0;
+                        // element of population p at the node dd along axis a3, and its face
+                        auto along = [&](int j6, int p, int dd) {
+                            const int c = a3 == 0 ? x : a3 == 1 ? row : z, ext = a3 == 0 ? nx : a3 == 1 ? b.hy : b.hz;
+                            const int stride = a3 == 0 ? 1 : a3 == 1 ? nx : layer, cp = c + dd;
+                            int at = (p - 1) * S + l + dd * stride;
+                            if (cp < 0 || cp >= ext) {
+                                const bool lo = cp < 0;
+                                const int side = lo ? 0 : 1;
+                                const int nb = a3 == 0 ? (bc[0] == BC_PER ? RES_SELF : RES_MIRROR) : b.nbr[2 * (a3 - 1) + side];
+                                const bool grid = a3 == 0 || (a3 == 1 ? (lo ? b.y0 == 0 : b.y0 + b.hy == ny)
+                                                                      : (lo ? b.z0 == 0 : b.z0 + b.hz == nz));
+                                const unsigned fc = 1u + 2 * a3 + side;
+                                if (nb == RES_MIRROR) {
+                                    const int m = lo ? -1 - cp : 2 * ext - 1 - cp, po = (p & 1) ? p + 1 : p - 1;
+                                    at = (po - 1) * S + l + (m - c) * stride;
+                                    if (bc[a3] != BC_MIR) L.face |= (8u | fc) << (4 * j6);
+                                } else {
+                                    if (grid) L.face |= fc << (4 * j6);
+                                    if (nb == RES_SELF) {
+                                        at += (lo ? ext : -ext) * stride;
+                                    } else {
+                                        const int far = lo ? -cp : cp - ext + 1;   // 1 or 2 layers beyond
+                                        const int q = far == 2 ? 2 : p == 2 * a3 + 1 + side ? 0 : 1;
+                                        at = NP * S + b.recv[2 * (a3 - 1) + side] + (a3 == 1 ? q * nx * b.hz + ez : q * layer + in);
+                                    }
+                                }
+                            }
+                            L.at[j6] = (uint16_t)at;
+                        };
+                        along(0, ib, 0);
+                        along(1, ib, dir);
+                        along(2, i, 0);
+                        along(3, i, -dir);
+                        along(4, i, -2 * dir);
+                        along(5, ib, -dir);
+                        link_coefficients(d->dlt[(size_t)(ib - 1) * P + s], d->lrho, L.A, L.B);
+                        lent[e++] = L;
+                    }
+                }
+            }
             rots[l] = rotation_m1(d, 1.f, x, gy, gz);
             if (GEN) thg[j] = __fmaf_rn(d->ctheta[2], (float)(gz + d->z0),
                                         __fmaf_rn(d->ctheta[1], (float)gy, __fmul_rn(d->ctheta[0], (float)x)));
@@ -161,10 +286,22 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
         if (f & 128u) send(to(1, ez), v3, stamp);
         if (f & 256u) send(to(2, in), v6, stamp);
         if (f & 512u) send(to(3, in), v5, stamp);
+        if (LK) {
+            const int ly = nx * b.hz;
+            if (f & 64u) send(to(0, ly + ez), v3, stamp);
+            if (f & 128u) send(to(1, ly + ez), v4, stamp);
+            if (f & 0x800u) send(to(0, 2 * ly + ez), v4, stamp);
+            if (f & 0x1000u) send(to(1, 2 * ly + ez), v3, stamp);
+            if (f & 256u) send(to(2, layer + in), v5, stamp);
+            if (f & 512u) send(to(3, layer + in), v6, stamp);
+            if (f & 0x2000u) send(to(2, 2 * layer + in), v6, stamp);
+            if (f & 0x4000u) send(to(3, 2 * layer + in), v5, stamp);
+        }
     };
+    constexpr unsigned SEND = S_SEND | (LK ? S_SEND2 : 0u);
 #pragma unroll
     for (int j = 0; j < SPT; ++j)
-        if (fl[j] & S_SEND) {   // the values that the first step pulls
+        if (fl[j] & SEND) {   // the values that the first step pulls
             const float2* v = lev + t + j * RES_NT;
             send_faces(fl[j], pl[j], 0, v[2 * S], v[3 * S], D2 ? v[0] : v[4 * S], D2 ? v[0] : v[5 * S]);
         }
@@ -197,6 +334,23 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
         __syncthreads();   // the level, its face values and the factors are complete
         const float2* fac = s_fac[n & 1];
         const float f = s_f[n & 1];
+        if (LK) {   // the listed links, one a thread
+            for (int e = t; e < s_links; e += RES_NT) {
+                const LinkEntry L = lent[e];
+                float2 v[6];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) v[q] = cur[L.at[q]];
+                if (L.face)
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) {
+                        const unsigned c = L.face >> (4 * q) & 15u;
+                        if (c & 8u) v[q].y = -v[q].y;
+                        if (c) v[q] = turn(v[q], fac[(c & 7u) - 1u]);
+                    }
+                lres[e] = link_sum(L.A, L.B, v[0], v[1], v[2], v[3], v[4], v[5]);
+            }
+            __syncthreads();
+        }
         const bool do_sig = k == sig, do_fld = field != nullptr && k == fstep;
         double zr = 0.0, zi = 0.0;
 #pragma unroll
@@ -238,6 +392,12 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
                     if (F & 0x100000u) g[6] = mix(c[4 * S], g[6], sh);
                 }
             }
+            if (LK && lk[j]) {
+                const float2* res = lres + (lk[j] & 0xffffu);
+#pragma unroll
+                for (int i = 1; i <= NP; ++i)
+                    if (lk[j] & (0x10000u << i)) g[i] = *res++;
+            }
             float2 q;
             if (GEN && f != 0.f && f != 1.f && f != -1.f) {   // rotation_m1's general form
                 float sn, cs;
@@ -253,7 +413,7 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
             collide_w(g, pe.x, mr, mi, a.w0, a.wxy, a.wz);
             p0[j] = g[0];
             // the faces first: a neighbour waits for them (nobody after the last step)
-            if ((F & S_SEND) && n + 1 < r.n_steps) send_faces(F, pl[j], n + 1, g[3], g[4], g[5], g[6]);
+            if ((F & SEND) && n + 1 < r.n_steps) send_faces(F, pl[j], n + 1, g[3], g[4], g[5], g[6]);
 #pragma unroll
             for (int i = 1; i <= NP; ++i) nxt[(i - 1) * S + l] = g[i];
             if (do_sig) mout[gs[j]] = make_float2(mr, mi);
@@ -368,28 +528,37 @@ __global__ void resident_series_kernel(const double2* __restrict__ zpart, const 
 
 using ResFn = void (*)(const SweepArgs, const ResArgs);
 
-template <bool D2, bool GEN>
+template <bool D2, bool GEN, bool LK>
 ResFn res_spt(int spt)
 {
-    return spt <= 1 ? sweep_resident_kernel<1, D2, GEN>
-           : spt <= 2 ? sweep_resident_kernel<2, D2, GEN> : sweep_resident_kernel<4, D2, GEN>;
+    return spt <= 1 ? sweep_resident_kernel<1, D2, GEN, LK>
+           : spt <= 2 ? sweep_resident_kernel<2, D2, GEN, LK> : sweep_resident_kernel<4, D2, GEN, LK>;
 }
-ResFn res_kernel(int spt, bool d2, bool gen)
+template <bool D2>
+ResFn res_kernel(int spt, bool gen, bool links)
 {
-    if (d2) return gen ? res_spt<true, true>(spt) : res_spt<true, false>(spt);
-    return gen ? res_spt<false, true>(spt) : res_spt<false, false>(spt);
+    if (links) return res_spt<D2, true, true>(spt);   // the general waveform form covers the others
+    return gen ? res_spt<D2, true, false>(spt) : res_spt<D2, false, false>(spt);
 }
 
 }  // namespace
 
 int resident_max_sites() { return RES_MAX_SITES; }
+size_t resident_link_bytes() { return sizeof(LinkEntry) + sizeof(float2); }
+cudaError_t launch_resident_links(const MemberDesc* members, const ResBlock* blocks, int n_blocks, bool d2, int* out,
+                                  cudaStream_t st)
+{
+    resident_links_kernel<<<n_blocks, 256, 0, st>>>(members, blocks, d2 ? 4 : 6, out);
+    return cudaGetLastError();
+}
 
 size_t resident_smem(int sites, int recv, bool d2) { return ((size_t)(d2 ? 9 : 13) * sites + 2 * recv) * sizeof(float2); }
 
 cudaError_t launch_resident(const SweepArgs& a, const ResArgs& r, int n_blocks, int max_sites, size_t smem, bool d2,
                             bool general, cudaStream_t st)
 {
-    const void* fn = (const void*)res_kernel((max_sites + RES_NT - 1) / RES_NT, d2, general);
+    const int spt = (max_sites + RES_NT - 1) / RES_NT;
+    const void* fn = (const void*)(d2 ? res_kernel<true>(spt, general, r.links) : res_kernel<false>(spt, general, r.links));
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     SweepArgs aa = a;

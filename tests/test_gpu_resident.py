@@ -116,3 +116,32 @@ def test_resident_batch_with_own_echoes_and_any_split(lb):
             v = fld.cpu().numpy()
         ref = v if ref is None else ref
         assert np.abs(ref).max() > 0 and np.array_equal(ref, v)
+
+
+# blocks of two and more layers, the rule's second neighbours across every kind
+# of face; random positions (any link, any compartment)
+@pytest.mark.parametrize("shape,bc,gG,wave,n,lattice", [
+    ((12, 10, 9), (0, 0, 0), (0.3, 0.2, 0.1), "pgse", 9, 0),
+    ((24, 31, 20), (1, 0, 1), (0.3, 0.0, 0.0), "cos", 8, 0),
+    ((2, 3, 5), (0, 0, 0), (0.2, 0.1, 0.3), "pgse", 6, 0),
+    ((1, 200, 200), (0, 0, 0), (0.3, 0.2, 0.0), "pgse", 30, 1),
+    ((1, 65, 130), (1, 1, 0), (0.0, 0.2, 0.0), "cos", 21, 1),
+    ((1, 37, 22), (0, 1, 0), (0.1, 0.0, 0.0), "pgse", 14, 1),
+])
+def test_resident_sweep_with_membrane_positions(lb, shape, bc, gG, wave, n, lattice):
+    """Against the register sweep's position rule: the same bits."""
+    g = _geom(shape, sum(shape) + 1)
+    f = _wave(wave, n)
+    delta = np.random.default_rng(3).uniform(0.1, 0.9, size=(6, *shape)).astype(np.float32)
+    out = []
+    for multi in (0, 1):
+        with _solver(lb, multi, [g], bc, gG, f, 0.05, lattice) as s:
+            s.set_link_distances(delta)
+            fld = torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda")
+            r = s.run(field=fld, series=True)
+            torch.cuda.synchronize()
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == (1 if multi else 3)
+            assert s.get_option(lb.OPT_KERNEL_USED) == 1
+            out.append((fld.cpu().numpy(), r))
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.abs(out[0][1]["series"] - out[1][1]["series"]).max() <= 2.0 ** -22 * g.n_sites
