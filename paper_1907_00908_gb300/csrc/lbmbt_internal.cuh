@@ -237,6 +237,12 @@ cudaError_t launch_resident_links(const MemberDesc* members, const ResBlock* blo
                                   cudaStream_t st);
 cudaError_t launch_resident(const SweepArgs& a, const ResArgs& r, int n_blocks, int max_sites, size_t smem, bool d2,
                             bool general, cudaStream_t st);
+// 2-D grids (D2Q5) in strips of whole rows (sweep_strip.cu): rows of a block at
+// most for this nx (0: too wide), its shared memory.
+int strip_rows(int nx);
+size_t strip_smem(int nx, int rows);
+cudaError_t launch_strip(const SweepArgs& a, const ResArgs& r, int n_blocks, int max_nx, size_t smem, bool general,
+                         cudaStream_t st);
 // out[m][parts], to be summed; rows: the thread sums of the bulk-copy sweep
 cudaError_t launch_signal(const MemberDesc* members, int n_members, bool rows, int block, int spt, int parts, double2* out,
                           cudaStream_t st);

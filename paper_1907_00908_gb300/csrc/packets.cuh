@@ -1,0 +1,56 @@
+// packets.cuh -- face values sent between the blocks of one cooperative launch:
+// 16-byte packets {re, stamp, im, stamp} that the receiver polls (see
+// sweep_resident.cu for why no packet is lost or taken twice).
+#pragma once
+#include "lbmbt_internal.cuh"
+#include "tma_common.cuh"
+
+namespace lbmbt {
+namespace {
+
+__device__ __forceinline__ void send(uint4* to, float2 v, unsigned stamp)
+{
+    asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(to), "r"(__float_as_uint(v.x)), "r"(stamp),
+                 "r"(__float_as_uint(v.y)), "r"(stamp)
+                 : "memory");
+}
+
+__device__ __forceinline__ uint4 peek(const uint4* from)
+{
+    uint4 p;
+    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(p.x), "=r"(p.y), "=r"(p.z), "=r"(p.w)
+                 : "l"(from)
+                 : "memory");
+    return p;
+}
+
+// Polls a packet until both halves carry the stamp; `dead` once the limit has passed.
+__device__ __noinline__ uint4 await(const uint4* from, unsigned stamp, bool& dead)
+{
+    uint4 p = peek(from);
+    const unsigned long long t0 = globaltimer();
+    for (unsigned n = 1; !dead && !(p.y == stamp && p.w == stamp); ++n) {
+        if ((n & 63u) == 0 && globaltimer() - t0 > WAIT_NS) dead = true;
+        p = peek(from);
+    }
+    return p;
+}
+
+// Site flags: bits 0..5 at a face of the grid, 6..9 on a face of the block (-y, +y,
+// -z, +z), 10 a site at all, 11..14 in the layer behind a face of the block, 16..21
+// the membrane links (of the half-link rule), 22..23 the phase.
+enum : unsigned { S_GRID = 63u, S_SEND = 0x3c0u, S_SEND2 = 0x7800u, S_ON = 1024u };
+
+// A listed link: elements of a level of own g_ib, g_ib behind, own g_i, g_i(y),
+// g_i behind y, g_ib(y); per value 4 bits, 1 + the boundary factor it takes and
+// 8 if conjugated first; the coefficients.
+struct LinkEntry {
+    uint16_t at[6];
+    uint32_t face;
+    float A[3], B[3];
+};
+static_assert(sizeof(LinkEntry) == 40, "link entry");
+
+}  // namespace
+}  // namespace lbmbt

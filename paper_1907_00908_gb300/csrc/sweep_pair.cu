@@ -46,6 +46,7 @@
 
 #include "lbmbt_internal.cuh"
 #include "sweep_common.cuh"
+#include "packed.cuh"
 #include "tma_common.cuh"
 
 namespace lbmbt {
@@ -57,40 +58,6 @@ constexpr int PAIR_GHOST = 2;    // ghost columns and rows on each side
 // A stage in 16-byte words: boxes of (rows of the grown tile) x ex pairs of
 // p0 p1 p2 p5 p6, then of one row more of p3 (from one row below) and p4.
 __host__ __device__ constexpr int stage_words(int nt) { return 7 * nt + 2 * PAIR_MAX_EX; }
-using u64 = unsigned long long;   // one complex value (re, im) as a packed pair
-
-__device__ __forceinline__ u64 pk(float x, float y)
-{
-    u64 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float2 unpk(u64 v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c)
-{
-    u64 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ u64 add2(u64 a, u64 b)
-{
-    u64 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
-__device__ __forceinline__ u64 sub2(u64 a, u64 b)
-{
-    u64 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 __device__ __forceinline__ void tma_box(void* dst, const CUtensorMap* map, int x, int y, int z, int p, uint64_t* bar)
 {
     asm volatile(
@@ -98,52 +65,6 @@ __device__ __forceinline__ void tma_box(void* dst, const CUtensorMap* map, int x
             smem_u32(dst)),
         "l"(map), "r"(x), "r"(y), "r"(z), "r"(p), "r"(smem_u32(bar))
         : "memory");
-}
-
-// Transform of a value pulled across a face (see pull()).
-__device__ __forceinline__ u64 face2(u64 p, int bc, float2 f)
-{
-    if (bc == BC_MIR) return p;
-    float2 v = unpk(p);
-    if (bc == BC_MIR_CONJ) v.y = -v.y;
-    v = cmul(v, f);
-    return pk(v.x, v.y);
-}
-
-// Membrane link: v <- o + s (v - o) (mix() of sweep_common.cuh) where bit `B` of
-// mk is set, by predication: in tissue nearly every warp has some such lane in
-// every direction, and a divergent branch per direction and column costs more.
-template <unsigned B>
-__device__ __forceinline__ void mix_if(unsigned mk, u64& v, u64 o, u64 s2)
-{
-    asm("{\n\t.reg .pred p;\n\t.reg .b32 b;\n\t.reg .b64 d;\n\t"
-        "and.b32 b, %1, %4;\n\tsetp.ne.u32 p, b, 0;\n\t"
-        "sub.rn.f32x2 d, %0, %2;\n\t"
-        "@p fma.rn.f32x2 %0, %3, d, %2;\n\t}"
-        : "+l"(v)
-        : "r"(mk), "l"(o), "l"(s2), "n"(B));
-}
-
-// react() and collide(): g <- g + g q, M = sum g, g <- g + omega (w M - g),
-// the last as g - omega (g - w M): the same rounding, w M being exact (w is a
-// power of two).  Returns M.
-__device__ __forceinline__ u64 react_collide(u64 (&g)[Q], float2 q, float om)
-{
-    const u64 qx = pk(q.x, q.x), qy = pk(-q.y, q.y);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const float2 v = unpk(g[i]);
-        g[i] = fma2(g[i], qx, fma2(pk(v.y, v.x), qy, g[i]));
-    }
-    u64 m = g[0];
-#pragma unroll
-    for (int i = 1; i < Q; ++i) m = add2(m, g[i]);
-    const u64 no = pk(-om, -om);
-    const float2 mv = unpk(m);
-    const u64 m0 = pk(W0 * mv.x, W0 * mv.y), mi = pk(WI * mv.x, WI * mv.y);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) g[i] = fma2(no, sub2(g[i], i == 0 ? m0 : mi), g[i]);
-    return m;
 }
 
 // Exact running sum (two-sum) of one component.
@@ -487,8 +408,8 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
                 rotb = signed_rot(nrb, f1);
             }
             const float2 pa = s_phase[(mk >> 6) & 3u], pb = s_phase[mk >> 14];
-            const u64 ma = react_collide(ga, reaction_q(rota, pa.y), pa.x);
-            const u64 mb = react_collide(gb, reaction_q(rotb, pb.y), pb.x);
+            const u64 ma = react_collide<Q>(ga, reaction_q(rota, pa.y), pa.x);
+            const u64 mb = react_collide<Q>(gb, reaction_q(rotb, pb.y), pb.x);
             if ((obs & 21u) && zi >= it.z0 && zi < it.z1) observe(ssum + t, obs, fl, ma, mb, z);
             if (STEPS == 1) {
                 store(z, ga, gb);
@@ -561,8 +482,8 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
                     rotb = signed_rot(qrb, f2);
                 }
                 const float2 pa = s_phase[(mkp >> 6) & 3u], pb = s_phase[mkp >> 14];
-                const u64 ma = react_collide(ga, reaction_q(rota, pa.y), pa.x);
-                const u64 mb = react_collide(gb, reaction_q(rotb, pb.y), pb.x);
+                const u64 ma = react_collide<Q>(ga, reaction_q(rota, pa.y), pa.x);
+                const u64 mb = react_collide<Q>(gb, reaction_q(rotb, pb.y), pb.x);
                 store(z, ga, gb);
                 if (obs & 42u) observe(ssum + NT + t, obs >> 1, fl, ma, mb, z);
             }

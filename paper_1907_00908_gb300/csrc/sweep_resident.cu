@@ -35,57 +35,14 @@
 #include "lbmbt_internal.cuh"
 #include "sweep_common.cuh"
 #include "links.cuh"
-#include "tma_common.cuh"
+#include "packed.cuh"
+#include "packets.cuh"
 
 namespace lbmbt {
 namespace {
 
 constexpr int RES_NT = 512;           // threads of a block
 constexpr int RES_MAX_SITES = 2048;   // sites of a block: 13 x 8 B each in shared memory
-
-__device__ __forceinline__ void send(uint4* to, float2 v, unsigned stamp)
-{
-    asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(to), "r"(__float_as_uint(v.x)), "r"(stamp),
-                 "r"(__float_as_uint(v.y)), "r"(stamp)
-                 : "memory");
-}
-
-__device__ __forceinline__ uint4 peek(const uint4* from)
-{
-    uint4 p;
-    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(p.x), "=r"(p.y), "=r"(p.z), "=r"(p.w)
-                 : "l"(from)
-                 : "memory");
-    return p;
-}
-
-// Polls a packet until both halves carry the stamp; `dead` once the limit has passed.
-__device__ __noinline__ uint4 await(const uint4* from, unsigned stamp, bool& dead)
-{
-    uint4 p = peek(from);
-    const unsigned long long t0 = globaltimer();
-    for (unsigned n = 1; !dead && !(p.y == stamp && p.w == stamp); ++n) {
-        if ((n & 63u) == 0 && globaltimer() - t0 > WAIT_NS) dead = true;
-        p = peek(from);
-    }
-    return p;
-}
-
-// Site flags: bits 0..5 at a face of the grid, 6..9 on a face of the block (-y, +y,
-// -z, +z), 10 a site at all, 11..14 in the layer behind a face of the block, 16..21
-// the membrane links (of the half-link rule), 22..23 the phase.
-enum : unsigned { S_GRID = 63u, S_SEND = 0x3c0u, S_SEND2 = 0x7800u, S_ON = 1024u };
-
-// A listed link: elements of a level of own g_ib, g_ib behind, own g_i, g_i(y),
-// g_i behind y, g_ib(y); per value 4 bits, 1 + the boundary factor it takes and
-// 8 if conjugated first; the coefficients.
-struct LinkEntry {
-    uint16_t at[6];
-    uint32_t face;
-    float A[3], B[3];
-};
-static_assert(sizeof(LinkEntry) == 40, "link entry");
 
 // cmul() with its roundings written out: as the register sweep's reads beyond a
 // face come out of the compiler, so that the fields are the same bits.
@@ -163,7 +120,7 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
     const unsigned P = (unsigned)d->plane, sxy = (unsigned)nx * ny;
     const float2* __restrict__ src = d->state + (size_t)r.lsrc * 7 * P;
     const int bc[3] = {d->bc[0], d->bc[1], d->bc[2]};
-    const float sh = d->s_share;
+    const u64 sh2 = pk(d->s_share, d->s_share);
     const int es = d->end_step;
     const int sig = es >= 0 ? es : r.sig_step, fstep = es >= 0 ? es : r.field_step;
     float2* const field = d->field;
@@ -175,13 +132,13 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
     // level, 16 bits each: -y, +y and -z, +z)
     unsigned gs[SPT], fl[SPT], pl[SPT], oy[SPT], oz[SPT];
     unsigned lk[SPT];   // LK: first result of the site's listed links, their directions << 16
-    float2 p0[SPT];
+    u64 p0[SPT];
     float thg[SPT];
 #pragma unroll
     for (int j = 0; j < SPT; ++j) {
         const int l = t + j * RES_NT;
         gs[j] = fl[j] = pl[j] = oy[j] = oz[j] = lk[j] = 0u;
-        p0[j] = make_float2(0.f, 0.f);
+        p0[j] = 0ull;
         thg[j] = 0.f;
         if (l < S) {
             const int z = l / layer, in = l - z * layer, row = in / nx, x = in - row * nx;
@@ -264,7 +221,7 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
             rots[l] = rotation_m1(d, 1.f, x, gy, gz);
             if (GEN) thg[j] = __fmaf_rn(d->ctheta[2], (float)(gz + d->z0),
                                         __fmaf_rn(d->ctheta[1], (float)gy, __fmul_rn(d->ctheta[0], (float)x)));
-            p0[j] = __ldcg(src + s);
+            p0[j] = __ldcg(reinterpret_cast<const u64*>(src) + s);
 #pragma unroll
             for (int i = 1; i <= NP; ++i) lev[(i - 1) * S + l] = __ldcg(src + (size_t)i * P + s);
         }
@@ -358,42 +315,41 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
             const int l = t + j * RES_NT;
             const unsigned F = fl[j];
             if (!(F & S_ON)) continue;
-            const float2* c = cur + l;
-            float2 g[Q];
+            const u64* const cur2 = reinterpret_cast<const u64*>(cur);
+            const u64* c = cur2 + l;
+            u64 g[NP + 1];
             g[0] = p0[j];
             // x: the block spans the axis
             g[1] = (F & 1u) ? (bc[0] == BC_PER ? c[nx - 1] : c[S]) : c[-1];
             g[2] = (F & 2u) ? (bc[0] == BC_PER ? c[S - (nx - 1)] : c[0]) : c[S + 1];
-            g[3] = cur[oy[j] & 0xffffu];
-            g[4] = cur[oy[j] >> 16];
+            g[3] = cur2[oy[j] & 0xffffu];
+            g[4] = cur2[oy[j] >> 16];
             if (!D2) {
-                g[5] = cur[oz[j] & 0xffffu];
-                g[6] = cur[oz[j] >> 16];
-            } else {
-                g[5] = g[6] = make_float2(0.f, 0.f);
+                g[NP - 1] = cur2[oz[j] & 0xffffu];
+                g[NP] = cur2[oz[j] >> 16];
             }
             if (F & S_GRID) {
-                if (F & 1u) g[1] = face_fix(g[1], bc[0], fac[0]);
-                if (F & 2u) g[2] = face_fix(g[2], bc[0], fac[1]);
-                if (F & 4u) g[3] = face_fix(g[3], bc[1], fac[2]);
-                if (F & 8u) g[4] = face_fix(g[4], bc[1], fac[3]);
+                if (F & 1u) g[1] = face2(g[1], bc[0], fac[0]);
+                if (F & 2u) g[2] = face2(g[2], bc[0], fac[1]);
+                if (F & 4u) g[3] = face2(g[3], bc[1], fac[2]);
+                if (F & 8u) g[4] = face2(g[4], bc[1], fac[3]);
                 if (!D2) {
-                    if (F & 16u) g[5] = face_fix(g[5], bc[2], fac[4]);
-                    if (F & 32u) g[6] = face_fix(g[6], bc[2], fac[5]);
+                    if (F & 16u) g[NP - 1] = face2(g[NP - 1], bc[2], fac[4]);
+                    if (F & 32u) g[NP] = face2(g[NP], bc[2], fac[5]);
                 }
             }
             if (F & 0x3f0000u) {   // half-link membranes (Eq. B5)
-                if (F & 0x20000u) g[1] = mix(c[S], g[1], sh);
-                if (F & 0x10000u) g[2] = mix(c[0], g[2], sh);
-                if (F & 0x80000u) g[3] = mix(c[3 * S], g[3], sh);
-                if (F & 0x40000u) g[4] = mix(c[2 * S], g[4], sh);
+                mix_if<0x20000u>(F, g[1], c[S], sh2);
+                mix_if<0x10000u>(F, g[2], c[0], sh2);
+                mix_if<0x80000u>(F, g[3], c[3 * S], sh2);
+                mix_if<0x40000u>(F, g[4], c[2 * S], sh2);
                 if (!D2) {
-                    if (F & 0x200000u) g[5] = mix(c[5 * S], g[5], sh);
-                    if (F & 0x100000u) g[6] = mix(c[4 * S], g[6], sh);
+                    mix_if<0x200000u>(F, g[NP - 1], c[5 * S], sh2);
+                    mix_if<0x100000u>(F, g[NP], c[4 * S], sh2);
                 }
             }
             if (LK && lk[j]) {
-                const float2* res = lres + (lk[j] & 0xffffu);
+                const u64* res = reinterpret_cast<const u64*>(lres) + (lk[j] & 0xffffu);
 #pragma unroll
                 for (int i = 1; i <= NP; ++i)
                     if (lk[j] & (0x10000u << i)) g[i] = *res++;
@@ -408,19 +364,19 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
                 q = make_float2(__fmul_rn(v.x, fabsf(f)), __fmul_rn(v.y, f));
             }
             const float2 pe = s_phase[F >> 22 & 3u];
-            float mr, mi;
-            react(g, reaction_q(q, pe.y), mr, mi);
-            collide_w(g, pe.x, mr, mi, a.w0, a.wxy, a.wz);
+            const u64 M = react_collide(g, reaction_q(q, pe.y), pe.x, a.w0, a.wxy);
             p0[j] = g[0];
             // the faces first: a neighbour waits for them (nobody after the last step)
-            if ((F & SEND) && n + 1 < r.n_steps) send_faces(F, pl[j], n + 1, g[3], g[4], g[5], g[6]);
+            if ((F & SEND) && n + 1 < r.n_steps) 
+                send_faces(F, pl[j], n + 1, unpk(g[3]), unpk(g[4]), unpk(g[NP - 1]), unpk(g[NP]));
 #pragma unroll
-            for (int i = 1; i <= NP; ++i) nxt[(i - 1) * S + l] = g[i];
-            if (do_sig) mout[gs[j]] = make_float2(mr, mi);
-            if (do_fld) field[gs[j]] = make_float2(mr, mi);
-            if (r.series) {
-                zr += mr;
-                zi += mi;
+            for (int i = 1; i <= NP; ++i) reinterpret_cast<u64*>(nxt)[(i - 1) * S + l] = g[i];
+            if (do_sig || do_fld || r.series) {
+                const float2 v = unpk(M);
+                if (do_sig) mout[gs[j]] = v;
+                if (do_fld) field[gs[j]] = v;
+                zr += v.x;
+                zi += v.y;
             }
         }
         if (t < 6) s_fac[(n & 1) ^ 1][t] = fnext;
@@ -450,7 +406,7 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
     for (int j = 0; j < SPT; ++j) {
         const int l = t + j * RES_NT;
         if (!(fl[j] & S_ON)) continue;
-        dst[gs[j]] = p0[j];
+        dst[gs[j]] = unpk(p0[j]);
 #pragma unroll
         for (int i = 1; i <= NP; ++i) dst[(size_t)i * P + gs[j]] = end[(i - 1) * S + l];
         if (D2)
