@@ -404,6 +404,7 @@ static void* adj_kernel(int shape)
            : shape == 2 ? (void*)adjoint_tma_kernel<480, 1>
                         : (void*)adjoint_tma_kernel<256, 2>;
 }
+int adj_tma_consumers(int shape) { return shape == 1 ? 512 : shape == 2 ? 480 : 256; }
 static int adj_threads(int shape) { return shape == 1 ? 544 : shape == 2 ? 512 : 288; }
 
 cudaError_t adj_tma_prepare(int cap, int nst, int shape, int* ctas_per_sm)

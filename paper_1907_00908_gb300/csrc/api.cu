@@ -183,6 +183,8 @@ struct lbmbt_ctx {
     size_t cap_ck = 0;
     float2* d_seg = nullptr;
     size_t cap_seg = 0;
+    float* d_gsite = nullptr;     // resident adjoint: the sites' sensitivities of a segment
+    size_t cap_gs = 0;
     double* d_gacc = nullptr;
     size_t cap_gacc = 0;
     double* d_gout = nullptr;
@@ -312,7 +314,7 @@ extern "C" int lbmbt_destroy(lbmbt_ctx* c)
     cudaFree(c->d_adj_unit_start); cudaFree(c->d_halo); cudaFree(c->d_pair_items); cudaFree(c->d_pair_start);
     cudaFree(c->d_pair_maps);
     cudaFree(c->d_res_blocks); cudaFree(c->d_packets); cudaFree(c->d_mout); cudaFree(c->d_idx);
-    cudaFree(c->d_res_start); cudaFree(c->d_zpart);
+    cudaFree(c->d_res_start); cudaFree(c->d_zpart); cudaFree(c->d_gsite);
     cudaFree(c->d_ck); cudaFree(c->d_seg); cudaFree(c->d_gacc); cudaFree(c->d_gout); cudaFree(c->d_laminit);
     if (c->owned_stream) cudaStreamDestroy(c->owned_stream);
     delete c;
@@ -901,7 +903,7 @@ static bool any_slab(const lbmbt_ctx* c);
 // SMs.  Where they fit it is the fastest sweep at every size measured (us a step,
 // one-step / two-step / resident): 16^3 5.7 / 8.0 / 1.5, 32^3 6.8 / 8.5 / 1.5, 48^3
 // 9.4 / 8.6 / 2.8, 64^3 12.8 / 10.3 / 4.5, eight members of 24^3 8.6 / 8.7 / 2.7.
-static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
+static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, bool adjoint = false)
 {
     c->res_ok = false;
     if (c->kernel_opt != 0 || c->scheme != 0 || c->test_wait_ns > 0 || any_slab(c) || c->n_steps < 2) return LBMBT_OK;
@@ -939,8 +941,9 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
     int cap = 0;
     std::vector<Cut> cuts(descs.size());
     c->res_strip_nx = 0;
-    if (total <= (long long)c->sm_count * resident_max_sites())
-    for (int t = 64; t <= resident_max_sites(); t += t < 1024 ? 64 : 128) {
+    const int most = adjoint ? adj_resident_max_sites() : resident_max_sites();
+    if (total <= (long long)c->sm_count * most)
+    for (int t = 64; t <= most; t += t < 1024 ? 64 : 128) {
         long long n = 0;
         int recv = 0;
         bool ok = true;
@@ -950,10 +953,11 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
             n += (long long)cuts[m].cy * cuts[m].cz;
             recv = std::max(recv, cuts[m].recv);
         }
-        if (ok && n <= c->sm_count && resident_smem(t, recv, c->lattice == 1) <= (size_t)limit) { cap = t; break; }
+        const size_t smem = adjoint ? adj_resident_smem(t, recv) : resident_smem(t, recv, c->lattice == 1);
+        if (ok && n <= c->sm_count && smem <= (size_t)limit) { cap = t; break; }
     }
     // (1000 x 1000: 11.4 us a step against 31 for the one-step sweep)
-    if (!cap && c->lattice == 1 && !links) {   // larger 2-D grids: strips, all of the least height that will do
+    if (!cap && c->lattice == 1 && !links && !adjoint) {   // larger 2-D grids: strips, all of the least height that will do
         for (int h = 1; h <= 8 && !c->res_strip_nx; ++h) {
             long long n = 0;
             int widest = 0;
@@ -1640,6 +1644,29 @@ static int sum_signal(lbmbt_ctx* c)
 // series mode fewer: the parts of Z of every step wait in memory for their sum).
 constexpr long long RES_CHUNK = 1 << 15, RES_SERIES_CHUNK = 1 << 12;
 
+// Arguments of a launch of n steps from step k on (the levels and what is observed
+// are the caller's); takes n stamps.
+static ResArgs resident_args(lbmbt_ctx* c, long long k, long long n)
+{
+    ResArgs r;
+    memset(&r, 0, sizeof r);
+    r.blocks = c->d_res_blocks;
+    r.packets = c->d_packets;
+    r.recv_max = std::max(c->res_recv, 1);
+    r.k0 = (int)k;
+    r.n_steps = (int)n;
+    if (c->res_stamp > 0xffffffffu - (unsigned)n) {   // stamps used up: start over on clean buffers
+        cudaMemsetAsync(c->d_packets, 0, c->cap_pk, c->stream);
+        c->res_stamp = 1;
+    }
+    r.stamp0 = c->res_stamp;
+    c->res_stamp += (unsigned)n;
+    r.sig_step = r.field_step = -1;
+    r.links = c->res_links ? 1 : 0;
+    r.max_links = c->res_max_links;
+    return r;
+}
+
 static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_step)
 {
     const SweepArgs a = sweep_args(c);
@@ -1650,26 +1677,13 @@ static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_ste
         if (rc) return rc;
     }
     for (long long k = c->k_cur, end = c->k_cur + n; k < end;) {
-        ResArgs r;
-        r.blocks = c->d_res_blocks;
-        r.packets = c->d_packets;
-        r.recv_max = std::max(c->res_recv, 1);
-        r.k0 = (int)k;
-        r.n_steps = (int)std::min(chunk, end - k);
+        ResArgs r = resident_args(c, k, std::min(chunk, end - k));
         r.lsrc = (int)((k - c->slot_base) & 1);
         r.ldst = (int)((k + r.n_steps - c->slot_base) & 1);
-        if (c->res_stamp > 0xffffffffu - (unsigned)r.n_steps) {   // stamps used up: start over on clean buffers
-            CU(c, cudaMemsetAsync(c->d_packets, 0, c->cap_pk, c->stream));
-            c->res_stamp = 1;
-        }
-        r.stamp0 = c->res_stamp;
-        c->res_stamp += (unsigned)r.n_steps;
         r.sig_step = sig_step;
         r.field_step = field_step;
         r.series = c->series_mode ? 1 : 0;
         r.zpart = c->d_zpart;
-        r.links = c->res_links ? 1 : 0;
-        r.max_links = c->res_max_links;
         if (c->res_strip_nx) CU(c, launch_strip(a, r, nb, c->res_strip_nx, c->res_smem, c->general, c->stream));
         else
             CU(c, launch_resident(a, r, nb, c->res_sites, c->res_smem, c->lattice == 1, c->general, c->stream));
@@ -2085,6 +2099,34 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
     if (rc) return rc;
     // per-member bases of checkpoints and segment levels
     std::vector<float2*> ckb(n), segb(n);
+    // small grids: resident forward and adjoint (blocks as the adjoint can hold them)
+    bool res = false;
+    if (adj_tma && c->adjoint_opt == 0 && (c->multi_opt == 0 || c->multi_opt == 3)) {
+        if ((rc = plan_resident(c, c->descs, true)) || (rc = build_resident(c))) return rc;
+        res = c->res_ok;
+        c->res_ok = false;   // no prepared run stands on it
+    }
+    const int L_max = (int)std::min<long long>(ck, K);
+    size_t sites = 0;
+    if (res) {
+        for (auto& d : c->descs) sites += (size_t)d.N;
+        rc = grow(c, &c->d_mout, &c->cap_mo, sizeof(float2) * sites);
+        if (!rc) rc = grow(c, &c->d_gsite, &c->cap_gs, sizeof(float) * 3 * sites * L_max);
+        if (rc == LBMBT_ENOMEM) {   // no room: one step a launch
+            cudaGetLastError();
+            c->err.clear();
+            res = false;
+            rc = LBMBT_OK;
+        }
+        c->sig_parts = 16;
+        std::vector<long long> idx(n + 1);
+        std::iota(idx.begin(), idx.end(), 0LL);
+        if (!rc) rc = grow(c, &c->d_idx, &c->cap_ix, sizeof(long long) * idx.size());
+        if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n * c->sig_parts);
+        if (rc) return rc;
+        CU(c, cudaMemcpyAsync(c->d_idx, idx.data(), sizeof(long long) * idx.size(), cudaMemcpyHostToDevice, c->stream));
+        if ((rc = sync(c))) return rc;
+    }
     {
         size_t oc = 0, os = 0;
         for (int m = 0; m < n; ++m) {
@@ -2106,10 +2148,41 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
     const long long k_last = (n_ck - 1) * ck;
     rc = write_ctl(c, (int)(K - 1), -1);
     if (rc) return rc;
-    if (n_ck > 1)
+    // resident: steps k0 .. k0 + ns - 1 from a level of the checkpoints; levels: they go to the segment
+    auto forward = [&](long long k0, long long ns, bool levels) -> int {
+        ResArgs r = resident_args(c, k0, ns);
+        r.lsrc = (int)(k0 / ck);
+        r.ldst = levels ? r.lsrc : r.lsrc + 1;   // a segment's last level is not needed
+        r.sig_step = (int)(K - 1);
+        r.field_step = -1;
+        r.levels = levels ? 1 : 0;
+        CU(c, launch_resident(sweep_args(c), r, (int)c->res_blocks.size(), c->res_sites, c->res_smem, false, c->general,
+                              c->stream));
+        c->launches++;
+        return LBMBT_OK;
+    };
+    std::vector<MemberDesc> rfd;
+    if (res) {
+        // state = the checkpoints, adj = the segment, mout = where M at the end goes
+        rfd = c->descs;
+        size_t at = 0;
+        for (int m = 0; m < n; ++m) {
+            if ((rc = copy_level(m, c->descs[m].state, ckb[m]))) return rc;
+            rfd[m].state = ckb[m];
+            rfd[m].adj = segb[m];
+            rfd[m].mout = c->d_mout + at;
+            at += (size_t)rfd[m].N;
+        }
+        CU(c, cudaMemcpyAsync(c->d_desc, rfd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
+        for (long long s = 0; s < n_ck; ++s)
+            if ((rc = forward(s * ck, std::min<long long>(ck, K - s * ck), s == n_ck - 1))) return rc;
+        c->k_cur = K;
+        if ((rc = sum_signal(c))) return rc;
+    }
+    if (n_ck > 1 && !res)
         for (int m = 0; m < n; ++m)
             if ((rc = copy_level(m, c->descs[m].state, ckb[m]))) return rc;
-    for (long long k = 0; k < K; ++k) {
+    for (long long k = res ? K : 0; k < K; ++k) {
         if (k == k_last) {
             std::vector<MemberDesc> fd = c->descs;
             for (int m = 0; m < n; ++m) {
@@ -2130,8 +2203,10 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
             }
     }
     c->k_cur = K;
-    CU(c, launch_reduce(c->d_partial, part_start(c), part_per(c), n, c->d_Z, nullptr, 0, c->d_ctl, c->stream));
-    c->launches++;
+    if (!res) {
+        CU(c, launch_reduce(c->d_partial, part_start(c), part_per(c), n, c->d_Z, nullptr, 0, c->d_ctl, c->stream));
+        c->launches++;
+    }
     std::vector<double2> Z(n);
     CU(c, cudaMemcpyAsync(Z.data(), c->d_Z, sizeof(double2) * n, cudaMemcpyDeviceToHost, c->stream));
     if ((rc = sync(c))) return rc;
@@ -2151,6 +2226,13 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
     for (int m = 0; m < n; ++m) {
         rd[m].adj = c->descs[m].state;
         rd[m].state = segb[m];
+    }
+    if (res) {   // and where the sites' sensitivities go
+        size_t at = 0;
+        for (int m = 0; m < n; ++m) {
+            rd[m].field = reinterpret_cast<float2*>(c->d_gsite + at);
+            at += 3 * (size_t)rd[m].N * L_max;
+        }
     }
     CU(c, cudaMemcpyAsync(c->d_desc, rd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
     CU(c, cudaMemsetAsync(c->d_gacc, 0, sizeof(double) * NGACC * n_gslots, c->stream));
@@ -2185,6 +2267,24 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
     int parity = 1;
     for (long long seg = n_ck - 1; seg >= 0; --seg) {
         const long long k0 = seg * ck, k1 = std::min(K, k0 + ck);
+        if (res) {
+            if (seg < n_ck - 1) {   // the last segment's levels are in place from the forward pass
+                CU(c, cudaMemcpyAsync(c->d_desc, rfd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
+                if ((rc = forward(k0, ck, true))) return rc;
+                CU(c, cudaMemcpyAsync(c->d_desc, rd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
+            }
+            ResArgs r = resident_args(c, k0, k1 - k0);
+            r.lsrc = r.ldst = 0;
+            aa.k = (int)k1;
+            aa.first = (k1 == K) ? 1 : 0;
+            aa.fwd_slot = (int)(k1 - 1 - k0);
+            CU(c, launch_adjoint_resident(aa, r, (int)c->res_blocks.size(), c->res_sites,
+                                          adj_resident_smem(c->res_sites, c->res_recv), c->general, c->stream));
+            CU(c, launch_adjoint_sum(aa, c->n_adj_units, (int)(k1 - k0), adj_grid, adj_tma_consumers(c->adj_shape_used),
+                                     c->adj_shape_used == 0 ? 2 : 1, adj_tma_slots_per_unit(), c->stream));
+            c->launches += 2;
+            continue;
+        }
         if (seg < n_ck - 1) {   // the last segment's levels are in place from the forward pass
             for (int m = 0; m < n; ++m) {
                 const size_t lv = (size_t)7 * c->descs[m].plane;

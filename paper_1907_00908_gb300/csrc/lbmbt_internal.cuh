@@ -227,6 +227,8 @@ struct ResArgs {
     int max_links;                // listed links of a block at most (rounded up to even)
     int series;                   // 1: zpart[n][block] = the block's part of Z after each step
     double2* zpart;
+    int levels;                   // 1: the levels of steps k0 .. k0 + n_steps - 1 go to the member's
+                                  // adj, one after the other (gradient segments)
 };
 int resident_max_sites();         // sites of a block
 size_t resident_smem(int sites, int recv, bool d2);
@@ -275,11 +277,24 @@ struct AdjointArgs {
 // run: consecutive tiles per block (the block keeps its gradient partials over them)
 cudaError_t launch_adjoint(const AdjointArgs& a, long long n_tiles, int block, int spt, int run, cudaStream_t st);
 // Sums gacc slots [tile_start[m]*per, tile_start[m+1]*per) per member.
+// resident adjoint (adjoint_resident.cu): steps a.k, a.k - 1, .. of r.n_steps; the
+// forward level of step a.k - 1 is in slot a.fwd_slot of the member's state, that of
+// the next in the slot before; nu^k is adj level r.lsrc, the result goes to
+// r.ldst; the sites' sensitivities go to the member's field, floats [step][3][N],
+// and launch_adjoint_sum adds them to gacc as the bulk-copy adjoint would (its
+// grid, consumer threads, sites per thread and slots per unit).
+int adj_resident_max_sites();
+size_t adj_resident_smem(int sites, int recv);
+cudaError_t launch_adjoint_sum(const AdjointArgs& a, long long n_units, int n_steps, int grid, int threads, int spt,
+                               int slots, cudaStream_t st);
+cudaError_t launch_adjoint_resident(const AdjointArgs& a, const ResArgs& r, int n_blocks, int max_sites, size_t smem,
+                                    bool general, cudaStream_t st);
 cudaError_t launch_reduce_grad(const double* gacc, const long long* tile_start, int per, int n_members, double* out,
                                cudaStream_t st);
 // bulk-copy adjoint (adjoint_tma.cu)
 int adj_tma_slots_per_unit();
 int adj_tma_max_sites(int shape);
+int adj_tma_consumers(int shape);          // threads that have sites; sites per thread: 2 for shape 0, else 1
 cudaError_t adj_tma_prepare(int cap, int nst, int shape, int* ctas_per_sm);
 cudaError_t launch_adjoint_tma(const AdjointArgs& a, long long n_units, int cap, int nst, int shape, int grid,
                                cudaStream_t st);

@@ -1,6 +1,7 @@
 // packets.cuh -- face values sent between the blocks of one cooperative launch:
 // 16-byte packets {re, stamp, im, stamp} that the receiver polls (see
-// sweep_resident.cu for why no packet is lost or taken twice).
+// sweep_resident.cu for why no packet is lost or taken twice), and the site flags
+// of the kernels that cut a grid into blocks.
 #pragma once
 #include "lbmbt_internal.cuh"
 #include "tma_common.cuh"
@@ -41,16 +42,6 @@ __device__ __noinline__ uint4 await(const uint4* from, unsigned stamp, bool& dea
 // -z, +z), 10 a site at all, 11..14 in the layer behind a face of the block, 16..21
 // the membrane links (of the half-link rule), 22..23 the phase.
 enum : unsigned { S_GRID = 63u, S_SEND = 0x3c0u, S_SEND2 = 0x7800u, S_ON = 1024u };
-
-// A listed link: elements of a level of own g_ib, g_ib behind, own g_i, g_i(y),
-// g_i behind y, g_ib(y); per value 4 bits, 1 + the boundary factor it takes and
-// 8 if conjugated first; the coefficients.
-struct LinkEntry {
-    uint16_t at[6];
-    uint32_t face;
-    float A[3], B[3];
-};
-static_assert(sizeof(LinkEntry) == 40, "link entry");
 
 }  // namespace
 }  // namespace lbmbt

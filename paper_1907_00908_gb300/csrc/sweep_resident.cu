@@ -44,6 +44,16 @@ namespace {
 constexpr int RES_NT = 512;           // threads of a block
 constexpr int RES_MAX_SITES = 2048;   // sites of a block: 13 x 8 B each in shared memory
 
+// A listed link: elements of a level of own g_ib, g_ib behind, own g_i, g_i(y),
+// g_i behind y, g_ib(y); per value 4 bits, 1 + the boundary factor it takes and
+// 8 if conjugated first; the coefficients.
+struct LinkEntry {
+    uint16_t at[6];
+    uint32_t face;
+    float A[3], B[3];
+};
+static_assert(sizeof(LinkEntry) == 40, "link entry");
+
 // cmul() with its roundings written out: as the register sweep's reads beyond a
 // face come out of the compiler, so that the fields are the same bits.
 __device__ __forceinline__ float2 turn(float2 a, float2 b)
@@ -229,6 +239,17 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
     if (t < 6) s_fac[0][t] = __ldg(a.fac + ((size_t)r.k0 * a.n_members + b.m) * 6 + t);
     if (t == 6) s_f[0] = __ldg(d->fw + r.k0);
 
+    // gradient segments: level n of the launch, n < n_steps, as it is at the start of step n
+    auto put_level = [&](int n, int l, unsigned s, u64 v0, const u64* v) {
+        u64* to = reinterpret_cast<u64*>(d->adj) + (size_t)n * 7 * P + s;
+        __stcs(to, v0);
+        for (int i = 1; i <= NP; ++i) __stcs(to + (size_t)i * P, v[(i - 1) * S + l]);
+    };
+    if (!D2 && r.levels)
+#pragma unroll
+        for (int j = 0; j < SPT; ++j)
+            if (fl[j] & S_ON) put_level(0, t + j * RES_NT, gs[j], p0[j], reinterpret_cast<const u64*>(lev));
+
     bool dead = false;
     const uint4* const mine = r.packets + (size_t)blockIdx.x * 4 * r.recv_max;
     // sends the populations that leave the block at a site on its faces, with the stamp of step n
@@ -371,6 +392,7 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
                 send_faces(F, pl[j], n + 1, unpk(g[3]), unpk(g[4]), unpk(g[NP - 1]), unpk(g[NP]));
 #pragma unroll
             for (int i = 1; i <= NP; ++i) reinterpret_cast<u64*>(nxt)[(i - 1) * S + l] = g[i];
+            if (!D2 && r.levels && n + 1 < r.n_steps) put_level(n + 1, l, gs[j], g[0], reinterpret_cast<const u64*>(nxt));
             if (do_sig || do_fld || r.series) {
                 const float2 v = unpk(M);
                 if (do_sig) mout[gs[j]] = v;

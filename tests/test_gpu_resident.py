@@ -151,3 +151,31 @@ def test_resident_sweep_with_membrane_positions(lb, shape, bc, gG, wave, n, latt
             out.append((fld.cpu().numpy(), r))
     assert np.array_equal(out[0][0], out[1][0])
     assert np.abs(out[0][1]["series"] - out[1][1]["series"]).max() <= 2.0 ** -22 * g.n_sites
+
+
+# one and two sites a thread, one segment and several, a short last one, faces of
+# every kind, two members of different geometry
+@pytest.mark.parametrize("shapes,bc,gG,wave,n,every", [
+    ([(48, 48, 48)], (0, 0, 0), (0.3, 0.2, 0.1), "pgse", 30, 8),
+    ([(20, 24, 32)], (0, 0, 0), (0.2, -0.3, 0.1), "cos", 17, 64),
+    ([(9, 31, 48)], (1, 1, 1), (0.0, 0.0, 0.4), "pgse", 21, 5),
+    ([(40, 30, 16)], (1, 0, 1), (0.4, 0.0, 0.0), "pgse", 12, 4),
+    ([(16, 32, 16), (7, 9, 48)], (0, 0, 0), (0.1, 0.2, 0.1), "pgse", 19, 6),
+])
+def test_resident_gradient_is_the_bulk_copy_one(lb, shapes, bc, gG, wave, n, every):
+    """Signal, gradients: the same arithmetic and the same groups of partial
+    sums, so the same numbers (1e-12 for the FP64 sums of the signal)."""
+    geoms = [_geom(s, sum(s)) for s in shapes]
+    f = _wave(wave, n)
+    out = []
+    for multi in (0, 1):
+        with _solver(lb, multi, geoms, bc, gG, f, 0.05, 0) as s:
+            m = lb.Solver.members([gG] * len(geoms), list(range(len(geoms))), 0.05)
+            c0 = s.launch_count()
+            r = s.grad_batch(m, checkpoint_every=every)
+            out.append((r, s.launch_count() - c0))
+    assert out[0][1] < out[1][1]   # it ran
+    assert np.allclose(out[0][0]["Z"], out[1][0]["Z"], rtol=1e-12, atol=0)
+    for k in ("dD", "dT2", "dkappa"):
+        a, b = out[0][0][k], out[1][0][k]
+        assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max(), (k, a, b)
