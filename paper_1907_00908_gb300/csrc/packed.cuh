@@ -73,11 +73,13 @@ __device__ __forceinline__ void mix_if(unsigned mk, u64& v, u64 o, u64 s2)
 template <int N>
 __device__ __forceinline__ u64 react_collide(u64 (&g)[N], float2 q, float om, float w0 = W0, float wi = WI)
 {
-    const u64 qx = pk(q.x, q.x), qy = pk(-q.y, q.y);
+    // the inner product takes the halves crosswise: two scalar operations, where a
+    // packed one would need them swapped first
+    const u64 qx = pk(q.x, q.x);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         const float2 v = unpk(g[i]);
-        g[i] = fma2(g[i], qx, fma2(pk(v.y, v.x), qy, g[i]));
+        g[i] = fma2(g[i], qx, pk(__fmaf_rn(-v.y, q.y, v.x), __fmaf_rn(v.x, q.y, v.y)));
     }
     u64 m = g[0];
 #pragma unroll

@@ -234,13 +234,16 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
             if (zb + q <= zl) issue(zb + q, q);
     __syncthreads();     // the shared constants are set
     ulonglong2 c5, o6;   // p5 of the plane below, own p6 of this plane
-    unsigned mkn;        // mask bytes of the next plane
+    // Mask bytes of the next plane and of the one after: a plane's are asked for two planes
+    // ahead (one ahead they arrived late: 128^3 cylinders 50.4 against 49.3 ms)
+    unsigned mkn, mkn2 = 0u;
     {
         const int z = wrapz(zb);
         c5 = make_ulonglong2(0ull, 0ull);
         if (z > 0 || !mir) c5 = load2(src + (size_t)(z > 0 ? z - 1 : nz - 1) * sxy + (5 * P + sa));
         o6 = load2(src + (size_t)z * sxy + (6 * P + sa));
         mkn = load_mask(z);
+        if (zb < zl) mkn2 = load_mask(wrapz(zb + 1));
     }
     // reaction rotation: the x and y parts are the column's
     const float2* __restrict__ et = d->etab;
@@ -341,8 +344,9 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
             const int z = wrapz(zi);
             const ulonglong2* __restrict__ q = sin + st * SW + t;
             const float2 ez = ezn;
+            mkn = mkn2;
+            if (zi + 1 < zl) mkn2 = load_mask(wrapz(zi + 2));
             if (zi < zl) {
-                mkn = load_mask(wrapz(zi + 1));
                 if (tz) ezn = __ldg(etz + wrapz(zi + 1));
             }
             u64 ga[Q], gb[Q];
@@ -541,13 +545,12 @@ __global__ void pair_init_kernel(const MemberDesc* __restrict__ members, int n_m
     }
 }
 
-// 224 threads x 2 columns, two blocks per SM (114 KB of shared memory each):
-// one block's barriers and item start are hidden by the other.
 // 256 threads x 2 columns, two blocks per SM (128 registers, 101 KB of shared
 // memory each): one block's barrier and item start are hidden by the other.
-// Measured (512^3 tissue / 128^3 cylinders / 16 odd packs, ms a pass): 222 / 49.7
-// / 27.7; 512 threads x 1 block 223 / 50.2 / 32.5; 448 x 1 with a third stage
-// 226 / 52.4 / 34.5; 224 x 2 with a third stage 230 / 55.7 / 31.2.
+// Measured before the masks were asked for two planes ahead (512^3 tissue / 128^3
+// cylinders / 16 odd packs, ms a pass): 222 / 49.7 / 27.7; 512 threads x 1 block 223 /
+// 50.2 / 32.5; 448 x 1 with a third stage 226 / 52.4 / 34.5; 224 x 2 with a third stage
+// 230 / 55.7 / 31.2.  Since: 222 / 49.2 / 27.5.
 constexpr int PNT = 256, PMB = 2;
 constexpr size_t PAIR_SMEM = (size_t)(PAIR_STAGES * stage_words(PNT) + 2 * 4 * PNT) * sizeof(ulonglong2) + 2 * PNT * sizeof(float4);
 
