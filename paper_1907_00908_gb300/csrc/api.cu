@@ -2077,8 +2077,9 @@ static size_t grad_bytes_per_member(const lbmbt_ctx* c, long long plane, int ck)
 
 // One group of members: checkpointed forward pass, then segments in reverse:
 // recompute the segment's forward levels from its checkpoint, then run the
-// adjoint sweep back through it.
-static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, double* sig, double* dD, double* dT2,
+// adjoint sweep back through it.  The last `keep` segments are not recomputed:
+// the forward pass writes their levels where the adjoint reads them.
+static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int keep, double* sig, double* dD, double* dT2,
                       double* dk)
 {
     const int saved_block = c->block;
@@ -2091,7 +2092,13 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
     size_t lvl_total = 0;
     for (auto& d : c->descs) lvl_total += (size_t)7 * d.plane;
     rc = grow(c, &c->d_ck, &c->cap_ck, lvl_total * n_ck * sizeof(float2));
-    if (!rc) rc = grow(c, &c->d_seg, &c->cap_seg, lvl_total * (ck + 1) * sizeof(float2));
+    if (!rc) rc = grow(c, &c->d_seg, &c->cap_seg, lvl_total * ((size_t)keep * ck + 1) * sizeof(float2));
+    if (rc == LBMBT_ENOMEM && keep > 1) {   // no room after all: the last segment only
+        cudaGetLastError();
+        c->err.clear();
+        keep = 1;
+        rc = grow(c, &c->d_seg, &c->cap_seg, lvl_total * (ck + 1) * sizeof(float2));
+    }
     const bool adj_tma = c->adjoint_opt == 2 || (c->adjoint_opt == 0 && c->adj_tma_ok);
     if (c->adjoint_opt == 2 && !c->adj_tma_ok)
         return fail(c, LBMBT_EINVAL, "bulk-copy adjoint needs nx %% 16 == 0 and nx <= %d", adj_tma_max_sites(1));
@@ -2137,7 +2144,7 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
             ckb[m] = c->d_ck + oc;
             segb[m] = c->d_seg + os;
             oc += lv * n_ck;
-            os += lv * (ck + 1);
+            os += lv * ((size_t)keep * ck + 1);
         }
     }
     auto copy_level = [&](int m, const float2* from, float2* to) -> int {
@@ -2145,20 +2152,22 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
         CU(c, cudaMemcpyAsync(to, from, lv * sizeof(float2), cudaMemcpyDeviceToDevice, c->stream));
         return LBMBT_OK;
     };
-    // forward with checkpoints u^0, u^ck, u^2ck, ...; from the last
+    // forward with checkpoints u^0, u^ck, u^2ck, ...; from the first kept
     // segment's first step on it writes its levels straight into the segment
-    // buffer (slot k - k_last), so that segment is not recomputed
-    const long long k_last = (n_ck - 1) * ck;
+    // buffer (slot k - k_keep)
+    const long long k_keep = (n_ck - keep) * ck;
     rc = write_ctl(c, (int)(K - 1), -1);
     if (rc) return rc;
-    // resident: steps k0 .. k0 + ns - 1 from a level of the checkpoints; levels: they go to the segment
-    auto forward = [&](long long k0, long long ns, bool levels) -> int {
+    // resident: steps k0 .. k0 + ns - 1 from a level of the checkpoints; levels: they go to
+    // the segment buffer from slot `slot` on
+    auto forward = [&](long long k0, long long ns, bool levels, long long slot) -> int {
         ResArgs r = resident_args(c, k0, ns);
         r.lsrc = (int)(k0 / ck);
-        r.ldst = levels ? r.lsrc : r.lsrc + 1;   // a segment's last level is not needed
+        r.ldst = std::min(r.lsrc + 1, (int)n_ck - 1);   // the next checkpoint (the last one's: a level not needed)
         r.sig_step = (int)(K - 1);
         r.field_step = -1;
         r.levels = levels ? 1 : 0;
+        r.level0 = (int)slot;
         CU(c, launch_resident(sweep_args(c), r, (int)c->res_blocks.size(), c->res_sites, c->res_smem, false, c->general,
                               c->stream));
         c->launches++;
@@ -2177,16 +2186,18 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
             at += (size_t)rfd[m].N;
         }
         CU(c, cudaMemcpyAsync(c->d_desc, rfd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
-        for (long long s = 0; s < n_ck; ++s)
-            if ((rc = forward(s * ck, std::min<long long>(ck, K - s * ck), s == n_ck - 1))) return rc;
+        for (long long s = 0; s < n_ck; ++s) {
+            const bool kept = s >= n_ck - keep;
+            if ((rc = forward(s * ck, std::min<long long>(ck, K - s * ck), kept, kept ? s * ck - k_keep : 0))) return rc;
+        }
         c->k_cur = K;
         if ((rc = sum_signal(c))) return rc;
     }
-    if (n_ck > 1 && !res)
+    if (k_keep > 0 && !res)
         for (int m = 0; m < n; ++m)
             if ((rc = copy_level(m, c->descs[m].state, ckb[m]))) return rc;
     for (long long k = res ? K : 0; k < K; ++k) {
-        if (k == k_last) {
+        if (k == k_keep) {
             std::vector<MemberDesc> fd = c->descs;
             for (int m = 0; m < n; ++m) {
                 const size_t lv = (size_t)7 * c->descs[m].plane;
@@ -2195,11 +2206,11 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
             }
             CU(c, cudaMemcpyAsync(c->d_desc, fd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
             c->k_cur = k;
-            if ((rc = write_ctl(c, (int)(K - 1), -1, (int)k, ck + 1))) return rc;
+            if ((rc = write_ctl(c, (int)(K - 1), -1, (int)k, keep * ck + 1))) return rc;
         }
         if ((rc = issue_step(c))) return rc;
         const long long kn = k + 1;
-        if (kn % ck == 0 && kn < k_last)
+        if (kn % ck == 0 && kn < k_keep)
             for (int m = 0; m < n; ++m) {
                 const size_t lv = (size_t)7 * c->descs[m].plane;
                 if ((rc = copy_level(m, c->descs[m].state + (kn & 1) * lv, ckb[m] + (kn / ck) * lv))) return rc;
@@ -2270,17 +2281,19 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
     int parity = 1;
     for (long long seg = n_ck - 1; seg >= 0; --seg) {
         const long long k0 = seg * ck, k1 = std::min(K, k0 + ck);
+        const bool kept = seg >= n_ck - keep;   // its levels are in place from the forward pass
+        const long long base = kept ? k_keep : k0;   // the step of slot 0
         if (res) {
-            if (seg < n_ck - 1) {   // the last segment's levels are in place from the forward pass
+            if (!kept) {
                 CU(c, cudaMemcpyAsync(c->d_desc, rfd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
-                if ((rc = forward(k0, ck, true))) return rc;
+                if ((rc = forward(k0, ck, true, 0))) return rc;
                 CU(c, cudaMemcpyAsync(c->d_desc, rd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
             }
             ResArgs r = resident_args(c, k0, k1 - k0);
             r.lsrc = r.ldst = 0;
             aa.k = (int)k1;
             aa.first = (k1 == K) ? 1 : 0;
-            aa.fwd_slot = (int)(k1 - 1 - k0);
+            aa.fwd_slot = (int)(k1 - 1 - base);
             CU(c, launch_adjoint_resident(aa, r, (int)c->res_blocks.size(), c->res_sites,
                                           adj_resident_smem(c->res_sites, c->res_recv), c->general, c->stream));
             CU(c, launch_adjoint_sum(aa, c->n_adj_units, (int)(k1 - k0), adj_grid, adj_tma_consumers(c->adj_shape_used),
@@ -2288,13 +2301,13 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
             c->launches += 2;
             continue;
         }
-        if (seg < n_ck - 1) {   // the last segment's levels are in place from the forward pass
+        if (!kept) {
             for (int m = 0; m < n; ++m) {
                 const size_t lv = (size_t)7 * c->descs[m].plane;
                 if ((rc = copy_level(m, ckb[m] + seg * lv, segb[m]))) return rc;
             }
         }
-        if (seg < n_ck - 1 && k1 - k0 - 1 > 0) {
+        if (!kept && k1 - k0 - 1 > 0) {
             c->k_cur = k0;
             if ((rc = write_ctl(c, -1, -1, (int)k0, ck + 1))) return rc;
             for (long long k = k0; k < k1 - 1; ++k)
@@ -2303,7 +2316,7 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, doub
         for (long long k = k1; k > k0; --k) {
             aa.k = (int)k;
             aa.first = (k == K) ? 1 : 0;
-            aa.fwd_slot = (int)(k - 1 - k0);
+            aa.fwd_slot = (int)(k - 1 - base);
             aa.lam_parity = parity;
             aa.fprev = (float)c->f[k - 1];
             if (adj_tma)
@@ -2371,7 +2384,7 @@ extern "C" int lbmbt_grad_batch(lbmbt_ctx* c, int n_members, const lbmbt_member*
     int m0 = 0;
     c->grad_groups = 0;
     while (m0 < n_members) {
-        size_t used = 0;
+        size_t used = 0, seg_bytes = 0;   // of the group; of a segment's levels
         int m1 = m0;
         while (m1 < n_members) {
             const lbmbt_member& mm = members[m1];
@@ -2381,10 +2394,21 @@ extern "C" int lbmbt_grad_batch(lbmbt_ctx* c, int n_members, const lbmbt_member*
             const size_t b = grad_bytes_per_member(c, plane, ck);
             if (m1 > m0 && used + b > budget) break;
             used += b;
+            seg_bytes += (size_t)ck * 7 * plane * sizeof(float2);
             ++m1;
         }
         if (used > budget) return fail(c, LBMBT_ENOMEM, "one member needs %zu bytes for the adjoint", used);
-        rc = grad_group(c, m1 - m0, members + m0, ck, signal_out + 3 * m0, dS_dD + (size_t)m0 * c->n_phases,
+        // Each further segment kept saves its recompute, ck - 1 of about 4.5 ck
+        // forward-step times of its gradient, and takes ck levels.  A quarter of the
+        // device memory that is free (before the first call) goes to it at most, and no
+        // more than the group itself takes: a caller who sets checkpoint_every low to
+        // leave room gets at most twice that.  10 members, 96^3, 128 steps, every 64: both
+        // segments kept, 58.7 ms against 69.8 (first call 66.9 against 74.2, with the
+        // allocation); 48^3, 400 steps: two of seven, 5.8 against 6.0.
+        const long long n_ck = (c->n_steps + ck - 1) / ck;
+        const size_t room = std::min({used, (free_b + held) / 4, budget - used});
+        const int keep = (int)std::min<long long>(n_ck, 1 + (long long)(room / seg_bytes));
+        rc = grad_group(c, m1 - m0, members + m0, ck, keep, signal_out + 3 * m0, dS_dD + (size_t)m0 * c->n_phases,
                         dS_dT2 + (size_t)m0 * c->n_phases, dS_dkappa + m0);
         if (rc) return rc;
         ++c->grad_groups;

@@ -228,7 +228,8 @@ struct ResArgs {
     int series;                   // 1: zpart[n][block] = the block's part of Z after each step
     double2* zpart;
     int levels;                   // 1: the levels of steps k0 .. k0 + n_steps - 1 go to the member's
-                                  // adj, one after the other (gradient segments)
+                                  // adj, one after the other from slot level0 (gradient segments)
+    int level0;
 };
 int resident_max_sites();         // sites of a block
 size_t resident_smem(int sites, int recv, bool d2);

@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
 
     // gradient segments: level n of the launch, n < n_steps, as it is at the start of step n
     auto put_level = [&](int n, int l, unsigned s, u64 v0, const u64* v) {
-        u64* to = reinterpret_cast<u64*>(d->adj) + (size_t)n * 7 * P + s;
+        u64* to = reinterpret_cast<u64*>(d->adj) + (size_t)(r.level0 + n) * 7 * P + s;
         __stcs(to, v0);
         for (int i = 1; i <= NP; ++i) __stcs(to + (size_t)i * P, v[(i - 1) * S + l]);
     };

@@ -245,3 +245,27 @@ def test_bulk_copy_adjoint_shape_falls_back_for_wide_rows(lb):
     a = _logvec(out[1], [2.0, 1.0], [80.0, 50.0], 0.05)
     b = _logvec(out[2], [2.0, 1.0], [80.0, 50.0], 0.05)
     assert np.abs(a - b).max() <= 1e-5 * np.abs(a).max()
+
+
+# checkpoint_every of a 40-step schedule against one segment of 40.  Of the n
+# segments the last 1 + (3 + n + every) // every are kept on an empty device and the
+# rest recomputed: 40 of 40; 7 of 14, the last of one step; 5 of 6 and a short
+# last one; 3 of 5; 2 of 3 and a short last one; 2 of 2 and a last one of one step.
+@pytest.mark.parametrize("kernel", [0, 1, 2])   # resident, register, bulk-copy adjoint
+@pytest.mark.parametrize("every", [1, 3, 7, 8, 16, 39])
+def test_kept_and_recomputed_segments_give_the_same_bits(lb, kernel, every):
+    K = 40
+    c = CASES["cylinders32_bulk"]
+    geom = c["geom"]()
+    f = np.cos(np.arange(K) * 0.2)
+    f[:12] = 1.0
+    gGs = [np.array(d) * 0.3 for d in ((0.6, -0.48, 0.64), (0.0, 1.0, 0.0))]
+    out = []
+    for ck in (K, every):
+        s = _setup(lb, geom, c["bc"], c["D"], c["T2"], c["kap"], c["dt"], f, gGs[0])
+        s.set_option(lb.OPT_ADJOINT_KERNEL, kernel)
+        out.append(s.grad_batch(lb.Solver.members(gGs, 0, c["kap"]), checkpoint_every=ck))
+        s.close()
+    # the same steps on the same levels, their sums added in the same order
+    for key in ("S", "dD", "dT2", "dkappa"):
+        np.testing.assert_array_equal(out[0][key], out[1][key])
