@@ -2401,12 +2401,13 @@ extern "C" int lbmbt_grad_batch(lbmbt_ctx* c, int n_members, const lbmbt_member*
         // Each further segment kept saves its recompute, ck - 1 of about 4.5 ck
         // forward-step times of its gradient, and takes ck levels.  A quarter of the
         // device memory that is free (before the first call) goes to it at most, and no
-        // more than the group itself takes: a caller who sets checkpoint_every low to
+        // more than the group itself takes (nothing when the members need several groups:
+        // those fill the memory already): a caller who sets checkpoint_every low to
         // leave room gets at most twice that.  10 members, 96^3, 128 steps, every 64: both
         // segments kept, 58.7 ms against 69.8 (first call 66.9 against 74.2, with the
         // allocation); 48^3, 400 steps: two of seven, 5.8 against 6.0.
         const long long n_ck = (c->n_steps + ck - 1) / ck;
-        const size_t room = std::min({used, (free_b + held) / 4, budget - used});
+        const size_t room = m1 - m0 < n_members ? 0 : std::min({used, (free_b + held) / 4, budget - used});
         const int keep = (int)std::min<long long>(n_ck, 1 + (long long)(room / seg_bytes));
         rc = grad_group(c, m1 - m0, members + m0, ck, keep, signal_out + 3 * m0, dS_dD + (size_t)m0 * c->n_phases,
                         dS_dT2 + (size_t)m0 * c->n_phases, dS_dkappa + m0);
