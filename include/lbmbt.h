@@ -243,8 +243,9 @@ typedef struct {
 
 /*
  * Batched run: n_members independent runs that share the set waveform f, dt
- * and phases, advanced together by one launch per time step over a work list
- * of (member, tile) (captured in a CUDA graph when enabled).  Members on the
+ * and phases, advanced together over one work list of all members: one launch
+ * per time step or per two (captured in a CUDA graph when enabled), or one for
+ * all steps where the grids fit on chip (LBMBT_OPT_MULTI_STEP).  Members on the
  * same geometry share its mask.  signal_out (host) [n_members][3] as in
  * lbmbt_run; series_out (host) [n_members][n_steps][2] or NULL.
  */
@@ -312,7 +313,10 @@ enum {
     LBMBT_OPT_KERNEL = 5,    /* 0 (default) auto, 1 register sweep, 2 bulk-copy
                                 (TMA) sweep; auto takes the bulk-copy sweep when
                                 every member has nx % 16 == 0 and nx <= 1024  */
-    LBMBT_OPT_KERNEL_USED = 6, /* read-only: 1 or 2 for the prepared run, else 0 */
+    LBMBT_OPT_KERNEL_USED = 6, /* read-only: 1 or 2 for the prepared run, else 0
+                                (the one-step sweep of these grids, by which
+                                a two-step or resident run sums its signals;
+                                LBMBT_OPT_MULTI_STEP_USED tells what runs)     */
     LBMBT_OPT_STAGES = 7,    /* shared-memory stages of the bulk-copy sweep, 2..6
                                 as far as they fit (3 of 1024-site units); more
                                 than fit give EINVAL                          */
@@ -391,7 +395,8 @@ enum {
                                 (default) auto: all of them in one launch
                                 (resident sweep) where the grids fit on chip,
                                 else two (two-step sweep) where nx, ny, nz >= 4
-                                on D3Q7 with half-link membranes, else one.  1
+                                on D3Q7 with half-link membranes and the planes
+                                are no thin columns, else one.  1
                                 one; 2 two where it can run; 3 resident where
                                 the grids fit.  The fields are the same bits */
     LBMBT_OPT_MULTI_STEP_USED = 19 /* read-only: 1, 2 or 3 for the prepared

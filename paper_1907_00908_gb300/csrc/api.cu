@@ -1058,6 +1058,10 @@ static int build_resident(lbmbt_ctx* c)
 // + 2 threads.  Narrow rows waste sectors at their ends.
 struct PairTiles { int tx, ty, w, h; };
 
+// what a tile of w columns a row costs more than a wide one (short rows: ghosts and
+// half-used sectors)
+static double pair_narrow(int w) { return 1.0 + 3.0 / (w + 2); }
+
 static PairTiles pair_tiles(int nx, int ny, int nt)
 {
     PairTiles best = {0, 0, 0, 0};
@@ -1070,7 +1074,7 @@ static PairTiles pair_tiles(int nx, int ny, int nt)
         if (w < 8 && best.tx) break;
         const int hm = std::min(ny, nt / ex - 2);
         const int ty = (ny + hm - 1) / hm, n = (nx + w - 1) / w;
-        const double cost = (double)n * ty * (1.0 + 3.0 / (w + 2));
+        const double cost = (double)n * ty * pair_narrow(w);
         if (cost < bc) { bc = cost; best = {n, ty, w, (ny + ty - 1) / ty}; }
     }
     return best;
@@ -1081,11 +1085,37 @@ static PairTiles pair_tiles(int nx, int ny, int nt)
 // the resident sweep's grids it was the faster one at every size measured (us a
 // step, one-step / two-step): 65^3 13.0 / 12.8, 72^3 17.0 / 10.3, 4 x 300 x 300 16.1
 // / 9.8, 96^3 22.1 / 16.6, 128^3 46.5 / 36.2, 40 members of 30^3 43.7 / 28.1.
+//
+// Not on thin columns: a tile holds one plane, and a plane of few sites leaves most of
+// its threads (and, with its ghosts, most of its rows in memory) without any.  By the
+// share of the tiles' columns that are sites, narrow tiles weighted as in pair_tiles(),
+// for nx x ny x nz, us a step one-step / two-step: 0.02 4 x 4 x 65536 39 / 254; 0.10
+// 8 x 8 x 16384 39 / 77; 0.23 12 x 12 x 20000 90 / 96; 0.27 5 x 150 x 2000 53 / 61; 0.28
+// 13 x 13 x 20000 103 / 122; 0.30 5 x 300 x 300 19.2 / 19.6; 0.31 4 x 1000 x 1000 114 /
+// 106; 0.32 14 x 14 x 20000 117 / 98; 0.34 20 x 20 x 10000 120 / 96; 0.37 6 x 300 x 300
+// 20.9 / 16.6; 160 members of 12^3 30 / 37, of 20^3 53 / 49.  The line is for the
+// register sweep; the bulk-copy sweep's units of rows are worse on such planes (0.23
+// 32 x 4 x 20000 231 / 96, 0.43 16 x 16 x 4096 55 / 28), so where it would run the
+// two-step sweep does.
+constexpr double PAIR_FILL = 0.30;
+
 static bool pair_eligible(const lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
 {
     if (c->kernel_opt != 0 || c->scheme != 0 || c->lattice != 0 || c->test_wait_ns > 0 || any_slab(c)) return false;
-    for (auto& d : descs)
+    bool bulk = true;   // the one-step sweep would be the bulk-copy one
+    double sites = 0, room = 0;
+    for (auto& d : descs) {
         if (d.dlt || d.nz < 4 || d.nx < 4 || d.ny < 4) return false;   // a column is near one face of an axis only
+        // with its ghosts, offsets within a level stay below 2^32 (they do not on
+        // thin grids of more than 10^8 sites, whose ghosts are most of the state)
+        const long long wide = (d.nx + 2 * pair_ghost() + 1) / 2 * 2, high = d.ny + 2 * pair_ghost();
+        if (7 * (wide * high * d.nz + 63) >= (1LL << 32)) return false;
+        bulk = bulk && d.nx % 16 == 0 && d.nx <= 1024;
+        const PairTiles t = pair_tiles(d.nx, d.ny, pair_threads());
+        sites += (double)d.N;
+        room += 2.0 * pair_threads() * t.tx * t.ty * d.nz * pair_narrow(t.w);
+    }
+    if (c->multi_opt == 0 && !bulk && sites < PAIR_FILL * room) return false;
     return c->n_steps >= 2;
 }
 

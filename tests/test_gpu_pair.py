@@ -89,6 +89,29 @@ def test_two_step_sweep_gives_the_one_step_bits(lb, shape, bc, gG, wave, n, kap)
     assert np.abs(out[0][1]["series"] - out[1][1]["series"]).max() <= 2.0 ** -22 * g.n_sites
 
 
+# nz x ny x nx: columns of planes too thin for the tiles, by themselves and among
+# others, and the ones just above; rows of a multiple of 16 whatever the plane
+@pytest.mark.parametrize("shapes,used", [
+    ([(9000, 5, 7)], 1), ([(5000, 8, 8), (4500, 8, 9)], 1), ([(3000, 12, 12)], 1), ([(400, 150, 5)], 3),
+    ([(3000, 150, 5)], 1), ([(600, 300, 6)], 2), ([(5000, 8, 8), (70, 66, 68)], 1),
+    ([(300, 8, 8), (70, 66, 68)], 2), ([(4000, 4, 32)], 2), ([(2500, 16, 16)], 2),
+])
+def test_thin_columns_take_the_one_step_sweep_with_the_same_bits(lb, shapes, used):
+    geoms = [_geom(sh, sum(sh)) for sh in shapes]
+    gs = [(0.2, 0.1, -0.3)] * len(geoms)
+    out = []
+    for multi in (0, 2):
+        with _solver(lb, 0, geoms, (0, 0, 0), gs[0], _wave("pgse", 10)) as s:
+            s.set_option(lb.OPT_MULTI_STEP, multi)
+            fields = [torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda") for g in geoms]
+            s.run_batch(lb.Solver.members(gs, list(range(len(geoms))), 0.03), fields=fields)
+            torch.cuda.synchronize()
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == (used if multi == 0 else 2)
+            out.append([v.cpu().numpy() for v in fields])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
 def test_batch_members_end_on_either_step_and_runs_continue_in_any_split(lb):
     geoms = [_geom((24, 20, 33), 5), _geom((9, 41, 16), 6), _geom((48, 16, 16), 7)]
     n = 21
