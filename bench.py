@@ -50,7 +50,7 @@ DELTA, BIG_DELTA = 10.0, 30.0
 D = [1.0, 2.5, 3.0]
 T2 = [50.0, 80.0, 80.0]
 KAPPA = 0.01
-BYTES_PER_SITE = 113  # 7 complex64 read + 7 written + 1 mask byte (algorithmic)
+BYTES_PER_SITE = 113  # 7 complex64 read + 7 written + 1 mask byte (algorithmic), one pass per step
 METRIC = "MLUPS (fused sweep, FP32, 3-direction batch)"
 
 
@@ -106,6 +106,10 @@ def sweep_source_hash():
     return _code_hash(("sweep_tma.cu", "sweep_common.cuh", "tma_common.cuh", "lbmbt_internal.cuh"))
 
 
+def pair_source_hash():
+    return _code_hash(("sweep_pair.cu", "packed.cuh", "sweep_common.cuh", "tma_common.cuh", "lbmbt_internal.cuh"))
+
+
 def links_source_hash():
     return _code_hash(("sweep.cu", "links.cuh", "sweep_common.cuh", "lbmbt_internal.cuh"))
 
@@ -124,17 +128,22 @@ def links_traffic_per_launch(n):
 
 
 def traffic_per_launch(site_updates, form):
-    """DRAM bytes per sweep launch of `site_updates` site-member updates in
-    the own-z form `form` ("z-marching", "staged", "prefetched"), from the
+    """DRAM bytes of `site_updates` site-member updates by the two-step sweep
+    (`form` "two-step") or the bulk-copy sweep in the own-z form `form`
+    ("z-marching", "staged", "prefetched"), from the
     bytes per update in the committed ncu summary, or None when the kernel
     source changed since it was captured or the form was not captured."""
     p = os.path.join(ROOT, "profiles", "sweep_traffic.json")
     if not os.path.exists(p):
         return None
     j = json.load(open(p))
-    if j.get("source_hash") != sweep_source_hash():
+    f = j.get("two_step") if form == "two-step" else j.get("by_form", {}).get(form)
+    if form == "two-step":
+        same = f is not None and f.get("source_hash") == pair_source_hash()
+    else:
+        same = j.get("source_hash") == sweep_source_hash()
+    if not same:
         return None
-    f = j.get("by_form", {}).get(form)
     return None if f is None else float(f["bytes_per_site_member"]) * site_updates
 
 
@@ -307,8 +316,25 @@ def _timed_advance(solver, stream, members, steps, warmup, want_signal=True):
     return e0.elapsed_time(e1) / steps, clk.summary(), sig
 
 
+def _sweep_kind(s, lbmbt):
+    """The sweep of the prepared run: "two-step", "resident" or, one pass a
+    step, "bulk-copy" or "register"."""
+    multi = s.get_option(lbmbt.OPT_MULTI_STEP_USED)
+    if multi > 1:
+        return {2: "two-step", 3: "resident"}[multi]
+    return "bulk-copy" if s.get_option(lbmbt.OPT_KERNEL_USED) == 2 else "register"
+
+
+def _bytes_per_update(kind):
+    """Bytes per site and step that sweep `kind` cannot do without: the
+    two-step sweep reads and writes the state and reads the mask once per two
+    steps.  (A resident run moves only block faces; the one-pass figure stands
+    for it, so its fraction is a comparison, not a bound.)"""
+    return BYTES_PER_SITE / 2 if kind == "two-step" else BYTES_PER_SITE
+
+
 def _launch_shape(s, lbmbt):
-    return {"kernel": "bulk-copy" if s.get_option(lbmbt.OPT_KERNEL_USED) == 2 else "register",
+    return {"kernel": _sweep_kind(s, lbmbt),
             "tma_shape": s.get_option(lbmbt.OPT_TMA_SHAPE), "stages": s.get_option(lbmbt.OPT_STAGES),
             "block": s.get_option(lbmbt.OPT_BLOCK), "spt": s.get_option(lbmbt.OPT_SPT)}
 
@@ -345,7 +371,7 @@ def measure_plain_c2(args, stream):
     return {"value": v, "unit": "MLUPS", "ms_per_step": ms, "steps": PLAIN_C2_STEPS, "warmup": PLAIN_C2_WARMUP,
             "workload": "128^3 permeable cylinders, dx 0.5 um, 1 member (PGSE b 1000 along x)",
             "l2": "state of 235 MB per time level pair, larger than L2; no flush needed",
-            "launch": shape, "roofline": _hbm_roofline(v, BYTES_PER_SITE, "sweep (" + shape["kernel"] + ")"),
+            "launch": shape, "roofline": _hbm_roofline(v, _bytes_per_update(shape["kernel"]), "sweep (" + shape["kernel"] + ")"),
             "clocks": clk}
 
 
@@ -377,7 +403,7 @@ def measure_batch(args, stream):
                         "(edges 48-160, dx 0.5 um, kappa U(0, 0.05) um/ms)",
             "members": len(members), "sites_per_step": total_sites,
             "pack_edges": [int(g.shape[0]) for g in packs], "geometry_gen_s": round(t_gen, 1),
-            "launch": shape, "roofline": _hbm_roofline(v, BYTES_PER_SITE, "sweep (" + shape["kernel"] + ")"),
+            "launch": shape, "roofline": _hbm_roofline(v, _bytes_per_update(shape["kernel"]), "sweep (" + shape["kernel"] + ")"),
             "clocks": clk}
 
 
@@ -638,7 +664,7 @@ def run_variants(args):
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / steps
         return {"MLUPS": n_sites * len(members) / (ms * 1e-3) / 1e6, "ms_per_step": ms,
-                "kernel": "bulk-copy" if s.get_option(lbmbt.OPT_KERNEL_USED) == 2 else "register"}
+                "kernel": _sweep_kind(s, lbmbt)}
 
     # D2Q5 vs D3Q7 on the same one-plane grid (cells of ~10 um in a 1 mm square)
     n2 = 4096
@@ -957,7 +983,7 @@ def main():
         torch.cuda.synchronize()
     clocks_main = clk.summary()
     launches = s.launch_count() - l0
-    shape = {"kernel": "bulk-copy" if s.get_option(lbmbt.OPT_KERNEL_USED) == 2 else "register",
+    shape = {"kernel": _sweep_kind(s, lbmbt),
              "tma_shape": s.get_option(lbmbt.OPT_TMA_SHAPE), "stages": s.get_option(lbmbt.OPT_STAGES),
              "block": s.get_option(lbmbt.OPT_BLOCK), "spt": s.get_option(lbmbt.OPT_SPT),
              "own_z": {0: None, 1: "prefetched", 2: "staged", 3: "z-marching"}[s.get_option(lbmbt.OPT_STAGE_OWN_Z_USED)],
@@ -967,8 +993,9 @@ def main():
     if world > 1:
         dist.barrier()
     value = n_sites * nm * args.steps * world / (ms * 1e-3) / 1e6
-    per_launch_s = ms * 1e-3 / args.steps
-    achieved = BYTES_PER_SITE * n_sites * nm / per_launch_s / 1e9
+    per_step_s = ms * 1e-3 / args.steps
+    bytes_site = _bytes_per_update(shape["kernel"])
+    achieved = bytes_site * n_sites * nm / per_step_s / 1e9
     peak, peak_kind = peaks()
 
     # end to end through the public API: host labels (pinned) -> mask,
@@ -1017,7 +1044,8 @@ def main():
             extras["adjoint_full_schedule"] = measure_adjoint(args, stream, None)
 
     if rank == 0:
-        tr = traffic_per_launch(n_sites * nm, shape["own_z"])
+        form = "two-step" if shape["kernel"] == "two-step" else shape["own_z"]
+        tr = traffic_per_launch(n_sites * nm, form)
         line = {
             "metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
@@ -1034,13 +1062,15 @@ def main():
             "gpu_launches": launches,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": tr, "peak_source": peak_kind,
-                         "traffic_gbs": tr / per_launch_s / 1e9 if tr is not None else None,
-                         "traffic_source": ("ncu DRAM bytes of the " + str(shape["own_z"]) + " form on the tissue's "
+                         "traffic_gbs": tr / per_step_s / 1e9 if tr is not None else None,
+                         "traffic_source": ("ncu DRAM bytes of the " + str(form) + " form on the tissue's "
                                             "first 128 planes, scaled by site updates (profiles/sweep_traffic.json)"
-                                            + ("" if shape["own_z"] == "z-marching" else
+                                            + ("" if form in ("two-step", "z-marching") else
                                                "; bytes per update rise with the planes, so a lower bound for "
                                                "the full grid")) if tr is not None else None,
-                         "bytes_per_site_member": BYTES_PER_SITE, "kernel": "sweep_tma_kernel"},
+                         "bytes_per_site_member": bytes_site,
+                         "kernel": {"two-step": "sweep_pair_kernel", "resident": "sweep_resident_kernel",
+                                    "register": "sweep_kernel"}.get(shape["kernel"], "sweep_tma_kernel")},
             "e2e": e2e,
             "cpu_baseline": cpu,
             "clocks": clocks_main,
