@@ -924,7 +924,7 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
     struct Cut { int cy, cz, recv; };
     auto cut = [&](const MemberDesc& d, int cap) {
         Cut best = {0, 0, 0};
-        for (int cz = 1; cz <= d.nz; ++cz) {
+        for (int cz = 1; cz <= std::min(d.nz, c->sm_count); ++cz) {   // more blocks would not fit
             const int hz = (d.nz + cz - 1) / cz;
             if ((d.nz + hz - 1) / hz != cz) continue;
             const long long rows = cap / ((long long)d.nx * hz);
