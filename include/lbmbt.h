@@ -261,7 +261,8 @@ int lbmbt_run_batch(lbmbt_ctx* ctx, int n_members, const lbmbt_member* members,
  *   n_steps  length of f, 1 .. the set sequence's n_steps (ignored when f is
  *            NULL): the member's signal and field are those at t = n_steps*dt
  *            (its echo); the batch runs to the longest, and a shorter member
- *            keeps stepping with f = 0 after its end, unobserved;
+ *            keeps stepping with f = 0 after its end, unobserved (without a
+ *            series the two-step sweep leaves those steps out);
  *   field_dev device complex64 [N of its geometry] receiving M(x) at the
  *            member's end, or NULL. */
 typedef struct {

@@ -140,6 +140,9 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
     const bool series = s_ctl[5];
     const int es = d->end_step;
     const int sig = es >= 0 ? es : s_ctl[3], fstep = es >= 0 ? es : s_ctl[4];
+    // A member past its own end, no series asked for: nothing of it is read any more (16
+    // members of four edges, echoes at 0.4 to 1 of 160 steps: 20.8 ms against 27.5).
+    if (es >= 0 && k > es && !series) return;
     // bits: M of step 1, 2 into the sums, the field, mout
     const bool fld = d->field != nullptr, out = d->mout != nullptr;
     const unsigned obs = (series || (k == sig && !out) ? 1u : 0u) | (series || (k + 1 == sig && !out) ? 2u : 0u) |
