@@ -553,7 +553,8 @@ __global__ void pair_init_kernel(const MemberDesc* __restrict__ members, int n_m
 // Measured before the masks were asked for two planes ahead (512^3 tissue / 128^3
 // cylinders / 16 odd packs, ms a pass): 222 / 49.7 / 27.7; 512 threads x 1 block 223 /
 // 50.2 / 32.5; 448 x 1 with a third stage 226 / 52.4 / 34.5; 224 x 2 with a third stage
-// 230 / 55.7 / 31.2.  Since: 222 / 49.2 / 27.5.
+// 230 / 55.7 / 31.2.  Since: 224 / 49.3 / 27.5 (20.8 with members past their echo
+// skipped).
 constexpr int PNT = 256, PMB = 2;
 constexpr size_t PAIR_SMEM = (size_t)(PAIR_STAGES * stage_words(PNT) + 2 * 4 * PNT) * sizeof(ulonglong2) + 2 * PNT * sizeof(float4);
 
