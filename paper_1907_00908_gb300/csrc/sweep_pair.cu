@@ -67,6 +67,16 @@ __device__ __forceinline__ void tma_box(void* dst, const CUtensorMap* map, int x
         : "memory");
 }
 
+// The maps lie in global memory and are rewritten by a copy from the host at each
+// set-up, at the same address.  They are read through a proxy of their own, which
+// neither the copy nor the launch orders: the thread that issues boxes acquires
+// each map it uses first.  Issued by thread 0 behind its ticket, the acquires cost 1 us a
+// launch (117 x 90 x 75, 480 steps: 8.5 ms; beside the ticket 8.4; 128^3: 50.2 and 49.6).
+__device__ __forceinline__ void acquire_map(const CUtensorMap* map)
+{
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
+
 // Exact running sum (two-sum) of one component.
 __device__ __forceinline__ void two_sum(float& s, float& c, float v)
 {
@@ -201,7 +211,9 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
     const int ze = STEPS == 2 ? it.z1 : it.z1 - 1;                            // last iteration
     auto wrapz = [&](int z) { return z < 0 ? z + nz : z >= nz ? z - nz : z; };
 
-    // Copies of a plane's inputs (thread 0)
+    // Copies of a plane's inputs, issued by the first thread of the second warp: the
+    // acquire of its maps runs beside the first warp's ticket
+    const bool copier = t == 32;
     const CUtensorMap* map = maps + (2 * it.m + lsrc);
     auto issue = [&](int zi, int st) {
         const int z = wrapz(zi);
@@ -232,9 +244,12 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
         return r;
     };
 
-    if (t == 0)
+    if (copier) {
+        acquire_map(map);
+        acquire_map(map + 2 * a.n_members);
         for (int q = 0; q < PAIR_STAGES - 1; ++q)
             if (zb + q <= zl) issue(zb + q, q);
+    }
     __syncthreads();     // the shared constants are set
     ulonglong2 c5, o6;   // p5 of the plane below, own p6 of this plane
     // Mask bytes of the next plane and of the one after: a plane's are asked for two planes
@@ -339,7 +354,7 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
     for (int zi = zb; zi <= ze; ++zi) {
         if (zi <= zl && !dead) dead = !mbar_wait(&full[st], ph);
         __syncthreads();   // plane zi's inputs and plane zi - 1's step-1 values are visible
-        if (t == 0 && zi + PAIR_STAGES - 1 <= zl) issue(zi + PAIR_STAGES - 1, st == 0 ? PAIR_STAGES - 1 : st - 1);
+        if (copier && zi + PAIR_STAGES - 1 <= zl) issue(zi + PAIR_STAGES - 1, st == 0 ? PAIR_STAGES - 1 : st - 1);
         const unsigned mk = mkn;
         ulonglong2 n0 = zero2, n5 = zero2, n6 = zero2;
         float2 nra = make_float2(0.f, 0.f), nrb = nra;

@@ -147,3 +147,34 @@ def test_batch_members_end_on_either_step_and_runs_continue_in_any_split(lb):
             v = fld.cpu().numpy()
         ref = v if ref is None else ref
         assert np.abs(ref).max() > 0 and np.array_equal(ref, v)
+
+
+# one context, one grid after the other: growing and shrinking, other tiles, batches,
+# on-chip grids in between (the tensor maps are rewritten where they lie)
+TURNS = [[(37, 23, 31)], [(70, 66, 68)], [(90, 75, 117)], [(4, 300, 300), (70, 66, 68), (66, 70, 81)], [(24, 24, 24)],
+         [(75, 90, 117)], [(70, 66, 68), (66, 70, 81)], [(64, 48, 160)], [(70, 66, 68)]]
+
+
+@pytest.mark.parametrize("multi", [0, 2])
+def test_one_context_over_many_grids_gives_what_a_fresh_one_gives(lb, multi):
+    gG = (0.2, 0.1, -0.3)
+
+    def job(s, shapes):
+        geoms = [_geom(sh, sum(sh)) for sh in shapes]
+        for i, g in enumerate(geoms):
+            (s.add_geometry if i else s.set_geometry)(g.labels, g.phase_of_label, g.dx, (0, 0, 0))
+        fields = [torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda") for g in geoms]
+        r = s.run_batch(lb.Solver.members([gG] * len(geoms), list(range(len(geoms))), 0.03), fields=fields)
+        torch.cuda.synchronize()
+        return [v.cpu().numpy() for v in fields], np.asarray(r["Z"])
+
+    with _solver(lb, 0, [_geom((8, 8, 8), 1)], (0, 0, 0), gG, _wave("pgse", 9)) as s:
+        s.set_option(lb.OPT_MULTI_STEP, multi)
+        for shapes in TURNS:
+            got = job(s, shapes)
+            with _solver(lb, 0, [_geom((8, 8, 8), 1)], (0, 0, 0), gG, _wave("pgse", 9)) as fresh:
+                fresh.set_option(lb.OPT_MULTI_STEP, multi)
+                want = job(fresh, shapes)
+            for a, b in zip(got[0], want[0]):
+                assert np.array_equal(a, b), shapes
+            assert np.array_equal(got[1], want[1]), shapes
