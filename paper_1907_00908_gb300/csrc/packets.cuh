@@ -1,7 +1,8 @@
 // packets.cuh -- face values sent between the blocks of one cooperative launch:
-// 16-byte packets {re, stamp, im, stamp} that the receiver polls (see
-// sweep_resident.cu for why no packet is lost or taken twice), and the site flags
-// of the kernels that cut a grid into blocks.
+// 16-byte packets {re, stamp, im, stamp} that the receiver polls (data and flag in one
+// word, as the low-latency protocol of NCCL has them; see sweep_resident.cu for why
+// no packet is lost or taken twice), and the site flags of the kernels that cut a grid
+// into blocks.
 #pragma once
 #include "lbmbt_internal.cuh"
 #include "tma_common.cuh"
@@ -9,9 +10,13 @@
 namespace lbmbt {
 namespace {
 
+// Each half of a packet, a value and its stamp, is one 64-bit element of the access: a
+// vector access is as many accesses as it has elements, in no stated order, so an
+// element is what arrives as a whole.
 __device__ __forceinline__ void send(uint4* to, float2 v, unsigned stamp)
 {
-    asm volatile("st.volatile.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(to), "r"(__float_as_uint(v.x)), "r"(stamp),
+    asm volatile("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
+                 "st.volatile.global.v2.u64 [%0], {a, b};\n\t}" ::"l"(to), "r"(__float_as_uint(v.x)),
                  "r"(__float_as_uint(v.y)), "r"(stamp)
                  : "memory");
 }
@@ -19,7 +24,8 @@ __device__ __forceinline__ void send(uint4* to, float2 v, unsigned stamp)
 __device__ __forceinline__ uint4 peek(const uint4* from)
 {
     uint4 p;
-    asm volatile("ld.volatile.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("{\n\t.reg .b64 a, b;\n\tld.volatile.global.v2.u64 {a, b}, [%4];\n\t"
+                 "mov.b64 {%0, %1}, a;\n\tmov.b64 {%2, %3}, b;\n\t}"
                  : "=r"(p.x), "=r"(p.y), "=r"(p.z), "=r"(p.w)
                  : "l"(from)
                  : "memory");
