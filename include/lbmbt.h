@@ -380,7 +380,9 @@ enum {
                                 control's error word after its producer has
                                 waited (bounded) for its own copies in
                                 flight, and the call returns LBMBT_EDEVICE.
-                                The context stays usable                  */,
+                                The context stays usable.  The two-step
+                                sweep's threads do the same.  Other sweeps
+                                have no such wait                         */,
     LBMBT_OPT_COLUMN_PLANES = 17, /* bulk-copy sweep, z-marching form: planes
                                 per column.  0 (default) auto: the longest
                                 power of two <= 32 that divides every

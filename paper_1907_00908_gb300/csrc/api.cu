@@ -1101,7 +1101,7 @@ constexpr double PAIR_FILL = 0.30;
 
 static bool pair_eligible(const lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
 {
-    if (c->kernel_opt != 0 || c->scheme != 0 || c->lattice != 0 || c->test_wait_ns > 0 || any_slab(c)) return false;
+    if (c->kernel_opt != 0 || c->scheme != 0 || c->lattice != 0 || any_slab(c)) return false;
     bool bulk = true;   // the one-step sweep would be the bulk-copy one
     double sites = 0, room = 0;
     for (auto& d : descs) {

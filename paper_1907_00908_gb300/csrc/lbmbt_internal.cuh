@@ -126,9 +126,10 @@ struct SweepArgs {
                                   // variant with the Eqs. B4a-B4c rule); 2: and angles
     float w0, wxy, wz;            // equilibrium weights (register sweep, init):
                                   // D3Q7 1/4, 1/8, 1/8; D2Q5 1/3, 1/6, 0 (Sec. 2.3)
-    unsigned long long test_wait_ns;  // bulk-copy sweep, tests of the timeout path only: > 0
-                                  // makes each consumer warp first wait, with this limit,
-                                  // on a barrier nothing completes (0: off)
+    unsigned long long test_wait_ns;  // bulk-copy and two-step sweeps, tests of the timeout
+                                  // path only: > 0 makes each consumer warp (each thread)
+                                  // first wait, with this limit, on a barrier nothing
+                                  // completes (0: off)
     int zc;                       // bulk-copy sweep, z-marching form: units per column
                                   // (consecutive z-planes of the same rows; a power of two
                                   // that divides every member's nz), else 0

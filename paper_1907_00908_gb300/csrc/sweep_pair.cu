@@ -114,7 +114,9 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
     __shared__ const uint8_t* s_mask;
     __shared__ unsigned s_sxym;
     __shared__ int s_wrap[2];        // element shift of the ghost copies in x and y, 0 for a mirror
-    __shared__ uint64_t full[PAIR_STAGES];   // the row copies of a stage have arrived
+    __shared__ uint64_t full[PAIR_STAGES];   // the boxes of a stage have arrived
+    __shared__ uint64_t never;               // nothing completes it (tests of the time-out)
+    __shared__ int s_dead;                   // a wait ran out
 
     const int t = threadIdx.x;
     const PairItem it = items[blockIdx.x];
@@ -127,7 +129,9 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
         s_ctl[4] = __ldcg(&a.ctl->field_step);
         s_ctl[5] = __ldcg(&a.ctl->series);
         for (int q = 0; q < PAIR_STAGES; ++q) mbar_init(&full[q], 1);
+        mbar_init(&never, 1);
         fence_mbar_init();
+        s_dead = 0;
     }
     __syncthreads();
     const int k = s_ctl[0];
@@ -244,11 +248,12 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
         return r;
     };
 
+    int issued = 0;   // the copier's: planes asked for
     if (copier) {
         acquire_map(map);
         acquire_map(map + 2 * a.n_members);
         for (int q = 0; q < PAIR_STAGES - 1; ++q)
-            if (zb + q <= zl) issue(zb + q, q);
+            if (zb + q <= zl) { issue(zb + q, q); ++issued; }
     }
     __syncthreads();     // the shared constants are set
     ulonglong2 c5, o6;   // p5 of the plane below, own p6 of this plane
@@ -350,11 +355,18 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
 
     int st = 0;           // stage of plane zi and the parity of its fill
     uint32_t ph = 0;
-    bool dead = false;    // a copy did not arrive within the limit: finish without waiting, report
+    // A copy did not arrive within the limit: the block finishes without waiting and
+    // without asking for more (what it computes is lost), and reports.
+    bool dead = false;
+    if (a.test_wait_ns && !mbar_wait(&never, 0u, a.test_wait_ns)) s_dead = 1;
     for (int zi = zb; zi <= ze; ++zi) {
-        if (zi <= zl && !dead) dead = !mbar_wait(&full[st], ph);
+        if (zi <= zl && !dead && !mbar_wait(&full[st], ph)) s_dead = 1;
         __syncthreads();   // plane zi's inputs and plane zi - 1's step-1 values are visible
-        if (copier && zi + PAIR_STAGES - 1 <= zl) issue(zi + PAIR_STAGES - 1, st == 0 ? PAIR_STAGES - 1 : st - 1);
+        dead = s_dead;     // of all threads
+        if (copier && !dead && zi + PAIR_STAGES - 1 <= zl) {
+            issue(zi + PAIR_STAGES - 1, st == 0 ? PAIR_STAGES - 1 : st - 1);
+            ++issued;
+        }
         const unsigned mk = mkn;
         ulonglong2 n0 = zero2, n5 = zero2, n6 = zero2;
         float2 nra = make_float2(0.f, 0.f), nrb = nra;
@@ -520,7 +532,11 @@ __global__ void __launch_bounds__(NT, MINB) sweep_pair_kernel(const SweepArgs a,
         st = st == PAIR_STAGES - 1 ? 0 : st + 1;
         ph = st == 0 ? ph ^ 1u : ph;
     }
-    if (dead) atomicOr(&a.ctl->err, 1);
+    if (dead && copier) {   // copies in flight end (wait bounded too) before their stages are used again or given back
+        for (int q = max(0, issued - PAIR_STAGES); q < issued; ++q)
+            mbar_wait(&full[q % PAIR_STAGES], (uint32_t)(q / PAIR_STAGES & 1));
+        atomicOr(&a.ctl->err, 1);
+    }
 
     if ((obs & 1u) || (STEPS == 2 && (obs & 2u))) {   // block-uniform
         __syncthreads();

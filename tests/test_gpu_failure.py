@@ -68,3 +68,47 @@ def test_test_wait_option_bounds(lb):
         with pytest.raises(lb.LbmbtError):
             s.set_option(lb.OPT_TEST_WAIT_NS, bad)
     s.close()
+
+
+def _times_out_and_recovers(lb, s, call, geom, bc, D, T2, kap, dt, f, gG):
+    """`call` fails with EDEVICE while the first wait runs out; then the same
+    context runs as the oracle does."""
+    s.set_option(lb.OPT_TEST_WAIT_NS, 1_000_000)           # 1 ms
+    t0 = time.perf_counter()
+    with pytest.raises(lb.LbmbtError) as e:
+        call()
+    assert e.value.code == -6 and "timed out" in str(e.value)
+    assert time.perf_counter() - t0 < 5.0
+    s.set_option(lb.OPT_TEST_WAIT_NS, 0)
+    fld = torch.zeros(geom.n_sites, dtype=torch.complex64, device="cuda")
+    r = s.run(field=fld)
+    torch.cuda.synchronize()
+    o = oracle.run(geom.labels, geom.dx, geom.phase_of_label, bc, D, T2, kap, dt, f, gG, want_field=True)
+    assert abs(r["S"] - o["S"]) <= 1e-5 * o["S"]
+    err = np.abs(fld.cpu().numpy().reshape(geom.labels.shape) - o["field"]).max() / np.abs(o["field"]).max()
+    assert err < 1e-4 and math.isfinite(r["S"])
+
+
+def _setup(lb, shape, n_steps, lattice=0):
+    rng = np.random.default_rng(9)
+    geom = synth.Geometry(rng.integers(0, 2, size=shape).astype(np.int32), np.array([0, 1], np.uint8), 0.5)
+    dt, gG, f, D, T2, kap = 0.02, [0.05, 0.0, 0.0], np.ones(n_steps), [2.0, 1.0], [80.0, 50.0], 0.04
+    s = lb.Solver(0)
+    s.set_option(lb.OPT_LATTICE, lattice)
+    s.set_geometry(geom.labels, geom.phase_of_label, geom.dx)
+    s.set_phases(D, T2)
+    s.set_permeability(kap)
+    s.set_sequence(dt, f, gG)
+    return s, (geom, (0, 0, 0), D, T2, kap, dt, f, gG)
+
+
+# one item and several, two steps and one more, a captured graph, sums in the kernel
+# (series) after the waits ran out
+@pytest.mark.parametrize("shape", [(4, 6, 18), (40, 21, 37)])
+@pytest.mark.parametrize("n_steps,series", [(2, False), (5, False), (20, False), (5, True)])
+def test_two_step_sweep_wait_timeout(lb, shape, n_steps, series):
+    s, job = _setup(lb, shape, n_steps)
+    s.set_option(lb.OPT_MULTI_STEP, 2)
+    _times_out_and_recovers(lb, s, lambda: s.run(series=series), *job)
+    assert s.get_option(lb.OPT_MULTI_STEP_USED) == 2
+    s.close()
