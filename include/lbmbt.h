@@ -381,8 +381,11 @@ enum {
                                 waited (bounded) for its own copies in
                                 flight, and the call returns LBMBT_EDEVICE.
                                 The context stays usable.  The two-step
-                                sweep's threads do the same.  Other sweeps
-                                have no such wait                         */,
+                                sweep's threads do the same; in the resident
+                                sweeps and the resident adjoint the blocks
+                                wait for packets that nobody sends.  A grid
+                                of one block and the register sweep have no
+                                waits                                     */,
     LBMBT_OPT_COLUMN_PLANES = 17, /* bulk-copy sweep, z-marching form: planes
                                 per column.  0 (default) auto: the longest
                                 power of two <= 32 that divides every

@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(NT, 1) adjoint_resident_kernel(const AdjointAr
     };
     auto factors = [&](int k) { return __ldg(a.ftab + ((size_t)k * a.n_members + b.m) * 6 + t); };
 
-    bool dead = false;
-    const uint4* const mine = r.packets + (size_t)blockIdx.x * 4 * r.recv_max;
+    Waits waits = {r.wait_ns, false};
+    const uint4* const mine = r.inbox + (size_t)blockIdx.x * 4 * r.recv_max;
     auto send_faces = [&](unsigned f, unsigned place, int n, u64 v3, u64 v4, u64 v5, u64 v6) {
         const unsigned stamp = r.stamp0 + (unsigned)n;
         const size_t turn = (size_t)(n & 3) * r.recv_max;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(NT, 1) adjoint_resident_kernel(const AdjointAr
             const uint4* box = mine + (size_t)(n & 3) * r.recv_max;
             for (int e = t; e < b.n_recv; e += NT) {
                 uint4 p = peek(box + e);
-                if (!(p.y == stamp && p.w == stamp)) p = await(box + e, stamp, dead);
+                if (!(p.y == stamp && p.w == stamp)) p = await(box + e, stamp, waits);
                 cur[NP * S + e] = pk(__uint_as_float(p.x), __uint_as_float(p.z));
             }
         }
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(NT, 1) adjoint_resident_kernel(const AdjointAr
 #pragma unroll
         for (int i = 1; i <= NP; ++i) nu_out[(size_t)((i & 1) ? i + 1 : i - 1) * P + gs[j]] = end[(i - 1) * S + l];
     }
-    if (dead) atomicOr(a.ctl_err, 1);
+    if (waits.dead) atomicOr(a.ctl_err, 1);
 }
 
 // The gradient partials of n_steps adjoint steps from the sites' sensitivities, as

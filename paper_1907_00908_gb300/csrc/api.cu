@@ -906,7 +906,7 @@ static bool any_slab(const lbmbt_ctx* c);
 static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, bool adjoint = false)
 {
     c->res_ok = false;
-    if (c->kernel_opt != 0 || c->scheme != 0 || c->test_wait_ns > 0 || any_slab(c) || c->n_steps < 2) return LBMBT_OK;
+    if (c->kernel_opt != 0 || c->scheme != 0 || any_slab(c) || c->n_steps < 2) return LBMBT_OK;
     if (!c->sm_count) CU(c, cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
     long long total = 0;
     bool links = false;
@@ -1012,6 +1012,8 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
     return LBMBT_OK;
 }
 
+static size_t resident_packets(const lbmbt_ctx* c) { return 4 * (size_t)std::max(c->res_recv, 1) * c->res_blocks.size(); }
+
 // Device side of the plan.
 static int build_resident(lbmbt_ctx* c)
 {
@@ -1021,7 +1023,8 @@ static int build_resident(lbmbt_ctx* c)
     std::vector<int> start(n + 1, 0);
     for (auto& b : c->res_blocks) start[b.m + 1]++;
     for (int m = 0; m < n; ++m) start[m + 1] += start[m];
-    const size_t pk = sizeof(uint4) * 4 * (size_t)std::max(c->res_recv, 1) * nb;
+    // (tests of the time-out: as much again, which nobody sends to)
+    const size_t pk = sizeof(uint4) * resident_packets(c) * (c->test_wait_ns ? 2 : 1);
     const bool fresh = c->cap_pk < pk;
     int rc = grow(c, &c->d_res_blocks, &c->cap_rb, sizeof(ResBlock) * nb);
     if (!rc) rc = grow(c, &c->d_packets, &c->cap_pk, pk);
@@ -1693,6 +1696,8 @@ static ResArgs resident_args(lbmbt_ctx* c, long long k, long long n)
         c->res_stamp = 1;
     }
     r.stamp0 = c->res_stamp;
+    r.inbox = c->d_packets + (c->test_wait_ns ? resident_packets(c) : 0);
+    r.wait_ns = c->test_wait_ns ? (unsigned long long)c->test_wait_ns : WAIT_NS;
     c->res_stamp += (unsigned)n;
     r.sig_step = r.field_step = -1;
     r.links = c->res_links ? 1 : 0;

@@ -33,6 +33,8 @@ enum BcMode : int {
                       // halo value times the wrap factor exp(+-i phi)
 };
 
+constexpr unsigned long long WAIT_NS = 2000000000ull;  // bound of every wait of a kernel: 2 s
+
 struct MemberDesc {
     float2* state;        // n_slots time levels, each 7 planes
     float2* adj;          // adjoint sweep: 2 levels of 7 planes (or nullptr)
@@ -126,10 +128,10 @@ struct SweepArgs {
                                   // variant with the Eqs. B4a-B4c rule); 2: and angles
     float w0, wxy, wz;            // equilibrium weights (register sweep, init):
                                   // D3Q7 1/4, 1/8, 1/8; D2Q5 1/3, 1/6, 0 (Sec. 2.3)
-    unsigned long long test_wait_ns;  // bulk-copy and two-step sweeps, tests of the timeout
-                                  // path only: > 0 makes each consumer warp (each thread)
-                                  // first wait, with this limit, on a barrier nothing
-                                  // completes (0: off)
+    unsigned long long test_wait_ns;  // tests of the timeout path only: > 0 makes each
+                                  // consumer warp of the bulk-copy sweep and each thread of
+                                  // the two-step sweep first wait, with this limit, on a
+                                  // barrier nothing completes (0: off; resident sweeps: ResArgs)
     int zc;                       // bulk-copy sweep, z-marching form: units per column
                                   // (consecutive z-planes of the same rows; a power of two
                                   // that divides every member's nz), else 0
@@ -219,6 +221,9 @@ struct ResBlock {
 struct ResArgs {
     const ResBlock* blocks;
     uint4* packets;               // [n_blocks][4 turns][recv_max]
+    const uint4* inbox;           // where they are waited for: packets (tests of the time-out:
+                                  // a place that nobody sends to)
+    unsigned long long wait_ns;   // bound of a wait
     int recv_max;
     int k0, n_steps;              // steps k0 .. k0 + n_steps - 1
     int lsrc, ldst;               // time levels read and written

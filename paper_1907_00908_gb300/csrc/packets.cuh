@@ -32,13 +32,20 @@ __device__ __forceinline__ uint4 peek(const uint4* from)
     return p;
 }
 
-// Polls a packet until both halves carry the stamp; `dead` once the limit has passed.
-__device__ __noinline__ uint4 await(const uint4* from, unsigned stamp, bool& dead)
+// A thread's waits: their bound, and whether it has passed (the thread then goes on
+// without waiting).
+struct Waits {
+    unsigned long long limit_ns;
+    bool dead;
+};
+
+// Polls a packet until both halves carry the stamp, or the bound has passed.
+__device__ __noinline__ uint4 await(const uint4* from, unsigned stamp, Waits& w)
 {
     uint4 p = peek(from);
     const unsigned long long t0 = globaltimer();
-    for (unsigned n = 1; !dead && !(p.y == stamp && p.w == stamp); ++n) {
-        if ((n & 63u) == 0 && globaltimer() - t0 > WAIT_NS) dead = true;
+    for (unsigned n = 1; !w.dead && !(p.y == stamp && p.w == stamp); ++n) {
+        if ((n & 63u) == 0 && globaltimer() - t0 > w.limit_ns) w.dead = true;
         p = peek(from);
     }
     return p;

@@ -250,8 +250,8 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
         for (int j = 0; j < SPT; ++j)
             if (fl[j] & S_ON) put_level(0, t + j * RES_NT, gs[j], p0[j], reinterpret_cast<const u64*>(lev));
 
-    bool dead = false;
-    const uint4* const mine = r.packets + (size_t)blockIdx.x * 4 * r.recv_max;
+    Waits waits = {r.wait_ns, false};
+    const uint4* const mine = r.inbox + (size_t)blockIdx.x * 4 * r.recv_max;
     // sends the populations that leave the block at a site on its faces, with the stamp of step n
     auto send_faces = [&](unsigned f, unsigned place, int n, float2 v3, float2 v4, float2 v5, float2 v6) {
         const unsigned stamp = r.stamp0 + (unsigned)n;
@@ -301,10 +301,10 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
             for (int e = t; e < b.n_recv; e += 2 * RES_NT) {
                 const bool two = e + RES_NT < b.n_recv;
                 uint4 p = peek(box + e), q = two ? peek(box + e + RES_NT) : p;
-                if (!(p.y == stamp && p.w == stamp)) p = await(box + e, stamp, dead);
+                if (!(p.y == stamp && p.w == stamp)) p = await(box + e, stamp, waits);
                 cur[NP * S + e] = make_float2(__uint_as_float(p.x), __uint_as_float(p.z));
                 if (two) {
-                    if (!(q.y == stamp && q.w == stamp)) q = await(box + e + RES_NT, stamp, dead);
+                    if (!(q.y == stamp && q.w == stamp)) q = await(box + e + RES_NT, stamp, waits);
                     cur[NP * S + e + RES_NT] = make_float2(__uint_as_float(q.x), __uint_as_float(q.z));
                 }
             }
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
         if (D2)
             for (int i = 5; i < Q; ++i) dst[(size_t)i * P + gs[j]] = make_float2(0.f, 0.f);
     }
-    if (dead) atomicOr(&a.ctl->err, 1);
+    if (waits.dead) atomicOr(&a.ctl->err, 1);
 }
 
 // Parts of Z per member (out[m][parts]) from the magnetisation M of its sites,

@@ -105,14 +105,14 @@ __global__ void __launch_bounds__(NT, 1) sweep_strip_kernel(const SweepArgs a, c
     if (t < 6) s_fac[0][t] = __ldg(a.fac + ((size_t)r.k0 * a.n_members + b.m) * 6 + t);
     if (t == 6) s_f[0] = __ldg(d->fw + r.k0);
 
-    bool dead = false;
-    const uint4* const mine = r.packets + (size_t)blockIdx.x * 4 * r.recv_max;
+    Waits waits = {r.wait_ns, false};
+    const uint4* const mine = r.inbox + (size_t)blockIdx.x * 4 * r.recv_max;
     // own packets: [turn][0: from below, 1: from above][nx]
     auto receive = [&](int n, int face, int x) {
         const uint4* from = mine + (size_t)(n & 3) * r.recv_max + b.recv[face] + x;
         const unsigned stamp = r.stamp0 + (unsigned)n;
         uint4 p = peek(from);
-        if (!(p.y == stamp && p.w == stamp)) p = await(from, stamp, dead);
+        if (!(p.y == stamp && p.w == stamp)) p = await(from, stamp, waits);
         return pk(__uint_as_float(p.x), __uint_as_float(p.z));
     };
     auto post = [&](int n, int face, int x, u64 v) {
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(NT, 1) sweep_strip_kernel(const SweepArgs a, c
             for (int i = 5; i < Q; ++i) dst[(size_t)i * P + s] = 0ull;
         }
     }
-    if (dead) atomicOr(&a.ctl->err, 1);
+    if (waits.dead) atomicOr(&a.ctl->err, 1);
 }
 
 using StripFn = void (*)(const SweepArgs, const ResArgs);

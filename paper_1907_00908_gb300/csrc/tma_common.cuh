@@ -7,8 +7,6 @@
 namespace lbmbt {
 namespace {
 
-constexpr unsigned long long WAIT_NS = 2000000000ull;  // bound of every wait: 2 s
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)

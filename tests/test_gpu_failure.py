@@ -83,7 +83,8 @@ def _times_out_and_recovers(lb, s, call, geom, bc, D, T2, kap, dt, f, gG):
     fld = torch.zeros(geom.n_sites, dtype=torch.complex64, device="cuda")
     r = s.run(field=fld)
     torch.cuda.synchronize()
-    o = oracle.run(geom.labels, geom.dx, geom.phase_of_label, bc, D, T2, kap, dt, f, gG, want_field=True)
+    o = oracle.run(geom.labels, geom.dx, geom.phase_of_label, bc, D, T2, kap, dt, f, gG, want_field=True,
+                   lattice="D2Q5" if s.get_option(lb.OPT_LATTICE) else "D3Q7")
     assert abs(r["S"] - o["S"]) <= 1e-5 * o["S"]
     err = np.abs(fld.cpu().numpy().reshape(geom.labels.shape) - o["field"]).max() / np.abs(o["field"]).max()
     assert err < 1e-4 and math.isfinite(r["S"])
@@ -112,3 +113,27 @@ def test_two_step_sweep_wait_timeout(lb, shape, n_steps, series):
     _times_out_and_recovers(lb, s, lambda: s.run(series=series), *job)
     assert s.get_option(lb.OPT_MULTI_STEP_USED) == 2
     s.close()
+
+
+# blocks in y and z, a few blocks, 2-D blocks and strips
+@pytest.mark.parametrize("shape,lattice", [((24, 31, 40), 0), ((4, 9, 5), 0), ((1, 120, 130), 1), ((1, 600, 900), 1)])
+@pytest.mark.parametrize("n_steps,series", [(2, False), (25, False), (5, True)])
+def test_resident_sweep_wait_timeout(lb, shape, lattice, n_steps, series):
+    s, job = _setup(lb, shape, n_steps, lattice)
+    _times_out_and_recovers(lb, s, lambda: s.run(series=series), *job)
+    assert s.get_option(lb.OPT_MULTI_STEP_USED) == 3
+    s.close()
+
+
+def test_resident_gradient_wait_timeout(lb):
+    s, job = _setup(lb, (20, 24, 32), 11)
+    geom, gG, kap = job[0], job[7], job[4]
+    m = lb.Solver.members([gG], 0, kap)
+    _times_out_and_recovers(lb, s, lambda: s.grad_batch(m, checkpoint_every=4), *job)
+    after = s.grad_batch(m, checkpoint_every=4)
+    s.close()
+    s, _ = _setup(lb, (20, 24, 32), 11)
+    fresh = s.grad_batch(m, checkpoint_every=4)
+    s.close()
+    for key in ("S", "dD", "dT2", "dkappa"):
+        np.testing.assert_array_equal(after[key], fresh[key])
