@@ -405,8 +405,16 @@ enum {
                                 are no thin columns, else one.  1
                                 one; 2 two where it can run; 3 resident where
                                 the grids fit.  The fields are the same bits */
-    LBMBT_OPT_MULTI_STEP_USED = 19 /* read-only: 1, 2 or 3 for the prepared
+    LBMBT_OPT_MULTI_STEP_USED = 19, /* read-only: 1, 2 or 3 for the prepared
                                 run, else 0                                  */
+    LBMBT_OPT_TEST_FAIL_ALLOC = 20, /* tests of scarce memory only: n > 0 makes
+                                the n-th allocation of a device buffer from
+                                now fail as if there were no room (once;
+                                LBMBT_ENOMEM where the call cannot do without);
+                                reads as those still to come; 0 (default) off */
+    LBMBT_OPT_TEST_STAMP = 21  /* tests of used-up stamps only: the stamp of the
+                                resident sweep's next packets (it can only be
+                                raised, to 2^32 - 1 at most)                 */
 };
 int lbmbt_set_option(lbmbt_ctx* ctx, int option, int64_t value);
 int lbmbt_get_option(lbmbt_ctx* ctx, int option, int64_t* value);

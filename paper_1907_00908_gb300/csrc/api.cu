@@ -155,7 +155,8 @@ struct lbmbt_ctx {
     size_t cap_ftab = 0;
     bool ftab_valid = false;      // d_ftab holds the prepared members' factors
     int grad_groups = 0;          // member groups of the last lbmbt_grad_batch
-    long long test_wait_ns = 0;   // tests of the bulk-copy sweep's timeout path (0: off)
+    long long test_wait_ns = 0;   // tests of the sweeps' timeout paths (0: off)
+    long long fail_alloc = 0;     // tests: this many allocations from now, one fails (0: off)
     float2* d_etab = nullptr;     // per-member rotation tables
     size_t cap_etab = 0;
     float2* d_halo = nullptr;     // slab halo planes, [member][2][nx*ny]
@@ -249,6 +250,8 @@ static int grow(lbmbt_ctx* c, T** p, size_t* cap, size_t bytes)
     if (*cap >= bytes && *p) return LBMBT_OK;
     if (*p) { cudaFree(*p); *p = nullptr; *cap = 0; }
     if (bytes == 0) return LBMBT_OK;
+    if (c->fail_alloc > 0 && --c->fail_alloc == 0)
+        return fail(c, LBMBT_ENOMEM, "allocation of %zu bytes failed (LBMBT_OPT_TEST_FAIL_ALLOC)", bytes);
     CU(c, cudaMalloc((void**)p, bytes));
     *cap = bytes;
     return LBMBT_OK;
@@ -1014,6 +1017,15 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
 
 static size_t resident_packets(const lbmbt_ctx* c) { return 4 * (size_t)std::max(c->res_recv, 1) * c->res_blocks.size(); }
 
+static int clear_packets(lbmbt_ctx* c)
+{
+    c->res_stamp = 1;
+    const cudaError_t e = cudaMemsetAsync(c->d_packets, 0, c->cap_pk, c->stream);
+    if (e != cudaSuccess) c->cap_pk = 0;   // not cleared: not to be used
+    CU(c, e);
+    return LBMBT_OK;
+}
+
 // Device side of the plan.
 static int build_resident(lbmbt_ctx* c)
 {
@@ -1025,15 +1037,14 @@ static int build_resident(lbmbt_ctx* c)
     for (int m = 0; m < n; ++m) start[m + 1] += start[m];
     // (tests of the time-out: as much again, which nobody sends to)
     const size_t pk = sizeof(uint4) * resident_packets(c) * (c->test_wait_ns ? 2 : 1);
-    const bool fresh = c->cap_pk < pk;
-    int rc = grow(c, &c->d_res_blocks, &c->cap_rb, sizeof(ResBlock) * nb);
-    if (!rc) rc = grow(c, &c->d_packets, &c->cap_pk, pk);
+    int rc = LBMBT_OK;
+    if (c->cap_pk < pk) {   // no packet there carries a stamp to come, whatever fails after this
+        rc = grow(c, &c->d_packets, &c->cap_pk, pk);
+        if (!rc) rc = clear_packets(c);
+    }
+    if (!rc) rc = grow(c, &c->d_res_blocks, &c->cap_rb, sizeof(ResBlock) * nb);
     if (!rc) rc = grow(c, &c->d_res_start, &c->cap_rs, sizeof(int) * start.size());
     if (rc) return rc;
-    if (fresh) {   // no packet there carries a stamp to come
-        CU(c, cudaMemsetAsync(c->d_packets, 0, c->cap_pk, c->stream));
-        c->res_stamp = 1;
-    }
     CU(c, cudaMemcpyAsync(c->d_res_blocks, c->res_blocks.data(), sizeof(ResBlock) * nb, cudaMemcpyHostToDevice, c->stream));
     CU(c, cudaMemcpyAsync(c->d_res_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, c->stream));
     c->res_max_links = 0;
@@ -1682,9 +1693,8 @@ constexpr long long RES_CHUNK = 1 << 15, RES_SERIES_CHUNK = 1 << 12;
 
 // Arguments of a launch of n steps from step k on (the levels and what is observed
 // are the caller's); takes n stamps.
-static ResArgs resident_args(lbmbt_ctx* c, long long k, long long n)
+static int resident_args(lbmbt_ctx* c, long long k, long long n, ResArgs& r)
 {
-    ResArgs r;
     memset(&r, 0, sizeof r);
     r.blocks = c->d_res_blocks;
     r.packets = c->d_packets;
@@ -1692,8 +1702,8 @@ static ResArgs resident_args(lbmbt_ctx* c, long long k, long long n)
     r.k0 = (int)k;
     r.n_steps = (int)n;
     if (c->res_stamp > 0xffffffffu - (unsigned)n) {   // stamps used up: start over on clean buffers
-        cudaMemsetAsync(c->d_packets, 0, c->cap_pk, c->stream);
-        c->res_stamp = 1;
+        const int rc = clear_packets(c);
+        if (rc) return rc;
     }
     r.stamp0 = c->res_stamp;
     r.inbox = c->d_packets + (c->test_wait_ns ? resident_packets(c) : 0);
@@ -1702,7 +1712,7 @@ static ResArgs resident_args(lbmbt_ctx* c, long long k, long long n)
     r.sig_step = r.field_step = -1;
     r.links = c->res_links ? 1 : 0;
     r.max_links = c->res_max_links;
-    return r;
+    return LBMBT_OK;
 }
 
 static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_step)
@@ -1715,7 +1725,9 @@ static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_ste
         if (rc) return rc;
     }
     for (long long k = c->k_cur, end = c->k_cur + n; k < end;) {
-        ResArgs r = resident_args(c, k, std::min(chunk, end - k));
+        ResArgs r;
+        const int rc = resident_args(c, k, std::min(chunk, end - k), r);
+        if (rc) return rc;
         r.lsrc = (int)((k - c->slot_base) & 1);
         r.ldst = (int)((k + r.n_steps - c->slot_base) & 1);
         r.sig_step = sig_step;
@@ -2062,6 +2074,14 @@ extern "C" int lbmbt_set_option(lbmbt_ctx* c, int opt, int64_t v)
         if (v < 0 || v > 3) return fail(c, LBMBT_EINVAL, "steps of a pass must be 0 (auto), 1, 2 or 3 (resident)");
         c->multi_opt = (int)v;
         break;
+    case LBMBT_OPT_TEST_FAIL_ALLOC:
+        if (v < 0) return fail(c, LBMBT_EINVAL, "allocations until one fails must be >= 0");
+        c->fail_alloc = v;
+        return LBMBT_OK;
+    case LBMBT_OPT_TEST_STAMP:
+        if (v < (long long)c->res_stamp || v > 0xffffffffLL) return fail(c, LBMBT_EINVAL, "stamps only rise, to 2^32 - 1");
+        c->res_stamp = (unsigned)v;
+        return LBMBT_OK;
     default: return fail(c, LBMBT_EINVAL, "unknown option %d", opt);
     }
     invalidate_run(c);
@@ -2086,6 +2106,8 @@ extern "C" int lbmbt_get_option(lbmbt_ctx* c, int opt, int64_t* v)
     case LBMBT_OPT_SCHEME: *v = c->scheme; break;
     case LBMBT_OPT_GRAD_GROUPS: *v = c->grad_groups; break;
     case LBMBT_OPT_TEST_WAIT_NS: *v = c->test_wait_ns; break;
+    case LBMBT_OPT_TEST_FAIL_ALLOC: *v = c->fail_alloc; break;
+    case LBMBT_OPT_TEST_STAMP: *v = c->res_stamp; break;
     case LBMBT_OPT_COLUMN_PLANES: *v = c->zc_opt; break;
     case LBMBT_OPT_MULTI_STEP: *v = c->multi_opt; break;
     case LBMBT_OPT_MULTI_STEP_USED: *v = !c->prepared ? 0 : c->res_ok ? 3 : c->pair_ok ? 2 : 1; break;
@@ -2196,7 +2218,9 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
     // resident: steps k0 .. k0 + ns - 1 from a level of the checkpoints; levels: they go to
     // the segment buffer from slot `slot` on
     auto forward = [&](long long k0, long long ns, bool levels, long long slot) -> int {
-        ResArgs r = resident_args(c, k0, ns);
+        ResArgs r;
+        const int rc = resident_args(c, k0, ns, r);
+        if (rc) return rc;
         r.lsrc = (int)(k0 / ck);
         r.ldst = std::min(r.lsrc + 1, (int)n_ck - 1);   // the next checkpoint (the last one's: a level not needed)
         r.sig_step = (int)(K - 1);
@@ -2324,7 +2348,8 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
                 if ((rc = forward(k0, ck, true, 0))) return rc;
                 CU(c, cudaMemcpyAsync(c->d_desc, rd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
             }
-            ResArgs r = resident_args(c, k0, k1 - k0);
+            ResArgs r;
+            if ((rc = resident_args(c, k0, k1 - k0, r))) return rc;
             r.lsrc = r.ldst = 0;
             aa.k = (int)k1;
             aa.first = (k1 == K) ? 1 : 0;

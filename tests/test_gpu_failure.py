@@ -137,3 +137,95 @@ def test_resident_gradient_wait_timeout(lb):
     s.close()
     for key in ("S", "dD", "dT2", "dkappa"):
         np.testing.assert_array_equal(after[key], fresh[key])
+
+
+# every allocation of a first call fails in turn: the call does without or says
+# ENOMEM, and the next call on the context gives what a fresh context gives
+@pytest.mark.parametrize("kind", ["resident", "strip", "links", "two-step", "bulk-copy"])
+def test_each_allocation_may_fail(lb, kind):
+    shape, lattice = {"resident": ((9, 31, 20), 0), "strip": ((1, 300, 1300), 1), "links": ((12, 10, 9), 0),
+                      "two-step": ((40, 21, 37), 0), "gradient": ((20, 24, 32), 0), "bulk-copy": ((20, 24, 32), 0)}[kind]
+    rng = np.random.default_rng(5)
+    delta = rng.uniform(0.1, 0.9, size=(6, *shape)).astype(np.float32)
+
+    def one(fail_at):
+        s, job = _setup(lb, shape, 4, lattice)
+        geom, kap, f, gG = job[0], job[4], job[6], job[7]
+        s.set_option(lb.OPT_MULTI_STEP, {"two-step": 2, "bulk-copy": 1}.get(kind, 0))
+        if kind == "links":
+            s.set_link_distances(delta)
+        m = lb.Solver.members([gG, (0.0, 0.1, 0.0)], 0, kap)
+        fields = [torch.zeros(geom.n_sites, dtype=torch.complex64, device="cuda") for _ in range(2)]
+
+        def call():
+            if kind == "gradient":
+                r = s.grad_batch(m, checkpoint_every=1)
+                return [r["dD"], r["dT2"], r["dkappa"]], np.asarray(r["Z"])
+            r = s.run_batch(m, waveforms=[f * 0.5, None], fields=fields)
+            torch.cuda.synchronize()
+            return [v.cpu().numpy() for v in fields], np.asarray(r["Z"])
+
+        first = None
+        s.set_option(lb.OPT_TEST_FAIL_ALLOC, fail_at)
+        try:
+            first = call()
+        except lb.LbmbtError as e:
+            assert e.code == -2
+        left = s.get_option(lb.OPT_TEST_FAIL_ALLOC)
+        s.set_option(lb.OPT_TEST_FAIL_ALLOC, 0)
+        again = call()
+        s.close()
+        return first, again, left
+
+    want, _, _ = one(0)
+    tol = 2.0 ** -22 * np.prod(shape)   # where memory is short the signal may be summed in other groups
+    for n in range(1, 60):
+        first, again, left = one(n)
+        for got in (first, again):
+            if got is None:
+                continue
+            for a, b in zip(got[0], want[0]):
+                np.testing.assert_allclose(a, b, rtol=1e-6 if kind == "gradient" else 0, atol=0)
+            assert np.abs(got[1] - want[1]).max() <= tol
+        if left:
+            break
+    assert left and n > 8      # the last one came after the last allocation
+
+
+def test_resident_stamps_start_over_when_used_up(lb):
+    s, job = _setup(lb, (24, 31, 40), 25)
+    geom = job[0]
+    out = []
+    for stamp in (None, 2 ** 32 - 1, 2 ** 32 - 30, None):
+        if stamp:
+            s.set_option(lb.OPT_TEST_STAMP, stamp)
+        fld = torch.zeros(geom.n_sites, dtype=torch.complex64, device="cuda")
+        s.run(field=fld)
+        torch.cuda.synchronize()
+        out.append(fld.cpu().numpy())
+        assert s.get_option(lb.OPT_TEST_STAMP) == {0: 26, 1: 26, 2: 2 ** 32 - 5, 3: 26}[len(out) - 1]
+    s.close()
+    for v in out[1:]:
+        np.testing.assert_array_equal(out[0], v)
+
+
+# a launch takes 32768 steps at most, 4096 with a series
+@pytest.mark.parametrize("n_steps,series", [(32768 + 3, False), (2 * 4096 + 1, True)])
+def test_resident_run_of_several_launches(lb, n_steps, series):
+    out = []
+    for multi in (0, 1):
+        s, job = _setup(lb, (6, 9, 10), n_steps)
+        geom = job[0]
+        s.set_sequence(0.02, 1e-3 * np.cos(np.arange(n_steps) * 0.01), [0.05, 0.0, 0.0])
+        s.set_phases([2.0, 1.0], [2e4, 2e4])
+        s.set_option(lb.OPT_MULTI_STEP, multi)
+        fld = torch.zeros(geom.n_sites, dtype=torch.complex64, device="cuda")
+        r = s.run(field=fld, series=series)
+        torch.cuda.synchronize()
+        assert s.get_option(lb.OPT_MULTI_STEP_USED) == (1 if multi else 3)
+        s.close()
+        out.append((fld.cpu().numpy(), r))
+    np.testing.assert_array_equal(out[0][0], out[1][0])
+    assert np.abs(out[0][0]).max() > 0.1
+    if series:
+        assert np.abs(out[0][1]["series"] - out[1][1]["series"]).max() <= 2.0 ** -22 * geom.n_sites
