@@ -2149,7 +2149,8 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
     size_t lvl_total = 0;
     for (auto& d : c->descs) lvl_total += (size_t)7 * d.plane;
     rc = grow(c, &c->d_ck, &c->cap_ck, lvl_total * n_ck * sizeof(float2));
-    if (!rc) rc = grow(c, &c->d_seg, &c->cap_seg, lvl_total * ((size_t)keep * ck + 1) * sizeof(float2));
+    if (rc) return rc;
+    rc = grow(c, &c->d_seg, &c->cap_seg, lvl_total * ((size_t)keep * ck + 1) * sizeof(float2));
     if (rc == LBMBT_ENOMEM && keep > 1) {   // no room after all: the last segment only
         cudaGetLastError();
         c->err.clear();

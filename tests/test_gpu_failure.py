@@ -141,7 +141,7 @@ def test_resident_gradient_wait_timeout(lb):
 
 # every allocation of a first call fails in turn: the call does without or says
 # ENOMEM, and the next call on the context gives what a fresh context gives
-@pytest.mark.parametrize("kind", ["resident", "strip", "links", "two-step", "bulk-copy"])
+@pytest.mark.parametrize("kind", ["resident", "strip", "links", "two-step", "gradient", "bulk-copy"])
 def test_each_allocation_may_fail(lb, kind):
     shape, lattice = {"resident": ((9, 31, 20), 0), "strip": ((1, 300, 1300), 1), "links": ((12, 10, 9), 0),
                       "two-step": ((40, 21, 37), 0), "gradient": ((20, 24, 32), 0), "bulk-copy": ((20, 24, 32), 0)}[kind]
