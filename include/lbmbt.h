@@ -292,7 +292,10 @@ int lbmbt_run_batch_ex(lbmbt_ctx* ctx, int n_members, const lbmbt_member_ex* mem
  * checkpointed every `checkpoint_every` steps (<= 0: 64) and recomputed
  * segment by segment; where device memory has room (a quarter of what is free
  * at most, and no more than the checkpoints and one segment take) the levels of
- * the last segments are kept instead of being recomputed.  signal_out[3] as in lbmbt_run; dS_dD[n_phases],
+ * the last segments are kept instead of being recomputed.  On small grids
+ * whose sensitivities wait for their sum (the resident adjoint) they take up to
+ * 0.5 GB besides.  These buffers stay with the context for its next call, until
+ * lbmbt_destroy.  signal_out[3] as in lbmbt_run; dS_dD[n_phases],
  * dS_dT2[n_phases] (host; T2 = INFINITY gives 0), dS_dkappa[1] (host).
  */
 int lbmbt_grad(lbmbt_ctx* ctx, int checkpoint_every, double* signal_out,

@@ -2132,6 +2132,11 @@ static size_t grad_bytes_per_member(const lbmbt_ctx* c, long long plane, int ck)
     return (size_t)(2 + n_ck + ck + 1) * 7 * plane * sizeof(float2);
 }
 
+// Steps of a launch of the resident adjoint: the sensitivities of their sites wait in
+// memory for their sum, 12 B a site and step, 0.48 GB at most (a resident adjoint has
+// 152 x 1024 sites at most), whatever the segment's length.
+constexpr long long ADJ_RES_STEPS = 256;
+
 // One group of members: checkpointed forward pass, then segments in reverse:
 // recompute the segment's forward levels from its checkpoint, then run the
 // adjoint sweep back through it.  The last `keep` segments are not recomputed:
@@ -2174,7 +2179,7 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
         res = c->res_ok;
         c->res_ok = false;   // no prepared run stands on it
     }
-    const int L_max = (int)std::min<long long>(ck, K);
+    const int L_max = (int)std::min<long long>({ck, K, ADJ_RES_STEPS});
     size_t sites = 0;
     if (res) {
         for (auto& d : c->descs) sites += (size_t)d.N;
@@ -2349,17 +2354,21 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
                 if ((rc = forward(k0, ck, true, 0))) return rc;
                 CU(c, cudaMemcpyAsync(c->d_desc, rd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
             }
-            ResArgs r;
-            if ((rc = resident_args(c, k0, k1 - k0, r))) return rc;
-            r.lsrc = r.ldst = 0;
-            aa.k = (int)k1;
-            aa.first = (k1 == K) ? 1 : 0;
-            aa.fwd_slot = (int)(k1 - 1 - base);
-            CU(c, launch_adjoint_resident(aa, r, (int)c->res_blocks.size(), c->res_sites,
-                                          adj_resident_smem(c->res_sites, c->res_recv), c->general, c->stream));
-            CU(c, launch_adjoint_sum(aa, c->n_adj_units, (int)(k1 - k0), adj_grid, adj_tma_consumers(c->adj_shape_used),
-                                     c->adj_shape_used == 0 ? 2 : 1, adj_tma_slots_per_unit(), c->stream));
-            c->launches += 2;
+            for (long long k = k1; k > k0;) {
+                const int steps = (int)std::min<long long>(L_max, k - k0);
+                ResArgs r;
+                if ((rc = resident_args(c, k - steps, steps, r))) return rc;
+                r.lsrc = r.ldst = 0;
+                aa.k = (int)k;
+                aa.first = (k == K) ? 1 : 0;
+                aa.fwd_slot = (int)(k - 1 - base);
+                CU(c, launch_adjoint_resident(aa, r, (int)c->res_blocks.size(), c->res_sites,
+                                              adj_resident_smem(c->res_sites, c->res_recv), c->general, c->stream));
+                CU(c, launch_adjoint_sum(aa, c->n_adj_units, steps, adj_grid, adj_tma_consumers(c->adj_shape_used),
+                                         c->adj_shape_used == 0 ? 2 : 1, adj_tma_slots_per_unit(), c->stream));
+                c->launches += 2;
+                k -= steps;
+            }
             continue;
         }
         if (!kept) {
@@ -2440,7 +2449,7 @@ extern "C" int lbmbt_grad_batch(lbmbt_ctx* c, int n_members, const lbmbt_member*
     // group members so one group's levels fit in the free device memory
     size_t free_b = 0, total_b = 0;
     CU(c, cudaMemGetInfo(&free_b, &total_b));
-    const size_t held = c->cap_state + c->cap_ck + c->cap_seg;
+    const size_t held = c->cap_state + c->cap_ck + c->cap_seg + c->cap_mo + c->cap_gs;
     const size_t budget = (size_t)((double)(free_b + held) * 0.8);
     int m0 = 0;
     c->grad_groups = 0;

@@ -179,3 +179,25 @@ def test_resident_gradient_is_the_bulk_copy_one(lb, shapes, bc, gG, wave, n, eve
     for k in ("dD", "dT2", "dkappa"):
         a, b = out[0][0][k], out[1][0][k]
         assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max(), (k, a, b)
+
+
+# segments longer than a launch of the resident adjoint (256 steps): the same numbers,
+# and no more memory than the levels and the sensitivities of 256 steps
+@pytest.mark.parametrize("n,every", [(600, 600), (513, 300), (256, 256)])
+def test_resident_gradient_of_long_segments(lb, n, every):
+    g = _geom((31, 32, 48), 4)
+    f = 0.02 * _wave("cos", n)
+    out = []
+    for multi in (0, 1):
+        with _solver(lb, multi, [g], (0, 0, 0), (0.3, 0.2, 0.1), f, 0.05, 0) as s:
+            torch.cuda.synchronize()
+            before = torch.cuda.mem_get_info()[0]
+            out.append(s.grad(checkpoint_every=every))
+            held = before - torch.cuda.mem_get_info()[0]
+            n_ck = -(-n // every)
+            levels = 2 + n_ck + n_ck * every + 1   # state, checkpoints, segments (all kept at most)
+            assert held <= g.n_sites * (56 * levels + 12 * 256 + 8) + (64 << 20)
+    assert np.allclose(out[0]["Z"], out[1]["Z"], rtol=1e-12, atol=0)
+    for k in ("dD", "dT2", "dkappa"):
+        a, b = np.asarray(out[0][k]), np.asarray(out[1][k])
+        assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max(), (k, a, b)
