@@ -110,6 +110,7 @@ struct lbmbt_ctx {
     // two-step sweep (auto kernel choice): work items, per-member item prefix
     bool pair_ok = false;
     int multi_opt = 0;            // steps of a pass: 0 auto, 1 one, 2 two, 3 resident
+    bool multi_planned = false;   // the set-up took the run to a multi-step sweep
     bool general = false;         // the run has a waveform value other than 0, +-1
     // resident sweep (auto kernel choice, small grids)
     bool res_ok = false;
@@ -255,6 +256,14 @@ static int grow(lbmbt_ctx* c, T** p, size_t* cap, size_t bytes)
     CU(c, cudaMalloc((void**)p, bytes));
     *cap = bytes;
     return LBMBT_OK;
+}
+
+template <class T>
+static void give_back(T** p, size_t* cap)
+{
+    cudaFree(*p);
+    *p = nullptr;
+    *cap = 0;
 }
 
 static void drop_graph(lbmbt_ctx* c)
@@ -1015,6 +1024,10 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
     return LBMBT_OK;
 }
 
+// A launch of the resident sweep takes at most RES_CHUNK steps (in series mode fewer:
+// the parts of Z of every step wait in memory for their sum).
+constexpr long long RES_CHUNK = 1 << 15, RES_SERIES_CHUNK = 1 << 12;
+
 static size_t resident_packets(const lbmbt_ctx* c) { return 4 * (size_t)std::max(c->res_recv, 1) * c->res_blocks.size(); }
 
 static int clear_packets(lbmbt_ctx* c)
@@ -1044,6 +1057,8 @@ static int build_resident(lbmbt_ctx* c)
     }
     if (!rc) rc = grow(c, &c->d_res_blocks, &c->cap_rb, sizeof(ResBlock) * nb);
     if (!rc) rc = grow(c, &c->d_res_start, &c->cap_rs, sizeof(int) * start.size());
+    if (!rc && c->series_mode)
+        rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * nb * std::min(c->n_steps, RES_SERIES_CHUNK));
     if (rc) return rc;
     CU(c, cudaMemcpyAsync(c->d_res_blocks, c->res_blocks.data(), sizeof(ResBlock) * nb, cudaMemcpyHostToDevice, c->stream));
     CU(c, cudaMemcpyAsync(c->d_res_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, c->stream));
@@ -1391,9 +1406,10 @@ static int autotune(lbmbt_ctx* c)
 
 // ex (optional, [n_members]): each member's own waveform (f, n_steps; f NULL
 // for the run's) and field output.
-static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool series, void* field_dev,
-                   const lbmbt_member_ex* ex = nullptr, bool whole_run = true, bool to_end = true)
+static int prepare_as(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool series, void* field_dev,
+                      const lbmbt_member_ex* ex, bool whole_run, bool to_end)
 {
+    c->multi_planned = false;
     if (c->geoms.empty()) return fail(c, LBMBT_ESTATE, "no geometry set");
     if (c->n_phases == 0) return fail(c, LBMBT_ESTATE, "phases not set");
     if (c->n_steps == 0) return fail(c, LBMBT_ESTATE, "sequence not set");
@@ -1517,6 +1533,7 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
         if (rc) return rc;
     }
     c->pair_ok = whole_run && (c->multi_opt == 0 || c->multi_opt == 2) && !c->res_ok && pair_eligible(c, descs);
+    c->multi_planned = c->res_ok || c->pair_ok;
     c->n_members = n_members;
     c->members.assign(mem, mem + n_members);
     c->descs = descs;
@@ -1676,6 +1693,34 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
     return LBMBT_OK;
 }
 
+// The set-up of a run.  Where memory is short, what a gradient left with the context is
+// given back first, then what the multi-step sweeps need besides the state: the one-step
+// sweeps run wherever they did by themselves.
+static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool series, void* field_dev,
+                   const lbmbt_member_ex* ex = nullptr, bool whole_run = true, bool to_end = true)
+{
+    int rc = prepare_as(c, n_members, mem, series, field_dev, ex, whole_run, to_end);
+    if (rc == LBMBT_ENOMEM && whole_run && c->cap_ck + c->cap_seg + c->cap_gs > 0) {
+        cudaGetLastError();
+        give_back(&c->d_ck, &c->cap_ck);
+        give_back(&c->d_seg, &c->cap_seg);
+        give_back(&c->d_gsite, &c->cap_gs);
+        rc = prepare_as(c, n_members, mem, series, field_dev, ex, whole_run, to_end);
+    }
+    if (rc == LBMBT_ENOMEM && c->multi_planned) {
+        cudaGetLastError();
+        give_back(&c->d_state, &c->cap_state);   // with ghosts
+        give_back(&c->d_mout, &c->cap_mo);
+        give_back(&c->d_packets, &c->cap_pk);
+        give_back(&c->d_zpart, &c->cap_zp);
+        give_back(&c->d_pair_items, &c->cap_pi);
+        give_back(&c->d_pair_maps, &c->cap_pm);
+        rc = prepare_as(c, n_members, mem, series, field_dev, ex, false, to_end);
+    }
+    if (!rc) c->err.clear();
+    return rc;
+}
+
 // Z of every member from its mout, with the one-step sweep's thread sums.
 static int sum_signal(lbmbt_ctx* c)
 {
@@ -1686,10 +1731,6 @@ static int sum_signal(lbmbt_ctx* c)
     c->launches += 2;
     return LBMBT_OK;
 }
-
-// n steps by the resident sweep.  A launch takes at most RES_CHUNK steps (in
-// series mode fewer: the parts of Z of every step wait in memory for their sum).
-constexpr long long RES_CHUNK = 1 << 15, RES_SERIES_CHUNK = 1 << 12;
 
 // Arguments of a launch of n steps from step k on (the levels and what is observed
 // are the caller's); takes n stamps.
@@ -1715,15 +1756,12 @@ static int resident_args(lbmbt_ctx* c, long long k, long long n, ResArgs& r)
     return LBMBT_OK;
 }
 
+// n steps by the resident sweep.
 static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_step)
 {
     const SweepArgs a = sweep_args(c);
     const int nb = (int)c->res_blocks.size();
     const long long chunk = c->series_mode ? RES_SERIES_CHUNK : RES_CHUNK;
-    if (c->series_mode) {
-        int rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * nb * std::min(n, chunk));
-        if (rc) return rc;
-    }
     for (long long k = c->k_cur, end = c->k_cur + n; k < end;) {
         ResArgs r;
         const int rc = resident_args(c, k, std::min(chunk, end - k), r);
@@ -2175,7 +2213,14 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
     // small grids: resident forward and adjoint (blocks as the adjoint can hold them)
     bool res = false;
     if (adj_tma && c->adjoint_opt == 0 && (c->multi_opt == 0 || c->multi_opt == 3)) {
-        if ((rc = plan_resident(c, c->descs, true)) || (rc = build_resident(c))) return rc;
+        rc = plan_resident(c, c->descs, true);
+        if (!rc) rc = build_resident(c);
+        if (rc == LBMBT_ENOMEM) {   // no room for its blocks and packets: one step a launch
+            cudaGetLastError();
+            c->err.clear();
+            rc = LBMBT_OK;
+        }
+        if (rc) return rc;
         res = c->res_ok;
         c->res_ok = false;   // no prepared run stands on it
     }
@@ -2183,20 +2228,23 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
     size_t sites = 0;
     if (res) {
         for (auto& d : c->descs) sites += (size_t)d.N;
+        c->sig_parts = 16;
+        const size_t part = c->cap_partial;
         rc = grow(c, &c->d_mout, &c->cap_mo, sizeof(float2) * sites);
         if (!rc) rc = grow(c, &c->d_gsite, &c->cap_gs, sizeof(float) * 3 * sites * L_max);
-        if (rc == LBMBT_ENOMEM) {   // no room: one step a launch
+        if (!rc) rc = grow(c, &c->d_idx, &c->cap_ix, sizeof(long long) * (n + 1));
+        if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n * c->sig_parts);
+        if (rc == LBMBT_ENOMEM) {   // no room: one step a launch, with its partials
             cudaGetLastError();
             c->err.clear();
             res = false;
-            rc = LBMBT_OK;
+            rc = grow(c, &c->d_partial, &c->cap_partial, part);
         }
-        c->sig_parts = 16;
+        if (rc) return rc;
+    }
+    if (res) {
         std::vector<long long> idx(n + 1);
         std::iota(idx.begin(), idx.end(), 0LL);
-        if (!rc) rc = grow(c, &c->d_idx, &c->cap_ix, sizeof(long long) * idx.size());
-        if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n * c->sig_parts);
-        if (rc) return rc;
         CU(c, cudaMemcpyAsync(c->d_idx, idx.data(), sizeof(long long) * idx.size(), cudaMemcpyHostToDevice, c->stream));
         if ((rc = sync(c))) return rc;
     }

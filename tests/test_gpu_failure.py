@@ -139,57 +139,87 @@ def test_resident_gradient_wait_timeout(lb):
         np.testing.assert_array_equal(after[key], fresh[key])
 
 
+KINDS = {"resident": ((9, 31, 20), 0, 0), "strip": ((1, 300, 1300), 1, 0), "links": ((12, 10, 9), 0, 0),
+         "resident series": ((9, 31, 20), 0, 0),
+         "two-step": ((40, 21, 37), 0, 2), "gradient": ((20, 24, 32), 0, 0), "bulk-copy": ((20, 24, 32), 0, 1),
+         "bulk-copy gradient": ((20, 24, 32), 0, 1)}
+
+
+def _with_one_failure(lb, kind, fail_at):
+    """(first call, second call, allocations to come): the first one's `fail_at`-th allocation
+    fails; None where it said ENOMEM."""
+    shape, lattice, multi = KINDS[kind]
+    s, job = _setup(lb, shape, 4, lattice)
+    geom, kap, f, gG = job[0], job[4], job[6], job[7]
+    s.set_option(lb.OPT_MULTI_STEP, multi)
+    if kind == "links":
+        s.set_link_distances(np.random.default_rng(5).uniform(0.1, 0.9, size=(6, *shape)).astype(np.float32))
+    m = lb.Solver.members([gG, (0.0, 0.1, 0.0)], 0, kap)
+    fields = [torch.zeros(geom.n_sites, dtype=torch.complex64, device="cuda") for _ in range(2)]
+
+    def call():
+        if "gradient" in kind:
+            r = s.grad_batch(m, checkpoint_every=1)
+            return [r["dD"], r["dT2"], r["dkappa"]], np.asarray(r["Z"])
+        r = s.run_batch(m, waveforms=[f * 0.5, None], fields=fields, series="series" in kind)
+        torch.cuda.synchronize()
+        return [v.cpu().numpy() for v in fields], np.asarray(r["Z"])
+
+    first = None
+    s.set_option(lb.OPT_TEST_FAIL_ALLOC, fail_at)
+    try:
+        first = call()
+    except lb.LbmbtError as e:
+        assert e.code == -2
+    left = s.get_option(lb.OPT_TEST_FAIL_ALLOC)
+    s.set_option(lb.OPT_TEST_FAIL_ALLOC, 0)
+    again = call()
+    s.close()
+    return first, again, left
+
+
 # every allocation of a first call fails in turn: the call does without or says
 # ENOMEM, and the next call on the context gives what a fresh context gives
-@pytest.mark.parametrize("kind", ["resident", "strip", "links", "two-step", "gradient", "bulk-copy"])
+@pytest.mark.parametrize("kind", list(KINDS))
 def test_each_allocation_may_fail(lb, kind):
-    shape, lattice = {"resident": ((9, 31, 20), 0), "strip": ((1, 300, 1300), 1), "links": ((12, 10, 9), 0),
-                      "two-step": ((40, 21, 37), 0), "gradient": ((20, 24, 32), 0), "bulk-copy": ((20, 24, 32), 0)}[kind]
-    rng = np.random.default_rng(5)
-    delta = rng.uniform(0.1, 0.9, size=(6, *shape)).astype(np.float32)
-
-    def one(fail_at):
-        s, job = _setup(lb, shape, 4, lattice)
-        geom, kap, f, gG = job[0], job[4], job[6], job[7]
-        s.set_option(lb.OPT_MULTI_STEP, {"two-step": 2, "bulk-copy": 1}.get(kind, 0))
-        if kind == "links":
-            s.set_link_distances(delta)
-        m = lb.Solver.members([gG, (0.0, 0.1, 0.0)], 0, kap)
-        fields = [torch.zeros(geom.n_sites, dtype=torch.complex64, device="cuda") for _ in range(2)]
-
-        def call():
-            if kind == "gradient":
-                r = s.grad_batch(m, checkpoint_every=1)
-                return [r["dD"], r["dT2"], r["dkappa"]], np.asarray(r["Z"])
-            r = s.run_batch(m, waveforms=[f * 0.5, None], fields=fields)
-            torch.cuda.synchronize()
-            return [v.cpu().numpy() for v in fields], np.asarray(r["Z"])
-
-        first = None
-        s.set_option(lb.OPT_TEST_FAIL_ALLOC, fail_at)
-        try:
-            first = call()
-        except lb.LbmbtError as e:
-            assert e.code == -2
-        left = s.get_option(lb.OPT_TEST_FAIL_ALLOC)
-        s.set_option(lb.OPT_TEST_FAIL_ALLOC, 0)
-        again = call()
-        s.close()
-        return first, again, left
-
-    want, _, _ = one(0)
-    tol = 2.0 ** -22 * np.prod(shape)   # where memory is short the signal may be summed in other groups
+    want, _, _ = _with_one_failure(lb, kind, 0)
+    tol = 2.0 ** -22 * np.prod(KINDS[kind][0])   # where memory is short the signal may be summed in other groups
     for n in range(1, 60):
-        first, again, left = one(n)
+        first, again, left = _with_one_failure(lb, kind, n)
         for got in (first, again):
             if got is None:
                 continue
             for a, b in zip(got[0], want[0]):
-                np.testing.assert_allclose(a, b, rtol=1e-6 if kind == "gradient" else 0, atol=0)
+                np.testing.assert_allclose(a, b, rtol=1e-6 if "gradient" in kind else 0, atol=0)
             assert np.abs(got[1] - want[1]).max() <= tol
         if left:
             break
     assert left and n > 8      # the last one came after the last allocation
+
+
+# what a multi-step sweep needs besides is no reason to refuse a call that the one-step
+# sweeps can do
+@pytest.mark.parametrize("kind", ["resident", "strip", "links", "two-step", "resident series"])
+def test_a_multi_step_run_falls_back_where_memory_is_short(lb, kind):
+    n = 1
+    while True:
+        first, _, left = _with_one_failure(lb, kind, n)
+        assert first is not None, n
+        if left:
+            return
+        n += 1
+
+
+def test_a_resident_gradient_falls_back_where_memory_is_short(lb):
+    refused = []
+    for kind in ("gradient", "bulk-copy gradient"):
+        n, left, k = 1, 0, 0
+        while not left:
+            first, _, left = _with_one_failure(lb, kind, n)
+            k += first is None
+            n += 1
+        refused.append(k)
+    assert refused[0] == refused[1]
 
 
 def test_resident_stamps_start_over_when_used_up(lb):
