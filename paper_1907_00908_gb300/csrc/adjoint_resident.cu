@@ -399,7 +399,7 @@ cudaError_t launch_adjoint_resident(const AdjointArgs& a, const ResArgs& r, int 
     const Fn k = max_sites <= NT ? (general ? adjoint_resident_kernel<1, true> : adjoint_resident_kernel<1, false>)
                                  : (general ? adjoint_resident_kernel<2, true> : adjoint_resident_kernel<2, false>);
     const void* fn = (const void*)k;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     AdjointArgs aa = a;
     ResArgs rr = r;

@@ -410,7 +410,7 @@ static int adj_threads(int shape) { return shape == 1 ? 544 : shape == 2 ? 512 :
 cudaError_t adj_tma_prepare(int cap, int nst, int shape, int* ctas_per_sm)
 {
     const size_t bytes = adj_stage_bytes(cap) * nst;
-    cudaError_t e = cudaFuncSetAttribute(adj_kernel(shape), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(adj_kernel(shape), bytes);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, adj_kernel(shape), adj_threads(shape), bytes);
 }

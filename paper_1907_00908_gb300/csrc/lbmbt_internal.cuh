@@ -9,9 +9,24 @@
 // (stride 7*plane): 2 for the ping-pong of a run, c+1 for an adjoint segment.
 #pragma once
 #include <cstdint>
+#include <mutex>
+
 #include <cuda_runtime.h>
 
 namespace lbmbt {
+
+// Lets launches of `fn` have `bytes` of dynamic shared memory.  The limit belongs to the
+// kernel, not to a context: it is only ever raised, so that no context takes away what
+// another one, prepared before or on another thread, launches with.
+inline cudaError_t allow_smem(const void* fn, size_t bytes)
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> hold(mu);
+    cudaFuncAttributes at;
+    const cudaError_t e = cudaFuncGetAttributes(&at, fn);
+    if (e != cudaSuccess || at.maxDynamicSharedSizeBytes >= (int)bytes) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 
 constexpr int Q = 7;
 // D3Q7 weights with eps_D = 1/4 (Sec. 2.3 pattern: w0 = eps_D, wi = eps_D/2).

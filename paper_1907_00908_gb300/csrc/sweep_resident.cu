@@ -537,7 +537,7 @@ cudaError_t launch_resident(const SweepArgs& a, const ResArgs& r, int n_blocks, 
 {
     const int spt = (max_sites + RES_NT - 1) / RES_NT;
     const void* fn = (const void*)(d2 ? res_kernel<true>(spt, general, r.links) : res_kernel<false>(spt, general, r.links));
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     SweepArgs aa = a;
     ResArgs rr = r;

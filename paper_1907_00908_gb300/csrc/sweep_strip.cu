@@ -294,7 +294,7 @@ cudaError_t launch_strip(const SweepArgs& a, const ResArgs& r, int n_blocks, int
     const StripFn k = max_nx <= 2 * NT ? (general ? sweep_strip_kernel<2, 8, true> : sweep_strip_kernel<2, 8, false>)
                                        : (general ? sweep_strip_kernel<3, 6, true> : sweep_strip_kernel<3, 6, false>);
     const void* fn = (const void*)k;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(fn, smem);
     if (e != cudaSuccess) return e;
     SweepArgs aa = a;
     ResArgs rr = r;

@@ -562,7 +562,7 @@ cudaError_t tma_prepare(int cap, int capx, int nst, int variant, int form, int* 
 {
     const size_t bytes = tma_smem_bytes(cap, capx, nst, form);
     void* fn = tma_kernel(variant, form);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e = allow_smem(fn, bytes);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, fn, tma_threads(variant), bytes);
 }

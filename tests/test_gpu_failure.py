@@ -10,6 +10,7 @@ so the producer never waits for a stage to be released.  The next run on the
 same context, with the option off, matches the oracle.
 """
 import math
+import threading
 import time
 
 import numpy as np
@@ -139,6 +140,27 @@ def test_resident_gradient_wait_timeout(lb):
         np.testing.assert_array_equal(after[key], fresh[key])
 
 
+# the shared memory that a kernel may have is the kernel's, not the context's
+@pytest.mark.parametrize("kernel", [2, 0])
+def test_a_context_runs_on_after_another_one_with_smaller_blocks_was_prepared(lb, kernel):
+    s, job = _setup(lb, (24, 40, 64), 6)
+    s.set_option(lb.OPT_KERNEL, kernel)
+    s.prepare()
+    s.advance(2)
+    other, _ = _setup(lb, (2, 2, 16), 6)
+    other.set_option(lb.OPT_KERNEL, kernel)
+    other.prepare()
+    other.advance(2)
+    s.advance(4)
+    z = s.run()["Z"]
+    other.close()
+    s.close()
+    s, job = _setup(lb, (24, 40, 64), 6)
+    s.set_option(lb.OPT_KERNEL, kernel)
+    assert s.run()["Z"] == z
+    s.close()
+
+
 KINDS = {"resident": ((9, 31, 20), 0, 0), "strip": ((1, 300, 1300), 1, 0), "links": ((12, 10, 9), 0, 0),
          "resident series": ((9, 31, 20), 0, 0),
          "two-step": ((40, 21, 37), 0, 2), "gradient": ((20, 24, 32), 0, 0), "bulk-copy": ((20, 24, 32), 0, 1),
@@ -259,3 +281,25 @@ def test_resident_run_of_several_launches(lb, n_steps, series):
     assert np.abs(out[0][0]).max() > 0.1
     if series:
         assert np.abs(out[0][1]["series"] - out[1][1]["series"]).max() <= 2.0 ** -22 * geom.n_sites
+
+
+def test_contexts_on_threads_with_blocks_of_different_size(lb):
+    shapes = [(20, 24, 32), (40, 48, 48), (7, 5, 16), (60, 57, 57)]
+    fail = []
+
+    def work(i):
+        try:
+            s, job = _setup(lb, shapes[i], 4)
+            z = {s.run()["Z"] for _ in range(60)} | {s.grad(checkpoint_every=2)["Z"] for _ in range(10)}
+            s.close()
+            if len({complex(round(v.real, 6), round(v.imag, 6)) for v in z}) != 1:
+                fail.append((i, z))
+        except lb.LbmbtError as e:
+            fail.append((i, e))
+
+    th = [threading.Thread(target=work, args=(i,)) for i in range(len(shapes))]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert not fail, fail
