@@ -109,6 +109,8 @@ struct lbmbt_ctx {
     std::map<std::string, Tuned> tune_cache;
     // two-step sweep (auto kernel choice): work items, per-member item prefix
     bool pair_ok = false;
+    bool pair_state = false;      // the state has its layout (else the one-step sweeps')
+    int other_advances = 0;       // calls in a row whose sweep would want the other layout
     int multi_opt = 0;            // steps of a pass: 0 auto, 1 one, 2 two, 3 resident
     bool multi_planned = false;   // the set-up took the run to a multi-step sweep
     bool general = false;         // the run has a waveform value other than 0, +-1
@@ -1259,13 +1261,18 @@ static int write_ctl(lbmbt_ctx* c, int sig_step, int field_step, int slot_base =
     return LBMBT_OK;
 }
 
+static long long max_plane(const lbmbt_ctx* c)
+{
+    long long mp = 0;
+    for (auto& d : c->descs) mp = std::max(mp, d.plane);
+    return mp;
+}
+
 static int init_state(lbmbt_ctx* c)
 {
     SweepArgs a = sweep_args(c);
     if (c->pair_ok) {
-        long long mp = 0;
-        for (auto& d : c->descs) mp = std::max(mp, d.plane);
-        CU(c, launch_pair_init(c->d_desc, c->n_members, mp, c->stream));
+        CU(c, launch_pair_init(c->d_desc, c->n_members, max_plane(c), c->stream));
     } else {
         CU(c, launch_init(a, c->n_tiles, c->tile_block, c->tile_spt, 0, c->stream));
     }
@@ -1816,6 +1823,34 @@ static bool any_slab(const lbmbt_ctx* c)
     return false;
 }
 
+// Whether n steps of a prepared run take the two-step sweep, and the state's layout for
+// it.  A step by itself is faster by the one-step sweeps (us a step, two-step sweep's
+// one-step form / one-step: 128^3 78 / 69, 256^3 402 / 331), so a run that is advanced
+// step by step keeps, or changes to, their layout.  A change costs about a step: on
+// the second such call in a row, or at once for a call of many steps.  M = 1, where
+// every run starts, is the same in both.
+constexpr long long RELAYOUT_STEPS = 8;
+
+static int pair_for(lbmbt_ctx* c, long long n, bool* pair)
+{
+    *pair = false;
+    if (!c->pair_ok) return LBMBT_OK;
+    const bool want = n >= 2;
+    if (c->k_cur == 0) c->pair_state = want;
+    if (c->pair_state == want) {
+        c->other_advances = 0;
+    } else if (n >= RELAYOUT_STEPS || c->other_advances++ > 0) {
+        CU(c, launch_pair_relayout(c->d_desc, c->n_members, max_plane(c), (int)((c->k_cur - c->slot_base) & 1), want,
+                                   c->stream));
+        c->launches++;
+        c->slot_base++;   // the level of step k is the other one now
+        c->pair_state = want;
+        c->other_advances = 0;
+    }
+    *pair = c->pair_state;
+    return LBMBT_OK;
+}
+
 // Advance n steps; the signal (and field) of the last step is produced when asked.
 static int advance(lbmbt_ctx* c, long long n, bool want_signal)
 {
@@ -1827,10 +1862,12 @@ static int advance(lbmbt_ctx* c, long long n, bool want_signal)
     if (n > 1 && any_slab(c))
         return fail(c, LBMBT_EINVAL, "a slab advances one step at a time, with a halo exchange between steps");
     const long long last = c->k_cur + n - 1;
-    int rc = write_ctl(c, want_signal ? (int)last : -1, (c->field_dev && last == c->n_steps - 1) ? (int)last : -1,
+    bool pair = false;
+    int rc = pair_for(c, n, &pair);
+    if (rc) return rc;
+    rc = write_ctl(c, want_signal ? (int)last : -1, (c->field_dev && last == c->n_steps - 1) ? (int)last : -1,
                        (int)c->slot_base);
     if (rc) return rc;
-    const bool pair = c->pair_ok;   // its state has a layout of its own
     long long left = n;
     const bool res = c->res_ok && n >= 2;
     if (res) {

@@ -222,6 +222,9 @@ cudaError_t pair_prepare(bool general, int* ctas_per_sm);
 cudaError_t launch_sweep_pair(const SweepArgs& a, const PairItem* items, const PairMap* maps, int n_items, bool general,
                               int steps, cudaStream_t st);
 cudaError_t launch_pair_init(const MemberDesc* members, int n_members, long long max_plane, cudaStream_t st);
+// Level src of every member to level src ^ 1, from rows of nx to the layout with ghosts or back.
+cudaError_t launch_pair_relayout(const MemberDesc* members, int n_members, long long max_plane, int src, bool to_pair,
+                                 cudaStream_t st);
 
 // ---- resident sweep (sweep_resident.cu) -----------------------------------
 // One block of a small grid: all of x, rows [y0, y0 + hy), planes [z0, z0 + hz)

@@ -579,6 +579,34 @@ __global__ void pair_init_kernel(const MemberDesc* __restrict__ members, int n_m
     }
 }
 
+// Copies level `src` of every member to the other one, from the one-step sweeps' layout to
+// this one with its ghosts (to_pair) or back.
+__global__ void pair_relayout_kernel(const MemberDesc* __restrict__ members, int n_members, int src, int to_pair)
+{
+    constexpr int G = PAIR_GHOST;
+    for (int m = blockIdx.y; m < n_members; m += gridDim.y) {
+        const MemberDesc& d = members[m];
+        const int nx = d.nx, ny = d.ny, rows = ny + 2 * G;
+        const long long n = to_pair ? (long long)d.pitch * rows * d.nz : d.N;
+        const float2* from = d.state + (size_t)src * 7 * d.plane;
+        float2* to = d.state + (size_t)(src ^ 1) * 7 * d.plane;
+        for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+            long long o;
+            if (to_pair) {   // ghosts are the wrapped sites; beyond a mirror face and nx + 4: any
+                const long long row = e / d.pitch, z = row / rows;
+                int x = (int)(e - row * d.pitch) - G, y = (int)(row - z * rows) - G;
+                x = x < 0 ? x + nx : x >= nx ? x - nx : x;
+                y = y < 0 ? y + ny : y >= ny ? y - ny : y;
+                o = (z * ny + y) * nx + x;
+            } else {
+                const long long row = e / nx, z = row / ny;
+                o = (z * rows + (row - z * ny) + G) * d.pitch + (e - row * nx) + G;
+            }
+            for (int i = 0; i < Q; ++i) to[(size_t)i * d.plane + e] = from[(size_t)i * d.plane + o];
+        }
+    }
+}
+
 // 256 threads x 2 columns, two blocks per SM (128 registers, 101 KB of shared
 // memory each): one block's barrier and item start are hidden by the other.
 // Measured before the masks were asked for two planes ahead (512^3 tissue / 128^3
@@ -647,6 +675,15 @@ cudaError_t launch_sweep_pair(const SweepArgs& a, const PairItem* items, const P
 {
     pair_kernel(general, steps)<<<(unsigned)n_items, PNT, PAIR_SMEM, st>>>(a, items, reinterpret_cast<const CUtensorMap*>(maps),
                                                                          n_items);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pair_relayout(const MemberDesc* members, int n_members, long long max_plane, int src, bool to_pair,
+                                 cudaStream_t st)
+{
+    const long long bx = std::min<long long>((max_plane + 255) / 256, 152 * 16);
+    pair_relayout_kernel<<<dim3((unsigned)bx, (unsigned)std::min(n_members, 65535)), 256, 0, st>>>(members, n_members, src,
+                                                                                                to_pair ? 1 : 0);
     return cudaGetLastError();
 }
 

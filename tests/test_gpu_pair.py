@@ -178,3 +178,31 @@ def test_one_context_over_many_grids_gives_what_a_fresh_one_gives(lb, multi):
             for a, b in zip(got[0], want[0]):
                 assert np.array_equal(a, b), shapes
             assert np.array_equal(got[1], want[1]), shapes
+
+
+# steps by themselves take the one-step sweep: the state changes its layout there and back
+@pytest.mark.parametrize("shape,bc,gG", [((37, 23, 31), (0, 0, 0), (0.2, 0.1, -0.3)), ((20, 34, 32), (1, 0, 0), (0.4, 0.0, 0.0)),
+                                         ((8, 4, 4), (0, 1, 1), (0.3, 0.0, 0.0)), ((33, 40, 35), (1, 1, 0), (0.0, 0.0, 0.3))])
+def test_runs_advanced_step_by_step_give_the_same_bits(lb, shape, bc, gG):
+    geoms, n = [_geom(shape, 3), _geom((9, 10, 11), 4)], 30
+    m = lb.Solver.members([gG, gG, (0.0, 0.0, 0.0)], [0, 1, 0], [0.03, INF, 0.1])
+    ref = None
+    for kernel, split in ((1, [30]), (0, [30]), (0, [1] * 30), (0, [10] + [1] * 7 + [8, 1, 1, 1, 2]),
+                          (0, [1, 1, 2, 2, 2, 1, 3, 1, 1, 1, 15]), (0, [2, 1, 9, 1, 1, 16]), (0, [1, 29]), (0, [29, 1])):
+        assert sum(split) == n
+        with _solver(lb, kernel, geoms, bc, gG, _wave("cos", n)) as s:
+            s.prepare(m)
+            z = [s.advance(k, True, 3) for k in split][-1][:, :2]
+            with _solver(lb, kernel, geoms[:1], bc, gG, _wave("cos", n)) as one:
+                fld = torch.zeros(geoms[0].n_sites, dtype=torch.complex64, device="cuda")
+                one.set_field(fld)
+                one.prepare()
+                zs = [one.advance(k, True) for k in split][-1][0, :2]
+                torch.cuda.synchronize()
+                v = fld.cpu().numpy()
+        if ref is None:
+            ref = (z, v)
+        assert np.array_equal(ref[1], v) and np.abs(v).max() > 0, split
+        tol = 2.0 ** -22 * geoms[0].n_sites
+        assert np.abs(z - ref[0]).max() <= tol, split
+        assert np.abs(zs - ref[0][0]).max() <= tol, split
