@@ -131,12 +131,13 @@ struct lbmbt_ctx {
     size_t cap_mo = 0;
     bool has_mout = false;        // the members have mout: the signal is summed from it
     int sig_parts = 0;            // parts of a member's signal
-    long long* d_idx = nullptr;   // 0 .. n_members
-    size_t cap_ix = 0;
-    int* d_res_start = nullptr;   // [n + 1] blocks of a member
+    std::vector<int> res_start;
+    int* d_res_start = nullptr;   // [n + 1] blocks of a member (series)
     size_t cap_rs = 0;
     double2* d_zpart = nullptr;
     size_t cap_zp = 0;
+    int pair_per_sm[2] = {0, 0};  // resident blocks of its two forms
+    std::vector<PairMap> pair_maps;
     PairMap* d_pair_maps = nullptr;
     size_t cap_pm = 0;
     std::vector<PairItem> pair_items;
@@ -327,7 +328,7 @@ extern "C" int lbmbt_destroy(lbmbt_ctx* c)
     cudaFree(c->d_ftab); cudaFree(c->d_unit_start); cudaFree(c->d_etab); cudaFree(c->d_cc_start);
     cudaFree(c->d_adj_unit_start); cudaFree(c->d_halo); cudaFree(c->d_pair_items); cudaFree(c->d_pair_start);
     cudaFree(c->d_pair_maps);
-    cudaFree(c->d_res_blocks); cudaFree(c->d_packets); cudaFree(c->d_mout); cudaFree(c->d_idx);
+    cudaFree(c->d_res_blocks); cudaFree(c->d_packets); cudaFree(c->d_mout);
     cudaFree(c->d_res_start); cudaFree(c->d_zpart); cudaFree(c->d_gsite);
     cudaFree(c->d_ck); cudaFree(c->d_seg); cudaFree(c->d_gacc); cudaFree(c->d_gout); cudaFree(c->d_laminit);
     if (c->owned_stream) cudaStreamDestroy(c->owned_stream);
@@ -929,6 +930,13 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
         links = links || d.dlt;
         total += d.N;
     }
+    // A run of few steps does not pay for the plan, a context's first one for its buffers
+    // (us a call by itself, one step a launch / resident, first call and later ones: 16^3, 4
+    // steps 189 / 169, 123 / 113; 48^3, 4 steps 284 / 354, 145 / 132, 8 steps 323 / 351, 188 /
+    // 146, 16 steps 443 / 394; 64^3, 8 steps 348 / 432, 223 / 181, 16 steps 512 / 468;
+    // 200 x 200, 8 steps 302 / 331, 177 / 114; 1000 x 1000, 8 steps 554 / 499).
+    const long long few = c->lattice == 1 ? std::min(7LL, 4 + total / 13000) : std::min(9LL, 4 + total / 52000);
+    if (c->multi_opt == 0 && !adjoint && c->n_steps < few) return LBMBT_OK;
     const int width = links ? 3 : 1, least = links ? 2 : 1;   // values a face site, layers of a block
     if ((int)descs.size() > c->sm_count) return LBMBT_OK;
     int limit = 0;
@@ -1047,9 +1055,6 @@ static int build_resident(lbmbt_ctx* c)
     if (!c->res_ok) return LBMBT_OK;
     c->res_ok = false;   // until it stands
     const int n = c->n_members, nb = (int)c->res_blocks.size();
-    std::vector<int> start(n + 1, 0);
-    for (auto& b : c->res_blocks) start[b.m + 1]++;
-    for (int m = 0; m < n; ++m) start[m + 1] += start[m];
     // (tests of the time-out: as much again, which nobody sends to)
     const size_t pk = sizeof(uint4) * resident_packets(c) * (c->test_wait_ns ? 2 : 1);
     int rc = LBMBT_OK;
@@ -1058,12 +1063,18 @@ static int build_resident(lbmbt_ctx* c)
         if (!rc) rc = clear_packets(c);
     }
     if (!rc) rc = grow(c, &c->d_res_blocks, &c->cap_rb, sizeof(ResBlock) * nb);
-    if (!rc) rc = grow(c, &c->d_res_start, &c->cap_rs, sizeof(int) * start.size());
-    if (!rc && c->series_mode)
-        rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * nb * std::min(c->n_steps, RES_SERIES_CHUNK));
+    if (!rc && c->series_mode) {
+        rc = grow(c, &c->d_res_start, &c->cap_rs, sizeof(int) * (n + 1));
+        if (!rc) rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * nb * std::min(c->n_steps, RES_SERIES_CHUNK));
+    }
     if (rc) return rc;
     CU(c, cudaMemcpyAsync(c->d_res_blocks, c->res_blocks.data(), sizeof(ResBlock) * nb, cudaMemcpyHostToDevice, c->stream));
-    CU(c, cudaMemcpyAsync(c->d_res_start, start.data(), sizeof(int) * start.size(), cudaMemcpyHostToDevice, c->stream));
+    if (c->series_mode) {
+        c->res_start.assign(n + 1, 0);
+        for (auto& b : c->res_blocks) c->res_start[b.m + 1]++;
+        for (int m = 0; m < n; ++m) c->res_start[m + 1] += c->res_start[m];
+        CU(c, cudaMemcpyAsync(c->d_res_start, c->res_start.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, c->stream));
+    }
     c->res_max_links = 0;
     if (c->res_links) {   // the lists lie in shared memory too
         int n_links = 0;
@@ -1078,8 +1089,7 @@ static int build_resident(lbmbt_ctx* c)
         CU(c, cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
         if (c->res_smem + 2048 > (size_t)limit || n_links > 0xffff) return LBMBT_OK;   // one step a launch
     }
-    CU(c, cudaStreamSynchronize(c->stream));   // the host buffers are given back
-    c->res_ok = true;
+    c->res_ok = true;   // (the host's lists are the context's: they outlast the copies)
     return LBMBT_OK;
 }
 
@@ -1130,6 +1140,12 @@ static PairTiles pair_tiles(int nx, int ny, int nt)
 // two-step sweep does.
 constexpr double PAIR_FILL = 0.30;
 
+// A run of few steps pays for the plan only on large grids (us a call, one-step / two-step,
+// first call of a context and later ones: 70 x 66 x 68, 8 steps 373 / 437, 244 / 228, 16 steps
+// 568 / 559, 431 / 369; 128^3, 4 steps 482 / 478, 337 / 341, 8 steps 691 / 672, 541 / 477;
+// 256^3, 2 steps 1408 / 1241, 1027 / 822).
+constexpr double PAIR_SITE_STEPS = 16e6;
+
 static bool pair_eligible(const lbmbt_ctx* c, const std::vector<MemberDesc>& descs)
 {
     if (c->kernel_opt != 0 || c->scheme != 0 || c->lattice != 0 || any_slab(c)) return false;
@@ -1147,6 +1163,7 @@ static bool pair_eligible(const lbmbt_ctx* c, const std::vector<MemberDesc>& des
         room += 2.0 * pair_threads() * t.tx * t.ty * d.nz * pair_narrow(t.w);
     }
     if (c->multi_opt == 0 && !bulk && sites < PAIR_FILL * room) return false;
+    if (c->multi_opt == 0 && c->n_steps < 10 && c->n_steps * sites < PAIR_SITE_STEPS) return false;
     return c->n_steps >= 2;
 }
 
@@ -1158,8 +1175,8 @@ static int build_pair(lbmbt_ctx* c)
     if (!c->pair_ok) return LBMBT_OK;
     c->pair_ok = false;   // until the plan stands
     if (!c->sm_count) CU(c, cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
-    int per_sm = 0;
-    CU(c, pair_prepare(c->general, &per_sm));
+    int& per_sm = c->pair_per_sm[c->general ? 1 : 0];
+    if (!per_sm) CU(c, pair_prepare(c->general, &per_sm));
     if (per_sm < 1) return fail(c, LBMBT_EINVAL, "two-step sweep does not fit on an SM");
     const long long slots = (long long)c->sm_count * per_sm;
     const int nt = pair_threads();
@@ -1221,12 +1238,13 @@ static int build_pair(lbmbt_ctx* c)
     }
     const size_t n = c->pair_items.size();
     if (n > 0x3fffffff) return fail(c, LBMBT_EINVAL, "work list too long");
+    const bool sums = c->series_mode || !c->has_mout;   // the sweep sums M itself
+    std::vector<PairMap>& maps = c->pair_maps;
+    maps.resize(4 * (size_t)c->n_members);
     int rc = grow(c, &c->d_pair_items, &c->cap_pi, sizeof(PairItem) * n);
-    if (!rc) rc = grow(c, &c->d_pair_start, &c->cap_ps, sizeof(long long) * (c->n_members + 1));
-    if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * 2 * n);
-    if (rc) return rc;
-    std::vector<PairMap> maps(4 * (size_t)c->n_members);
-    rc = grow(c, &c->d_pair_maps, &c->cap_pm, sizeof(PairMap) * maps.size());
+    if (!rc && sums) rc = grow(c, &c->d_pair_start, &c->cap_ps, sizeof(long long) * (c->n_members + 1));
+    if (!rc && sums) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * 2 * n);
+    if (!rc) rc = grow(c, &c->d_pair_maps, &c->cap_pm, sizeof(PairMap) * maps.size());
     if (rc) return rc;
     for (int m = 0; m < c->n_members; ++m) {
         const MemberDesc& d = c->descs[m];
@@ -1237,9 +1255,10 @@ static int build_pair(lbmbt_ctx* c)
     }
     CU(c, cudaMemcpyAsync(c->d_pair_maps, maps.data(), sizeof(PairMap) * maps.size(), cudaMemcpyHostToDevice, c->stream));
     CU(c, cudaMemcpyAsync(c->d_pair_items, c->pair_items.data(), sizeof(PairItem) * n, cudaMemcpyHostToDevice, c->stream));
-    CU(c, cudaMemcpyAsync(c->d_pair_start, c->pair_start.data(), sizeof(long long) * (c->n_members + 1),
-                          cudaMemcpyHostToDevice, c->stream));
-    CU(c, cudaStreamSynchronize(c->stream));   // the host buffers are given back
+    if (sums)
+        CU(c, cudaMemcpyAsync(c->d_pair_start, c->pair_start.data(), sizeof(long long) * (c->n_members + 1),
+                              cudaMemcpyHostToDevice, c->stream));
+    // (the host's lists are the context's: they outlast the copies)
     c->pair_ok = true;
     return LBMBT_OK;
 }
@@ -1603,13 +1622,8 @@ static int prepare_as(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool
         long long biggest = 0;
         for (auto& d : c->descs) biggest = std::max(biggest, d.N);
         c->sig_parts = (int)std::max<long long>(16, std::min<long long>(biggest >> 14, 1024));
-        std::vector<long long> idx(n_members + 1);
-        std::iota(idx.begin(), idx.end(), 0LL);
-        rc = grow(c, &c->d_idx, &c->cap_ix, sizeof(long long) * idx.size());
-        if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n_members * c->sig_parts);
+        rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n_members * c->sig_parts);
         if (rc) return rc;
-        CU(c, cudaMemcpyAsync(c->d_idx, idx.data(), sizeof(long long) * idx.size(), cudaMemcpyHostToDevice, c->stream));
-        CU(c, cudaStreamSynchronize(c->stream));
     }
     if (ex) {
         // members' own waveforms: f_k (zero past the member's end, one entry
@@ -1724,7 +1738,8 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
         give_back(&c->d_pair_maps, &c->cap_pm);
         rc = prepare_as(c, n_members, mem, series, field_dev, ex, false, to_end);
     }
-    if (!rc) c->err.clear();
+    if (rc) cudaStreamSynchronize(c->stream);   // no copy of a list is left in flight
+    else c->err.clear();
     return rc;
 }
 
@@ -1734,7 +1749,7 @@ static int sum_signal(lbmbt_ctx* c)
     CU(c, launch_signal(c->d_desc, c->n_members, c->use_tma, c->use_tma ? tma_consumers(c->tma_variant) : c->tile_block,
                         c->use_tma ? tma_sites_per_thread(c->tma_variant) : c->tile_spt, c->sig_parts, c->d_partial,
                         c->stream));
-    CU(c, launch_reduce(c->d_partial, c->d_idx, c->sig_parts, c->n_members, c->d_Z, nullptr, 0, c->d_ctl, c->stream));
+    CU(c, launch_reduce(c->d_partial, nullptr, c->sig_parts, c->n_members, c->d_Z, nullptr, 0, c->d_ctl, c->stream));
     c->launches += 2;
     return LBMBT_OK;
 }
@@ -2269,7 +2284,6 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
         const size_t part = c->cap_partial;
         rc = grow(c, &c->d_mout, &c->cap_mo, sizeof(float2) * sites);
         if (!rc) rc = grow(c, &c->d_gsite, &c->cap_gs, sizeof(float) * 3 * sites * L_max);
-        if (!rc) rc = grow(c, &c->d_idx, &c->cap_ix, sizeof(long long) * (n + 1));
         if (!rc) rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n * c->sig_parts);
         if (rc == LBMBT_ENOMEM) {   // no room: one step a launch, with its partials
             cudaGetLastError();
@@ -2278,12 +2292,6 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
             rc = grow(c, &c->d_partial, &c->cap_partial, part);
         }
         if (rc) return rc;
-    }
-    if (res) {
-        std::vector<long long> idx(n + 1);
-        std::iota(idx.begin(), idx.end(), 0LL);
-        CU(c, cudaMemcpyAsync(c->d_idx, idx.data(), sizeof(long long) * idx.size(), cudaMemcpyHostToDevice, c->stream));
-        if ((rc = sync(c))) return rc;
     }
     {
         size_t oc = 0, os = 0;

@@ -177,7 +177,8 @@ cudaError_t launch_init(const SweepArgs& a, long long n_tiles, int block, int sp
 // Register sweep (one block per tile), then the one-thread step advance.
 cudaError_t launch_sweep(const SweepArgs& a, long long n_tiles, int block, int spt, cudaStream_t st);
 cudaError_t links_prepare();   // dynamic shared memory of the membrane-position sweeps
-// Sums partial[tile_start[m]*per .. tile_start[m+1]*per) per member.  steps =
+// Sums partial[tile_start[m]*per .. tile_start[m+1]*per) per member (tile_start NULL: [m*per ..
+// (m+1)*per)).  steps =
 // 2 (series after a two-step launch): the second step's partials follow at
 // `stride`, and both steps enter the series.
 cudaError_t launch_reduce(const double2* partial, const long long* tile_start, int per, int n_members,

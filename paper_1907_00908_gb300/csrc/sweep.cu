@@ -378,7 +378,7 @@ __global__ void reduce_kernel(const double2* __restrict__ partial, const long lo
     const int m = blockIdx.x;
     const int back = gridDim.y - blockIdx.y;   // this block's step ends at step word k - back + 1
     partial += blockIdx.y * stride;
-    const long long t0 = tile_start[m] * per, t1 = tile_start[m + 1] * per;
+    const long long t0 = (tile_start ? tile_start[m] : m) * per, t1 = (tile_start ? tile_start[m + 1] : m + 1) * per;
     double2 v = make_double2(0.0, 0.0);
     for (long long t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
         v.x += partial[t].x;

@@ -206,3 +206,24 @@ def test_runs_advanced_step_by_step_give_the_same_bits(lb, shape, bc, gG):
         tol = 2.0 ** -22 * geoms[0].n_sites
         assert np.abs(z - ref[0]).max() <= tol, split
         assert np.abs(zs - ref[0][0]).max() <= tol, split
+
+
+# few steps do not pay for the plan: four for the resident sweep and one more for each
+# 52000 sites, ten or 16 M site-steps for the two-step sweep; a caller's choice is taken
+@pytest.mark.parametrize("shape,n,multi,used", [
+    ((12, 13, 14), 3, 0, 1), ((12, 13, 14), 4, 0, 3), ((12, 13, 14), 2, 3, 3), ((40, 41, 42), 4, 0, 1), ((40, 41, 42), 5, 0, 3),
+    ((70, 66, 68), 9, 0, 1), ((70, 66, 68), 10, 0, 2),
+    ((70, 66, 68), 2, 2, 2), ((200, 200, 200), 2, 0, 2), ((199, 200, 200), 2, 0, 1), ((12, 13, 14), 1, 0, 1),
+])
+def test_runs_of_few_steps(lb, shape, n, multi, used):
+    g = _geom(shape, 8)
+    out = []
+    for opt in (multi, 1):
+        with _solver(lb, 0, [g], (0, 0, 0), (0.2, 0.1, 0.3), _wave("cos", n)) as s:
+            s.set_option(lb.OPT_MULTI_STEP, opt)
+            fld = torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda")
+            s.run(field=fld)
+            torch.cuda.synchronize()
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == (used if opt == multi else 1)
+            out.append(fld.cpu().numpy())
+    assert np.array_equal(out[0], out[1])
