@@ -310,7 +310,9 @@ int lbmbt_grad_batch(lbmbt_ctx* ctx, int n_members, const lbmbt_member* members,
 /* Options. */
 enum {
     LBMBT_OPT_GRAPH = 1,     /* 1 (default): replay step loops as CUDA graphs   */
-    LBMBT_OPT_AUTOTUNE = 2,  /* 1: time launch shapes on first use (default 0)  */
+    LBMBT_OPT_AUTOTUNE = 2,  /* 1: time the one-step sweeps' launch shapes on first
+                                use (default 0); a whole run that takes none of
+                                them (LBMBT_OPT_MULTI_STEP) does not           */
     LBMBT_OPT_BLOCK = 3,     /* threads per block of the register sweep: a
                                 multiple of 32 in 64..512                      */
     LBMBT_OPT_SPT = 4,       /* sites per thread of the sweep (1, 2 or 4)       */

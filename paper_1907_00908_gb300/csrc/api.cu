@@ -1340,7 +1340,9 @@ static int issue_pair(lbmbt_ctx* c, int steps)
 
 // Times a few steps of every launch shape that fits -- register sweep block x
 // sites per thread, bulk-copy sweep consumer shape x stages -- and keeps the
-// fastest for this problem shape (cached per shape for the context's life).
+// fastest for this problem shape (cached per shape for the context's life).  Runs that
+// are prepared and advanced are tuned whatever sweep they take: single steps are
+// one-step sweeps.
 static int autotune(lbmbt_ctx* c)
 {
     std::string key = std::to_string(c->n_members);
@@ -1699,14 +1701,17 @@ static int prepare_as(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool
     rc = grow(c, &c->d_Z, &c->cap_Z, sizeof(double2) * n_members);
     if (!rc && series) rc = grow(c, &c->d_series, &c->cap_series, sizeof(double2) * n_members * c->n_steps);
     if (rc) return rc;
-    if (c->autotune) {
-        rc = autotune(c);
-        if (rc) return rc;
-    }
+    // the tuner times the one-step sweeps: a run to the end by a multi-step sweep takes none
+    const bool untuned = c->autotune && to_end && c->multi_planned;
+    if (untuned) c->tuned_kernel = c->tuned_oz = 0;
+    else if (c->autotune && (rc = autotune(c))) return rc;
     rc = build_worklist(c, c->block, c->spt);
     if (!rc) rc = build_resident(c);
     if (!rc) rc = build_pair(c);
     if (rc) return rc;
+    if (untuned && !c->res_ok && !c->pair_ok) {   // the blocks did not hold the links after all
+        if ((rc = autotune(c)) || (rc = build_worklist(c, c->block, c->spt))) return rc;
+    }
     rc = init_state(c);
     if (rc) return rc;
     c->field_dev = field_dev;

@@ -227,3 +227,20 @@ def test_runs_of_few_steps(lb, shape, n, multi, used):
             assert s.get_option(lb.OPT_MULTI_STEP_USED) == (used if opt == multi else 1)
             out.append(fld.cpu().numpy())
     assert np.array_equal(out[0], out[1])
+
+
+# the tuner times one-step sweeps: whole runs of the others do not wait for it
+@pytest.mark.parametrize("shape,multi,tuned", [((70, 66, 68), 0, False), ((20, 24, 32), 0, False), ((70, 66, 68), 1, True)])
+def test_the_tuner_is_left_out_of_runs_that_take_none_of_its_sweeps(lb, shape, multi, tuned):
+    g = _geom(shape, 8)
+    out = []
+    for tune in (0, 1):
+        with _solver(lb, 0, [g], (0, 0, 0), (0.2, 0.1, 0.3), _wave("pgse", 20)) as s:
+            s.set_option(lb.OPT_MULTI_STEP, multi)
+            s.set_option(lb.OPT_AUTOTUNE, tune)
+            fld = torch.zeros(g.n_sites, dtype=torch.complex64, device="cuda")
+            s.run(field=fld)
+            torch.cuda.synchronize()
+            out.append((fld.cpu().numpy(), s.launch_count()))
+    assert np.array_equal(out[0][0], out[1][0])
+    assert (out[1][1] > out[0][1] + 50) if tuned else out[1][1] == out[0][1]
