@@ -964,20 +964,31 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
     std::vector<Cut> cuts(descs.size());
     c->res_strip_nx = 0;
     const int most = adjoint ? adj_resident_max_sites() : resident_max_sites();
-    if (total <= (long long)c->sm_count * most)
-    for (int t = 64; t <= most; t += t < 1024 ? 64 : 128) {
+    // (the bound, and one cut for members of one shape: with every size tried on every
+    // member, 150 members of 12^3 took 556 us for 16 steps where it now takes 270, and 100 of
+    // 14^3, which do not fit, 703 for 468)
+    auto fewest = [&](int t) {   // no plan of blocks of t sites has fewer
         long long n = 0;
-        int recv = 0;
-        bool ok = true;
-        for (size_t m = 0; m < descs.size() && ok; ++m) {
-            cuts[m] = cut(descs[m], t);
-            ok = cuts[m].cy > 0;
-            n += (long long)cuts[m].cy * cuts[m].cz;
-            recv = std::max(recv, cuts[m].recv);
+        for (auto& d : descs) n += (d.N + t - 1) / t;
+        return n;
+    };
+    if (fewest(most) <= c->sm_count)
+        for (int t = 64; t <= most; t += t < 1024 ? 64 : 128) {
+            if (fewest(t) > c->sm_count) continue;
+            long long n = 0;
+            int recv = 0;
+            bool ok = true;
+            for (size_t m = 0; m < descs.size() && ok; ++m) {
+                const bool same = m > 0 && descs[m].nx == descs[m - 1].nx && descs[m].ny == descs[m - 1].ny &&
+                                  descs[m].nz == descs[m - 1].nz;
+                cuts[m] = same ? cuts[m - 1] : cut(descs[m], t);
+                n += (long long)cuts[m].cy * cuts[m].cz;
+                recv = std::max(recv, cuts[m].recv);
+                ok = cuts[m].cy > 0 && n <= c->sm_count;
+            }
+            const size_t smem = adjoint ? adj_resident_smem(t, recv) : resident_smem(t, recv, c->lattice == 1);
+            if (ok && smem <= (size_t)limit) { cap = t; break; }
         }
-        const size_t smem = adjoint ? adj_resident_smem(t, recv) : resident_smem(t, recv, c->lattice == 1);
-        if (ok && n <= c->sm_count && smem <= (size_t)limit) { cap = t; break; }
-    }
     // (1000 x 1000: 11.4 us a step against 31 for the one-step sweep)
     if (!cap && c->lattice == 1 && !links && !adjoint) {   // larger 2-D grids: strips, all of the least height that will do
         for (int h = 1; h <= 8 && !c->res_strip_nx; ++h) {

@@ -201,3 +201,25 @@ def test_resident_gradient_of_long_segments(lb, n, every):
     for k in ("dD", "dT2", "dkappa"):
         a, b = np.asarray(out[0][k]), np.asarray(out[1][k])
         assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max(), (k, a, b)
+
+
+# as many members as SMs, of one shape and of mixed ones in any order; one too many blocks
+@pytest.mark.parametrize("shapes,used", [
+    ([(12, 12, 12)] * 150, 3), ([(6, 7, 8), (6, 7, 8), (9, 5, 7), (6, 7, 8)] * 30, 3), ([(14, 14, 14)] * 100, 2),
+    ([(20, 20, 20), (8, 9, 10), (20, 20, 20)] * 8, 3), ([(8, 9, 10)] * 153, 1),
+])
+def test_resident_batches_of_many_members(lb, shapes, used):
+    geoms = [_geom(sh, sum(sh)) for sh in sorted(set(shapes))]
+    which = [sorted(set(shapes)).index(sh) for sh in shapes]
+    rng = np.random.default_rng(2)
+    gs = [tuple(v) for v in rng.normal(size=(len(shapes), 3)) * 0.2]
+    out = []
+    for multi in (0, 1):
+        with _solver(lb, multi, geoms, (0, 0, 0), gs[0], _wave("pgse", 12), 0.03, 0) as s:
+            fields = [torch.zeros(geoms[i].n_sites, dtype=torch.complex64, device="cuda") for i in which]
+            s.run_batch(lb.Solver.members(gs, which, 0.03), fields=fields)
+            torch.cuda.synchronize()
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == (1 if multi else used)
+            out.append([v.cpu().numpy() for v in fields])
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
