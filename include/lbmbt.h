@@ -417,9 +417,13 @@ enum {
                                 now fail as if there were no room (once;
                                 LBMBT_ENOMEM where the call cannot do without);
                                 reads as those still to come; 0 (default) off */
-    LBMBT_OPT_TEST_STAMP = 21  /* tests of used-up stamps only: the stamp of the
+    LBMBT_OPT_TEST_STAMP = 21, /* tests of used-up stamps only: the stamp of the
                                 resident sweep's next packets (it can only be
                                 raised, to 2^32 - 1 at most)                 */
+    LBMBT_OPT_TEST_WAIT_SWEEPS = 22 /* with LBMBT_OPT_TEST_WAIT_NS: n > 0, the
+                                first n one-step sweeps from now only, and the
+                                other option is off after them; 0 (default)
+                                all sweeps                                    */
 };
 int lbmbt_set_option(lbmbt_ctx* ctx, int option, int64_t value);
 int lbmbt_get_option(lbmbt_ctx* ctx, int option, int64_t* value);

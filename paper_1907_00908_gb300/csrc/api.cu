@@ -160,6 +160,7 @@ struct lbmbt_ctx {
     bool ftab_valid = false;      // d_ftab holds the prepared members' factors
     int grad_groups = 0;          // member groups of the last lbmbt_grad_batch
     long long test_wait_ns = 0;   // tests of the sweeps' timeout paths (0: off)
+    long long test_wait_sweeps = 0;   // sweeps to come of that kind (0: all)
     long long fail_alloc = 0;     // tests: this many allocations from now, one fails (0: off)
     float2* d_etab = nullptr;     // per-member rotation tables
     size_t cap_etab = 0;
@@ -1274,7 +1275,9 @@ static int build_pair(lbmbt_ctx* c)
     return LBMBT_OK;
 }
 
-static int write_ctl(lbmbt_ctx* c, int sig_step, int field_step, int slot_base = 0, int slot_mod = 2)
+// keep_err: within a call that looks at the error word at its end only.
+static int write_ctl(lbmbt_ctx* c, int sig_step, int field_step, int slot_base = 0, int slot_mod = 2,
+                     bool keep_err = false)
 {
     StepCtl h;
     memset(&h, 0, sizeof h);   // counters start at zero
@@ -1285,7 +1288,7 @@ static int write_ctl(lbmbt_ctx* c, int sig_step, int field_step, int slot_base =
     h.slot_base = slot_base;
     h.slot_mod = slot_mod;
     h.series = c->series_mode ? 1 : 0;
-    h.err = 0;
+    h.err = keep_err ? -1 : 0;
     CU(c, launch_ctl_set(c->d_ctl, h, c->stream));
     c->launches++;
     return LBMBT_OK;
@@ -1325,6 +1328,7 @@ static int issue_step(lbmbt_ctx* c)
         CU(c, launch_sweep(a, c->n_tiles, c->tile_block, c->tile_spt, c->stream));
     }
     c->launches += c->use_tma ? 1 : 2;   // the register sweep is followed by the step advance
+    if (c->test_wait_sweeps > 0 && --c->test_wait_sweeps == 0) c->test_wait_ns = 0;
     if (c->series_mode) {
         CU(c, launch_reduce(c->d_partial, part_start(c), part_per(c), c->n_members, c->d_Z, c->d_series, c->n_steps, c->d_ctl,
                             c->stream));
@@ -2180,6 +2184,10 @@ extern "C" int lbmbt_set_option(lbmbt_ctx* c, int opt, int64_t v)
         if (v < 0 || v > 3) return fail(c, LBMBT_EINVAL, "steps of a pass must be 0 (auto), 1, 2 or 3 (resident)");
         c->multi_opt = (int)v;
         break;
+    case LBMBT_OPT_TEST_WAIT_SWEEPS:
+        if (v < 0) return fail(c, LBMBT_EINVAL, "sweeps whose wait runs out must be >= 0 (0: all)");
+        c->test_wait_sweeps = v;
+        break;
     case LBMBT_OPT_TEST_FAIL_ALLOC:
         if (v < 0) return fail(c, LBMBT_EINVAL, "allocations until one fails must be >= 0");
         c->fail_alloc = v;
@@ -2212,6 +2220,7 @@ extern "C" int lbmbt_get_option(lbmbt_ctx* c, int opt, int64_t* v)
     case LBMBT_OPT_SCHEME: *v = c->scheme; break;
     case LBMBT_OPT_GRAD_GROUPS: *v = c->grad_groups; break;
     case LBMBT_OPT_TEST_WAIT_NS: *v = c->test_wait_ns; break;
+    case LBMBT_OPT_TEST_WAIT_SWEEPS: *v = c->test_wait_sweeps; break;
     case LBMBT_OPT_TEST_FAIL_ALLOC: *v = c->fail_alloc; break;
     case LBMBT_OPT_TEST_STAMP: *v = c->res_stamp; break;
     case LBMBT_OPT_COLUMN_PLANES: *v = c->zc_opt; break;
@@ -2380,7 +2389,7 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
             }
             CU(c, cudaMemcpyAsync(c->d_desc, fd.data(), sizeof(MemberDesc) * n, cudaMemcpyHostToDevice, c->stream));
             c->k_cur = k;
-            if ((rc = write_ctl(c, (int)(K - 1), -1, (int)k, keep * ck + 1))) return rc;
+            if ((rc = write_ctl(c, (int)(K - 1), -1, (int)k, keep * ck + 1, true))) return rc;
         }
         if ((rc = issue_step(c))) return rc;
         const long long kn = k + 1;
@@ -2488,7 +2497,7 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
         }
         if (!kept && k1 - k0 - 1 > 0) {
             c->k_cur = k0;
-            if ((rc = write_ctl(c, -1, -1, (int)k0, ck + 1))) return rc;
+            if ((rc = write_ctl(c, -1, -1, (int)k0, ck + 1, true))) return rc;
             for (long long k = k0; k < k1 - 1; ++k)
                 if ((rc = issue_step(c))) return rc;
         }

@@ -165,7 +165,7 @@ cudaError_t launch_build_mask(const int32_t* labels, const uint8_t* phase_of_lab
                               int nx, int ny, int nz, const int bc[3], uint8_t* mask, int* err,
                               cudaStream_t st);
 // Writes v to the control word (before a run of sweeps, which then advance
-// it themselves).
+// it themselves); v.err < 0 leaves the error word as it is.
 cudaError_t launch_ctl_set(StepCtl* ctl, const StepCtl& v, cudaStream_t st);
 // Boundary factors of every step 0..K for every member, table[k][m][6], from
 // each member's F table at k + F_shift (1 for the classical scheme, whose

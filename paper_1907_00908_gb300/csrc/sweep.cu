@@ -347,7 +347,12 @@ __global__ void __launch_bounds__(512, ANG ? 1 : 2) sweep_links_kernel(const Swe
 }
 
 // Control word: set before a run of sweeps.
-__global__ void ctl_set_kernel(StepCtl* ctl, StepCtl v) { *ctl = v; }
+// v.err < 0: the error word stays.
+__global__ void ctl_set_kernel(StepCtl* ctl, StepCtl v)
+{
+    if (v.err < 0) v.err = ctl->err;
+    *ctl = v;
+}
 
 // Step advance after a register sweep.  That sweep has one block per tile
 // (~10^5 a step on large grids); a ticket per block at its end, as the

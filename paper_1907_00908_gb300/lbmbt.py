@@ -28,7 +28,7 @@ OPT_ADJOINT_KERNEL, OPT_ADJOINT_SHAPE, OPT_LATTICE = 9, 10, 11
 OPT_STAGE_OWN_Z, OPT_STAGE_OWN_Z_USED, OPT_SCHEME, OPT_GRAD_GROUPS, OPT_TEST_WAIT_NS = 12, 13, 14, 15, 16
 OPT_COLUMN_PLANES = 17
 OPT_MULTI_STEP, OPT_MULTI_STEP_USED = 18, 19
-OPT_TEST_FAIL_ALLOC, OPT_TEST_STAMP = 20, 21
+OPT_TEST_FAIL_ALLOC, OPT_TEST_STAMP, OPT_TEST_WAIT_SWEEPS = 20, 21, 22
 
 # every entry point declared in include/lbmbt.h
 EXPORTS = [

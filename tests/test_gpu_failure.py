@@ -304,3 +304,22 @@ def test_contexts_on_threads_with_blocks_of_different_size(lb):
     for t in th:
         t.join()
     assert not fail, fail
+
+
+# one lost copy in the first sweep; step words written after it where the kept segments
+# (7 of 14, 5 of 6, all) start and where segments are recomputed
+@pytest.mark.parametrize("every", [3, 7, 40])
+def test_gradient_reports_a_time_out_of_its_first_sweep(lb, every):
+    s, job = _setup(lb, (4, 6, 16), 40)
+    s.set_option(lb.OPT_KERNEL, 2)
+    s.set_option(lb.OPT_MULTI_STEP, 1)
+    want = s.grad(checkpoint_every=every)
+    s.set_option(lb.OPT_TEST_WAIT_SWEEPS, 1)
+    s.set_option(lb.OPT_TEST_WAIT_NS, 1_000_000)
+    with pytest.raises(lb.LbmbtError) as e:
+        s.grad(checkpoint_every=every)
+    assert e.value.code == -6 and "timed out" in str(e.value)
+    assert s.get_option(lb.OPT_TEST_WAIT_NS) == 0
+    again = s.grad(checkpoint_every=every)
+    s.close()
+    assert again["Z"] == want["Z"] and np.array_equal(again["dD"], want["dD"])
