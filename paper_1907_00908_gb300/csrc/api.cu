@@ -332,6 +332,7 @@ extern "C" int lbmbt_destroy(lbmbt_ctx* c)
     cudaFree(c->d_res_blocks); cudaFree(c->d_packets); cudaFree(c->d_mout);
     cudaFree(c->d_res_start); cudaFree(c->d_zpart); cudaFree(c->d_gsite);
     cudaFree(c->d_ck); cudaFree(c->d_seg); cudaFree(c->d_gacc); cudaFree(c->d_gout); cudaFree(c->d_laminit);
+    cudaFree(c->d_wf); cudaFree(c->d_wF);
     if (c->owned_stream) cudaStreamDestroy(c->owned_stream);
     delete c;
     return LBMBT_OK;

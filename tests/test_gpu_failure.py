@@ -323,3 +323,17 @@ def test_gradient_reports_a_time_out_of_its_first_sweep(lb, every):
     again = s.grad(checkpoint_every=every)
     s.close()
     assert again["Z"] == want["Z"] and np.array_equal(again["dD"], want["dD"])
+
+
+def test_a_closed_context_holds_no_memory(lb):
+    def job():
+        s, job = _setup(lb, (4, 4, 4), 20000)
+        waves = [np.full(20000 - i, 1e-3) for i in range(64)]
+        s.run_batch(lb.Solver.members([job[7]] * 64, 0, job[4]), waveforms=waves)
+        s.close()
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    first = job()
+    last = [job() for _ in range(6)][-1]
+    assert first - last < 16 << 20      # the 64 waveforms and their integrals take 15 MB a context
