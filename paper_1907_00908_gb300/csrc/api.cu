@@ -2265,6 +2265,7 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
     int rc = prepare(c, n, mem, false, nullptr, nullptr, false);   // the adjoint reads every level
     c->block = saved_block;
     if (rc) return rc;
+    c->prepared = false;   // not a run to be advanced: the descriptors become those of the reverse pass
     const long long K = c->n_steps;
     const long long n_ck = (K + ck - 1) / ck;
     size_t lvl_total = 0;
@@ -2523,7 +2524,6 @@ static int grad_group(lbmbt_ctx* c, int n, const lbmbt_member* mem, int ck, int 
     std::vector<double> G((size_t)NGACC * n);
     CU(c, cudaMemcpyAsync(G.data(), c->d_gout, sizeof(double) * G.size(), cudaMemcpyDeviceToHost, c->stream));
     if ((rc = check_device_error(c))) return rc;
-    c->prepared = false;  // descriptors now describe the reverse pass
     // chain rule to the physical parameters
     const double eps = c->lattice == 1 ? EPS_D2 : EPS_D;
     for (int m = 0; m < n; ++m) {

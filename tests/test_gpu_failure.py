@@ -337,3 +337,21 @@ def test_a_closed_context_holds_no_memory(lb):
     first = job()
     last = [job() for _ in range(6)][-1]
     assert first - last < 16 << 20      # the 64 waveforms and their integrals take 15 MB a context
+
+
+@pytest.mark.parametrize("kind", ["time-out", "memory", "none"])
+def test_nothing_is_prepared_after_a_gradient_however_it_ended(lb, kind):
+    s, job = _setup(lb, (20, 24, 32), 11)
+    s.set_option(lb.OPT_TEST_WAIT_NS, 1_000_000 if kind == "time-out" else 0)
+    s.set_option(lb.OPT_TEST_FAIL_ALLOC, 14 if kind == "memory" else 0)   # after the forward pass's set-up
+    if kind == "none":
+        s.grad(checkpoint_every=4)
+    else:
+        with pytest.raises(lb.LbmbtError) as e:
+            s.grad(checkpoint_every=4)
+        assert e.value.code == (-6 if kind == "time-out" else -2)
+    s.set_option(lb.OPT_TEST_FAIL_ALLOC, 0)
+    with pytest.raises(lb.LbmbtError) as e:
+        s.advance(1)
+    assert e.value.code == -7
+    s.close()
