@@ -8,6 +8,7 @@
 // 512-byte aligned.  A member owns `n_slots` such time levels back to back
 // (stride 7*plane): 2 for the ping-pong of a run, c+1 for an adjoint segment.
 #pragma once
+#include <cstddef>
 #include <cstdint>
 #include <mutex>
 
@@ -63,6 +64,10 @@ struct MemberDesc {
     int rpu;              // x-rows per unit of the bulk-copy sweep
     int rpu_adj;          // x-rows per unit of the bulk-copy adjoint sweep
     long long unit0_adj;  // first row-unit of this member (bulk-copy adjoint)
+    // resident and two-step sweeps: where M goes at the signal step, for
+    // launch_signal to sum (the field buffer, if it is written at that step
+    // too); nullptr (two-step only): the sweep sums M itself
+    float2* mout;
     int nx, ny, nz;
     int pitch;            // two-step sweep: length of the state's rows, with ghost columns
                           // (the other sweeps' rows are nx long)
@@ -103,14 +108,16 @@ struct MemberDesc {
     // run's shared tables unless the member has a waveform of its own
     const float* fw;
     const double* Fw;
-    // resident and two-step sweeps: where M goes at the signal step, for
-    // launch_signal to sum (the field buffer, if it is written at that step
-    // too); nullptr (two-step only): the sweep sums M itself
-    float2* mout;
     // step whose end signal partials (and field, if any) are this member's
     // own: its echo when it is shorter than the run; -1: the step control's
     int end_step;
 };
+// Where the extents and faces lie decides how every thread of the register sweep loads
+// them at its start: with nx .. pitch off a 16-byte word it took 0.4 us a step more (2-D,
+// 1400 x 1100: 48.9 us for 48.5); with pitch and mout after the rest, where that sweep was
+// as fast, the two-step sweep and the strips were 1 to 1.5 % slower.
+static_assert(offsetof(MemberDesc, nx) % 16 == 0 && offsetof(MemberDesc, pitch) == offsetof(MemberDesc, nx) + 12 &&
+              offsetof(MemberDesc, bc) % 16 == 0 && sizeof(MemberDesc) % 16 == 0, "extents on one 16-byte word");
 
 // Step control word in device memory.  Every block of a sweep reads k at its
 // start.  The bulk-copy sweep's last CTA to be done with it (a two-level

@@ -152,7 +152,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& a)
     const float2* __restrict__ src = sd->state + (size_t)((k - sbase) % smod) * 7 * P;
     float2* __restrict__ dst = sd->state + (size_t)((k + 1 - sbase) % smod) * 7 * P;
     const uint8_t* __restrict__ mask = sd->mask;
-    const int nx = sd->nx, ny = sd->ny, nz = sd->nz;
+    const int4 dim = *reinterpret_cast<const int4*>(&sd->nx);   // nx, ny, nz, pitch
+    const int nx = dim.x, ny = dim.y, nz = dim.z;
     const int bcx = sd->bc[0], bcy = sd->bc[1], bcz0 = sd->zbc[0], bcz1 = sd->zbc[1];
     const unsigned sxy = (unsigned)nx * ny;
     const unsigned N = (unsigned)sd->N;
