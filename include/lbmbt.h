@@ -404,12 +404,18 @@ enum {
                                 scheme, no slabs and no membrane angles: how
                                 many steps a pass over the state makes.  0
                                 (default) auto: all of them in one launch
-                                (resident sweep) where the grids fit on chip,
-                                else two (two-step sweep) where nx, ny, nz >= 4
-                                on D3Q7 with half-link membranes and the planes
-                                are no thin columns, else one.  1
-                                one; 2 two where it can run; 3 resident where
-                                the grids fit.  The fields are the same bits */
+                                (resident sweep) where the grids fit on chip
+                                and the run has at least 4 to 9 steps, else
+                                two (two-step sweep) where nx, ny, nz >= 4 on
+                                D3Q7 with half-link membranes, the planes are
+                                no thin columns and the run has 10 steps or 16
+                                million site-steps, else one.  1 one; 2 two
+                                where it can run; 3 resident where the grids
+                                fit.  Steps that lbmbt_advance makes one by one
+                                are one-step sweeps.  The fields are the same
+                                bits; where memory has no room for M, a
+                                two-step run's signals are summed in other
+                                groups (2^-22 of the sum of |M|)             */
     LBMBT_OPT_MULTI_STEP_USED = 19, /* read-only: 1, 2 or 3 for the prepared
                                 run, else 0                                  */
     LBMBT_OPT_TEST_FAIL_ALLOC = 20, /* tests of scarce memory only: n > 0 makes

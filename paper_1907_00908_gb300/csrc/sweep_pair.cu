@@ -9,8 +9,8 @@
 // A thread has two neighbouring columns (x, x + 1); the block covers the tile
 // grown by two columns in x and one in y on each side.  It marches along z.
 // At plane z
-//   step 1  every thread computes hat g(t^(k+1)) of its columns at z from
-//           global memory, the halo columns included;
+//   step 1  every thread computes hat g(t^(k+1)) of its columns at z, the halo
+//           columns included, from the plane's inputs in shared memory;
 //   step 2  the threads of the tile compute hat g(t^(k+2)) at plane z - 1 from
 //           the step-1 values around it and store it.
 // Populations 0, 5 and 6 move along the thread's own columns: their step-1
