@@ -316,6 +316,15 @@ def _timed_advance(solver, stream, members, steps, warmup, want_signal=True):
     return e0.elapsed_time(e1) / steps, clk.summary(), sig
 
 
+def _own_z_options(s, lbmbt, args):
+    """The own-z form asked for.  The forms are of the one-step bulk-copy sweep,
+    so asking for one asks for that sweep."""
+    s.set_option(lbmbt.OPT_STAGE_OWN_Z, args.stage_own_z)
+    s.set_option(lbmbt.OPT_COLUMN_PLANES, args.column_planes)
+    if args.stage_own_z or args.column_planes:
+        s.set_option(lbmbt.OPT_MULTI_STEP, 1)
+
+
 def _sweep_kind(s, lbmbt):
     """The sweep of the prepared run: "two-step", "resident" or, one pass a
     step, "bulk-copy" or "register"."""
@@ -384,8 +393,7 @@ def measure_batch(args, stream):
     cyl, packs, members, f = batch_workload()
     t_gen = time.perf_counter() - t0
     s = lbmbt.Solver(0, stream)
-    s.set_option(lbmbt.OPT_STAGE_OWN_Z, args.stage_own_z)
-    s.set_option(lbmbt.OPT_COLUMN_PLANES, args.column_planes)
+    _own_z_options(s, lbmbt, args)
     s.set_option(lbmbt.OPT_AUTOTUNE, 0 if args.no_autotune else 1)
     s.set_geometry(cyl.labels, cyl.phase_of_label, 0.5)
     for g in packs:
@@ -881,8 +889,8 @@ def main():
     ap.add_argument("--adjoint-kernel", type=int, default=0, choices=[0, 1, 2],
                     help="adjoint sweep: 0 auto, 1 register, 2 bulk copy")
     ap.add_argument("--stage-own-z", type=int, default=0, choices=[0, 1, 2, 3],
-                    help="bulk-copy sweep: own z values 0 auto, 1 prefetched into registers, 2 staged, "
-                         "3 z-marching columns")
+                    help="one-step bulk-copy sweep: own z values 1 prefetched into registers, 2 staged, "
+                         "3 z-marching columns (0: auto, and whichever sweep the library chooses)")
     ap.add_argument("--column-planes", type=int, default=0,
                     help="bulk-copy sweep, z-marching form: planes per column (0 auto, else a power of two)")
     ap.add_argument("--members", type=int, default=60, help="adjoint workload: number of members (<= 60)")
@@ -955,8 +963,7 @@ def main():
     nm = len(seqs)
 
     s = lbmbt.Solver(local, stream)
-    s.set_option(lbmbt.OPT_STAGE_OWN_Z, args.stage_own_z)
-    s.set_option(lbmbt.OPT_COLUMN_PLANES, args.column_planes)
+    _own_z_options(s, lbmbt, args)
     if not args.no_autotune:
         s.set_option(lbmbt.OPT_AUTOTUNE, 1)
     if args.block:

@@ -90,3 +90,19 @@ def test_clock_samplers_keep_their_own_records():
     nvidia-smi record, so a line's clocks are those of its own region."""
     a, b = bench.Clocks(0), bench.Clocks(0)
     assert a.path != b.path
+
+
+def test_an_own_z_form_asked_for_is_a_one_step_sweep():
+    import types
+
+    from paper_1907_00908_gb300 import lbmbt
+
+    class Fake(dict):
+        def set_option(self, opt, value):
+            self[opt] = value
+
+    for own_z, planes, multi in ((0, 0, None), (2, 0, 1), (3, 8, 1), (0, 16, 1)):
+        s = Fake()
+        bench._own_z_options(s, lbmbt, types.SimpleNamespace(stage_own_z=own_z, column_planes=planes))
+        assert (s[lbmbt.OPT_STAGE_OWN_Z], s[lbmbt.OPT_COLUMN_PLANES]) == (own_z, planes)
+        assert s.get(lbmbt.OPT_MULTI_STEP) == multi
