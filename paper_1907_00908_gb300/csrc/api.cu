@@ -112,6 +112,7 @@ struct lbmbt_ctx {
     bool pair_state = false;      // the state has its layout (else the one-step sweeps')
     int other_advances = 0;       // calls in a row whose sweep would want the other layout
     int multi_opt = 0;            // steps of a pass: 0 auto, 1 one, 2 two, 3 resident
+    bool lists_in_flight = false; // copies of the context's lists to the device may not be done
     bool multi_planned = false;   // the set-up took the run to a multi-step sweep
     bool general = false;         // the run has a waveform value other than 0, +-1
     // resident sweep (auto kernel choice, small grids)
@@ -346,6 +347,7 @@ extern "C" const char* lbmbt_last_error(const lbmbt_ctx* c)
 static int sync(lbmbt_ctx* c)
 {
     CU(c, cudaStreamSynchronize(c->stream));
+    c->lists_in_flight = false;
     return LBMBT_OK;
 }
 
@@ -1008,6 +1010,10 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
         }
     }
     if (!cap && !c->res_strip_nx) return LBMBT_OK;
+    if (c->lists_in_flight) {   // after a call that ended early
+        const int rc = sync(c);
+        if (rc) return rc;
+    }
     c->res_blocks.clear();
     c->res_sites = c->res_recv = 0;
     for (size_t m = 0; m < descs.size(); ++m) {
@@ -1081,6 +1087,7 @@ static int build_resident(lbmbt_ctx* c)
         if (!rc) rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * nb * std::min(c->n_steps, RES_SERIES_CHUNK));
     }
     if (rc) return rc;
+    c->lists_in_flight = true;
     CU(c, cudaMemcpyAsync(c->d_res_blocks, c->res_blocks.data(), sizeof(ResBlock) * nb, cudaMemcpyHostToDevice, c->stream));
     if (c->series_mode) {
         c->res_start.assign(n + 1, 0);
@@ -1225,6 +1232,10 @@ static int build_pair(lbmbt_ctx* c)
         if (est < best) { best = est; best_zc = zc; }
         if (n > 64 * slots) break;
     }
+    if (c->lists_in_flight) {   // after a call that ended early
+        const int rc = sync(c);
+        if (rc) return rc;
+    }
     c->pair_items.clear();
     c->pair_start.assign(c->n_members + 1, 0);
     for (int m = 0; m < c->n_members; ++m) {
@@ -1266,13 +1277,14 @@ static int build_pair(lbmbt_ctx* c)
                 CU(c, pair_encode_map(&maps[2 * ((size_t)more * c->n_members + m) + lvl],
                                       d.state + (size_t)lvl * 7 * d.plane, d, tl[m].w / 2 + 2, tl[m].h + 2 + more));
     }
+    c->lists_in_flight = true;
     CU(c, cudaMemcpyAsync(c->d_pair_maps, maps.data(), sizeof(PairMap) * maps.size(), cudaMemcpyHostToDevice, c->stream));
     CU(c, cudaMemcpyAsync(c->d_pair_items, c->pair_items.data(), sizeof(PairItem) * n, cudaMemcpyHostToDevice, c->stream));
     if (sums)
         CU(c, cudaMemcpyAsync(c->d_pair_start, c->pair_start.data(), sizeof(long long) * (c->n_members + 1),
                               cudaMemcpyHostToDevice, c->stream));
-    // (the host's lists are the context's: they outlast the copies)
-    c->pair_ok = true;
+    c->pair_ok = true;   // (the host's lists are the context's: they outlast the copies)
+
     return LBMBT_OK;
 }
 
@@ -1759,8 +1771,7 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
         give_back(&c->d_pair_maps, &c->cap_pm);
         rc = prepare_as(c, n_members, mem, series, field_dev, ex, false, to_end);
     }
-    if (rc) cudaStreamSynchronize(c->stream);   // no copy of a list is left in flight
-    else c->err.clear();
+    if (!rc) c->err.clear();
     return rc;
 }
 
@@ -1951,7 +1962,8 @@ static int check_device_error(lbmbt_ctx* c)
 {
     int err = 0;
     CU(c, cudaMemcpyAsync(&err, &c->d_ctl->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    CU(c, cudaStreamSynchronize(c->stream));
+    const int rc = sync(c);
+    if (rc) return rc;
     if (err) return fail(c, LBMBT_EDEVICE, "a device-side wait timed out (error word %d)", err);
     return LBMBT_OK;
 }
