@@ -133,8 +133,12 @@ struct lbmbt_ctx {
     bool has_mout = false;        // the members have mout: the signal is summed from it
     int sig_parts = 0;            // parts of a member's signal
     std::vector<int> res_start;
-    int* d_res_start = nullptr;   // [n + 1] blocks of a member (series)
+    int* d_res_start = nullptr;   // series: [n + 1] where a member's parts of Z start
     size_t cap_rs = 0;
+    float2* d_mser = nullptr;     // series (blocks): M after each step of a launch
+    size_t cap_ms = 0;
+    long long ser_sites = 0;      // sites of all members
+    int ser_parts = 0;            // parts of a member's sum
     double2* d_zpart = nullptr;
     size_t cap_zp = 0;
     int pair_per_sm[2] = {0, 0};  // resident blocks of its two forms
@@ -331,7 +335,7 @@ extern "C" int lbmbt_destroy(lbmbt_ctx* c)
     cudaFree(c->d_adj_unit_start); cudaFree(c->d_halo); cudaFree(c->d_pair_items); cudaFree(c->d_pair_start);
     cudaFree(c->d_pair_maps);
     cudaFree(c->d_res_blocks); cudaFree(c->d_packets); cudaFree(c->d_mout);
-    cudaFree(c->d_res_start); cudaFree(c->d_zpart); cudaFree(c->d_gsite);
+    cudaFree(c->d_res_start); cudaFree(c->d_mser); cudaFree(c->d_zpart); cudaFree(c->d_gsite);
     cudaFree(c->d_ck); cudaFree(c->d_seg); cudaFree(c->d_gacc); cudaFree(c->d_gout); cudaFree(c->d_laminit);
     cudaFree(c->d_wf); cudaFree(c->d_wF);
     if (c->owned_stream) cudaStreamDestroy(c->owned_stream);
@@ -1053,9 +1057,19 @@ static int plan_resident(lbmbt_ctx* c, const std::vector<MemberDesc>& descs, boo
     return LBMBT_OK;
 }
 
-// A launch of the resident sweep takes at most RES_CHUNK steps (in series mode fewer:
-// the parts of Z of every step wait in memory for their sum).
-constexpr long long RES_CHUNK = 1 << 15, RES_SERIES_CHUNK = 1 << 12;
+// A launch of the resident sweep takes at most RES_CHUNK steps, for a series
+// RES_SERIES_CHUNK: the parts of Z of every step wait in memory for their sum.  Strips
+// make them on chip, in FP64; for blocks M after each step waits, as many steps as 256
+// MB hold, 32 at least, and the parts are made of the one-step sweeps' thread sums.  (Made
+// on chip, a step's Z of free diffusion on 46 x 23 x 41, where the FP32 roundings of all
+// rows are alike, was off the one-step sweep's by 6e-8 of the largest.)
+constexpr long long RES_CHUNK = 1 << 15, RES_SERIES_CHUNK = 1 << 12, RES_SERIES_BYTES = 256 << 20;
+
+static long long series_chunk(const lbmbt_ctx* c)
+{
+    if (c->res_strip_nx) return RES_SERIES_CHUNK;
+    return std::min(RES_SERIES_CHUNK, std::max(32LL, RES_SERIES_BYTES / (long long)(sizeof(float2) * c->ser_sites)));
+}
 
 static size_t resident_packets(const lbmbt_ctx* c) { return 4 * (size_t)std::max(c->res_recv, 1) * c->res_blocks.size(); }
 
@@ -1083,8 +1097,18 @@ static int build_resident(lbmbt_ctx* c)
     }
     if (!rc) rc = grow(c, &c->d_res_blocks, &c->cap_rb, sizeof(ResBlock) * nb);
     if (!rc && c->series_mode) {
+        long long biggest = 0;
+        c->ser_sites = 0;
+        for (auto& d : c->descs) {
+            c->ser_sites += d.N;
+            biggest = std::max(biggest, d.N);
+        }
+        c->ser_parts = (int)std::max<long long>(1, std::min<long long>(biggest >> 13, 64));
+        const long long steps = std::min(c->n_steps, series_chunk(c));
+        const int parts = c->res_strip_nx ? nb : n * c->ser_parts;
         rc = grow(c, &c->d_res_start, &c->cap_rs, sizeof(int) * (n + 1));
-        if (!rc) rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * nb * std::min(c->n_steps, RES_SERIES_CHUNK));
+        if (!rc) rc = grow(c, &c->d_zpart, &c->cap_zp, sizeof(double2) * parts * steps);
+        if (!rc && !c->res_strip_nx) rc = grow(c, &c->d_mser, &c->cap_ms, sizeof(float2) * c->ser_sites * steps);
     }
     if (rc) return rc;
     c->lists_in_flight = true;
@@ -1092,7 +1116,7 @@ static int build_resident(lbmbt_ctx* c)
     if (c->series_mode) {
         c->res_start.assign(n + 1, 0);
         for (auto& b : c->res_blocks) c->res_start[b.m + 1]++;
-        for (int m = 0; m < n; ++m) c->res_start[m + 1] += c->res_start[m];
+        for (int m = 0; m < n; ++m) c->res_start[m + 1] = c->res_strip_nx ? c->res_start[m] + c->res_start[m + 1] : (m + 1) * c->ser_parts;
         CU(c, cudaMemcpyAsync(c->d_res_start, c->res_start.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, c->stream));
     }
     c->res_max_links = 0;
@@ -1649,8 +1673,12 @@ static int prepare_as(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool
             if (own && d.field) d.mout = d.field;
             else { d.mout = c->d_mout + at; at += (size_t)d.N; }
         }
-        long long biggest = 0;
-        for (auto& d : c->descs) biggest = std::max(biggest, d.N);
+        long long biggest = 0, sites = 0;
+        for (auto& d : c->descs) {
+            biggest = std::max(biggest, d.N);
+            d.moff = c->res_ok ? (int)sites : 0;   // (grids on chip: few enough for an int)
+            sites += d.N;
+        }
         c->sig_parts = (int)std::max<long long>(16, std::min<long long>(biggest >> 14, 1024));
         rc = grow(c, &c->d_partial, &c->cap_partial, sizeof(double2) * (size_t)n_members * c->sig_parts);
         if (rc) return rc;
@@ -1767,6 +1795,7 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
         give_back(&c->d_mout, &c->cap_mo);
         give_back(&c->d_packets, &c->cap_pk);
         give_back(&c->d_zpart, &c->cap_zp);
+        give_back(&c->d_mser, &c->cap_ms);
         give_back(&c->d_pair_items, &c->cap_pi);
         give_back(&c->d_pair_maps, &c->cap_pm);
         rc = prepare_as(c, n_members, mem, series, field_dev, ex, false, to_end);
@@ -1775,11 +1804,14 @@ static int prepare(lbmbt_ctx* c, int n_members, const lbmbt_member* mem, bool se
     return rc;
 }
 
+// Threads and sites a thread of the one-step sweep, whose thread sums signals are made of.
+static int signal_block(const lbmbt_ctx* c) { return c->use_tma ? tma_consumers(c->tma_variant) : c->tile_block; }
+static int signal_spt(const lbmbt_ctx* c) { return c->use_tma ? tma_sites_per_thread(c->tma_variant) : c->tile_spt; }
+
 // Z of every member from its mout, with the one-step sweep's thread sums.
 static int sum_signal(lbmbt_ctx* c)
 {
-    CU(c, launch_signal(c->d_desc, c->n_members, c->use_tma, c->use_tma ? tma_consumers(c->tma_variant) : c->tile_block,
-                        c->use_tma ? tma_sites_per_thread(c->tma_variant) : c->tile_spt, c->sig_parts, c->d_partial,
+    CU(c, launch_signal(c->d_desc, c->n_members, c->use_tma, signal_block(c), signal_spt(c), c->sig_parts, c->d_partial,
                         c->stream));
     CU(c, launch_reduce(c->d_partial, nullptr, c->sig_parts, c->n_members, c->d_Z, nullptr, 0, c->d_ctl, c->stream));
     c->launches += 2;
@@ -1815,7 +1847,7 @@ static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_ste
 {
     const SweepArgs a = sweep_args(c);
     const int nb = (int)c->res_blocks.size();
-    const long long chunk = c->series_mode ? RES_SERIES_CHUNK : RES_CHUNK;
+    const long long chunk = c->series_mode ? series_chunk(c) : RES_CHUNK;
     for (long long k = c->k_cur, end = c->k_cur + n; k < end;) {
         ResArgs r;
         const int rc = resident_args(c, k, std::min(chunk, end - k), r);
@@ -1824,15 +1856,23 @@ static int issue_resident(lbmbt_ctx* c, long long n, int sig_step, int field_ste
         r.ldst = (int)((k + r.n_steps - c->slot_base) & 1);
         r.sig_step = sig_step;
         r.field_step = field_step;
+        const bool strips = c->res_strip_nx > 0;
         r.series = c->series_mode ? 1 : 0;
         r.zpart = c->d_zpart;
-        if (c->res_strip_nx) CU(c, launch_strip(a, r, nb, c->res_strip_nx, c->res_smem, c->general, c->stream));
+        r.mser = c->series_mode && !strips ? c->d_mser : nullptr;
+        r.mstride = c->ser_sites;
+        if (strips) CU(c, launch_strip(a, r, nb, c->res_strip_nx, c->res_smem, c->general, c->stream));
         else
             CU(c, launch_resident(a, r, nb, c->res_sites, c->res_smem, c->lattice == 1, c->general, c->stream));
         c->launches++;
         if (c->series_mode) {
-            CU(c, launch_resident_series(c->d_zpart, c->d_res_start, c->n_members, nb, r.n_steps, k, c->n_steps, c->d_series,
-                                         c->stream));
+            if (!strips) {
+                CU(c, launch_series_parts(c->d_desc, c->n_members, c->use_tma, signal_block(c), signal_spt(c), c->ser_parts,
+                                          c->d_mser, c->ser_sites, r.n_steps, c->d_zpart, c->stream));
+                c->launches++;
+            }
+            CU(c, launch_resident_series(c->d_zpart, c->d_res_start, c->n_members, strips ? nb : c->n_members * c->ser_parts,
+                                         r.n_steps, k, c->n_steps, c->d_series, c->stream));
             c->launches++;
         }
         k += r.n_steps;

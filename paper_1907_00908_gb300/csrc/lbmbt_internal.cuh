@@ -111,6 +111,7 @@ struct MemberDesc {
     // step whose end signal partials (and field, if any) are this member's
     // own: its echo when it is shorter than the run; -1: the step control's
     int end_step;
+    int moff;             // resident sweep, series: where its sites start among all members'
 };
 // Where the extents and faces lie decides how every thread of the register sweep loads
 // them at its start: with nx .. pitch off a 16-byte word it took 0.4 us a step more (2-D,
@@ -257,11 +258,13 @@ struct ResArgs {
     int sig_step, field_step;     // as in StepCtl; a member's own end step goes before them
     int links;                    // 1: a member has membrane positions
     int max_links;                // listed links of a block at most (rounded up to even)
-    int series;                   // 1: zpart[n][block] = the block's part of Z after each step
+    int series;                   // strips: zpart[n][block] = the block's part of Z after each step
     double2* zpart;
     int levels;                   // 1: the levels of steps k0 .. k0 + n_steps - 1 go to the member's
                                   // adj, one after the other from slot level0 (gradient segments)
     int level0;
+    float2* mser;                 // blocks, series: M after each step, [n_steps][mstride], a
+    long long mstride;            // member's from moff on; else nullptr
 };
 int resident_max_sites();         // sites of a block
 size_t resident_smem(int sites, int recv, bool d2);
@@ -281,6 +284,10 @@ cudaError_t launch_strip(const SweepArgs& a, const ResArgs& r, int n_blocks, int
 // out[m][parts], to be summed; rows: the thread sums of the bulk-copy sweep
 cudaError_t launch_signal(const MemberDesc* members, int n_members, bool rows, int block, int spt, int parts, double2* out,
                           cudaStream_t st);
+// Parts of Z after each step from mser, with the same thread sums: [n_steps][n_members][parts].
+cudaError_t launch_series_parts(const MemberDesc* members, int n_members, bool rows, int block, int spt, int parts,
+                                const float2* mser, long long mstride, int n_steps, double2* zpart, cudaStream_t st);
+// Their sums: zpart[n][n_blocks], a member's from block_start[m] to block_start[m + 1].
 cudaError_t launch_resident_series(const double2* zpart, const int* block_start, int n_members, int n_blocks, int n_steps,
                                    long long k0, long long stride, double2* series, cudaStream_t st);
 

@@ -108,7 +108,6 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
     __shared__ float2 s_fac[2][6];   // boundary factors of this step and of the next
     __shared__ float s_f[2];
     __shared__ float2 s_phase[4];    // (omega, eps) per phase
-    __shared__ double2 s_red[RES_NT / 32];
 
     constexpr int NP = D2 ? 4 : 6;   // populations in shared memory: 1 .. NP
     const int t = threadIdx.x;
@@ -330,7 +329,6 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
             __syncthreads();
         }
         const bool do_sig = k == sig, do_fld = field != nullptr && k == fstep;
-        double zr = 0.0, zi = 0.0;
 #pragma unroll
         for (int j = 0; j < SPT; ++j) {
             const int l = t + j * RES_NT;
@@ -393,32 +391,15 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
 #pragma unroll
             for (int i = 1; i <= NP; ++i) reinterpret_cast<u64*>(nxt)[(i - 1) * S + l] = g[i];
             if (!D2 && r.levels && n + 1 < r.n_steps) put_level(n + 1, l, gs[j], g[0], reinterpret_cast<const u64*>(nxt));
-            if (do_sig || do_fld || r.series) {
+            if (do_sig || do_fld || r.mser) {
                 const float2 v = unpk(M);
                 if (do_sig) mout[gs[j]] = v;
                 if (do_fld) field[gs[j]] = v;
-                zr += v.x;
-                zi += v.y;
+                if (r.mser) r.mser[(size_t)n * r.mstride + d->moff + gs[j]] = v;
             }
         }
         if (t < 6) s_fac[(n & 1) ^ 1][t] = fnext;
         if (t == 6) s_f[(n & 1) ^ 1] = fnext.x;
-        if (r.series) {   // this block's part of Z after the step
-            for (int o = 16; o > 0; o >>= 1) {
-                zr += __shfl_down_sync(0xffffffffu, zr, o);
-                zi += __shfl_down_sync(0xffffffffu, zi, o);
-            }
-            if ((t & 31) == 0) s_red[t >> 5] = make_double2(zr, zi);
-            __syncthreads();
-            if (t == 0) {
-                double2 v = make_double2(0.0, 0.0);
-                for (int w = 0; w < RES_NT / 32; ++w) {
-                    v.x += s_red[w].x;
-                    v.y += s_red[w].y;
-                }
-                r.zpart[(size_t)n * gridDim.x + blockIdx.x] = v;
-            }
-        }
     }
 
     // each site's values are this thread's own
@@ -443,19 +424,17 @@ __global__ void __launch_bounds__(RES_NT, 1) sweep_resident_kernel(const SweepAr
 // depend on which sweep ran: the register sweep's thread has sites s, s + block,
 // .. of a tile of block x spt, the bulk-copy sweep's l, l + block, .. of a unit of
 // rpu rows.
-__global__ void signal_kernel(const MemberDesc* __restrict__ members, int rows, int block, int spt,
-                              double2* __restrict__ out)
+__device__ __forceinline__ void signal_part(const MemberDesc& d, const float2* __restrict__ M, int rows, int block, int spt,
+                                            int part, int parts, double2* out)
 {
     __shared__ double2 sh[256];
-    const MemberDesc& d = members[blockIdx.x];
-    const float2* __restrict__ M = d.mout;
     const long long N = d.N;
     // units of a plane (rows != 0) or tiles of the whole grid
     const long long span = rows ? (long long)d.nx * d.ny : N;
     const int unit = rows ? d.rpu * d.nx : block * spt;
     const long long per = (span + unit - 1) / unit, n_units = per * (N / span);
     double2 v = make_double2(0.0, 0.0);
-    for (long long u = blockIdx.y; u < n_units; u += gridDim.y) {
+    for (long long u = part; u < n_units; u += parts) {
         const long long s0 = (u / per) * span + (u % per) * unit, s1 = min(s0 + unit, (u / per + 1) * span);
         for (int t = threadIdx.x; t < block; t += 256) {
             float zr = 0.f, zi = 0.f;
@@ -480,10 +459,27 @@ __global__ void signal_kernel(const MemberDesc* __restrict__ members, int rows, 
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) out[(size_t)blockIdx.x * gridDim.y + blockIdx.y] = sh[0];
+    if (threadIdx.x == 0) *out = sh[0];
 }
 
-// series[m][k0 + n] = sum of the member's blocks' parts of step n (one warp each).
+__global__ void signal_kernel(const MemberDesc* __restrict__ members, int rows, int block, int spt,
+                              double2* __restrict__ out)
+{
+    const MemberDesc& d = members[blockIdx.x];
+    signal_part(d, d.mout, rows, block, spt, blockIdx.y, gridDim.y, out + (size_t)blockIdx.x * gridDim.y + blockIdx.y);
+}
+
+// The same of every step of a launch: blocks (member, part) x step.
+__global__ void series_part_kernel(const MemberDesc* __restrict__ members, int rows, int block, int spt, int parts,
+                                   const float2* __restrict__ mser, long long mstride, double2* __restrict__ zpart)
+{
+    const int m = blockIdx.x / parts, part = blockIdx.x - m * parts;
+    const MemberDesc& d = members[m];
+    signal_part(d, mser + (size_t)blockIdx.y * mstride + d.moff, rows, block, spt, part, parts,
+                zpart + (size_t)blockIdx.y * gridDim.x + blockIdx.x);
+}
+
+// series[m][k0 + n] = sum of the member's parts of step n (one warp each).
 __global__ void resident_series_kernel(const double2* __restrict__ zpart, const int* __restrict__ block_start,
                                        int n_members, int n_blocks, int n_steps, long long k0, long long stride,
                                        double2* __restrict__ series)
@@ -549,6 +545,14 @@ cudaError_t launch_signal(const MemberDesc* members, int n_members, bool rows, i
                           cudaStream_t st)
 {
     signal_kernel<<<dim3(n_members, parts), 256, 0, st>>>(members, rows ? 1 : 0, block, spt, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_series_parts(const MemberDesc* members, int n_members, bool rows, int block, int spt, int parts,
+                                const float2* mser, long long mstride, int n_steps, double2* zpart, cudaStream_t st)
+{
+    series_part_kernel<<<dim3((unsigned)(n_members * parts), (unsigned)n_steps), 256, 0, st>>>(members, rows ? 1 : 0, block, spt,
+                                                                                              parts, mser, mstride, zpart);
     return cudaGetLastError();
 }
 

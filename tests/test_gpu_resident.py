@@ -223,3 +223,22 @@ def test_resident_batches_of_many_members(lb, shapes, used):
             out.append([v.cpu().numpy() for v in fields])
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+# every step's signal is made of the one-step sweep's thread sums; free diffusion along x,
+# where the roundings of all rows are alike and add up; several launches (32 steps at
+# least of what 256 MB hold), blocks and strips, members of two sizes
+@pytest.mark.parametrize("shapes,lattice,n", [([(23, 41, 46)], 0, 60), ([(32, 32, 32)], 0, 60), ([(1, 500, 1000)], 1, 75),
+                                              ([(20, 24, 33), (7, 9, 10)], 0, 20), ([(1, 61, 90)], 1, 40)])
+def test_resident_series_is_the_one_step_series(lb, shapes, lattice, n):
+    geoms = [synth.Geometry(np.zeros(sh, np.int32), np.zeros(1, np.uint8), 1.0) for sh in shapes]
+    out = []
+    for multi in (0, 1):
+        with _solver(lb, multi, geoms, (0, 0, 0), (0.4, 0.0, 0.0), _wave("pgse", n), INF, lattice) as s:
+            m = lb.Solver.members([(0.4, 0.0, 0.0), (0.1, 0.0, 0.0)] * len(geoms), list(range(len(geoms))) * 2, INF)
+            r = s.run_batch(m, series=True)
+            assert s.get_option(lb.OPT_MULTI_STEP_USED) == (1 if multi else 3)
+            out.append(np.asarray(r["series"]))
+    assert np.abs(out[1]).min() > 0
+    strips = lattice == 1 and geoms[0].n_sites > 400000
+    assert np.abs(out[0] - out[1]).max() <= (2.0 ** -22 if strips else 1e-13) * max(g.n_sites for g in geoms)
