@@ -413,9 +413,12 @@ enum {
                                 where it can run; 3 resident where the grids
                                 fit.  Steps that lbmbt_advance makes one by one
                                 are one-step sweeps.  The fields are the same
-                                bits; where memory has no room for M, a
-                                two-step run's signals are summed in other
-                                groups (2^-22 of the sum of |M|)             */
+                                bits, and the signals the same numbers but for
+                                the order of their FP64 sums.  A two-step run's
+                                series and that of a 2-D grid above 311000
+                                sites, and a two-step run's signals where memory
+                                has no room for M, are summed in other groups
+                                (2^-22 of the sum of |M| at most)             */
     LBMBT_OPT_MULTI_STEP_USED = 19, /* read-only: 1, 2 or 3 for the prepared
                                 run, else 0                                  */
     LBMBT_OPT_TEST_FAIL_ALLOC = 20, /* tests of scarce memory only: n > 0 makes
