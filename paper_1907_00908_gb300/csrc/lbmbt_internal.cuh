@@ -115,8 +115,9 @@ struct MemberDesc {
 };
 // Where the extents and faces lie decides how every thread of the register sweep loads
 // them at its start: with nx .. pitch off a 16-byte word it took 0.4 us a step more (2-D,
-// 1400 x 1100: 48.9 us for 48.5); with pitch and mout after the rest, where that sweep was
-// as fast, the two-step sweep and the strips were 1 to 1.5 % slower.
+// 1400 x 1100: 48.9 us for 48.4); with pitch and mout after the rest, where that sweep was
+// as fast, the two-step sweep and the strips were 1 to 1.5 % slower.  That sweep is told
+// the alignment; told to all kernels, it made the bulk-copy adjoint 1.5 % slower.
 static_assert(offsetof(MemberDesc, nx) % 16 == 0 && offsetof(MemberDesc, pitch) == offsetof(MemberDesc, nx) + 12 &&
               offsetof(MemberDesc, bc) % 16 == 0 && sizeof(MemberDesc) % 16 == 0, "extents on one 16-byte word");
 

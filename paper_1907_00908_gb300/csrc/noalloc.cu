@@ -46,6 +46,7 @@ constexpr size_t OFF_PART = (OFF_FTAB + (NA_MAX_STEPS + 1) * 6 * sizeof(float2) 
 constexpr size_t NA_SCRATCH_BYTES = OFF_PART + NA_MAX_TILES * sizeof(double2);
 static_assert(sizeof(StepCtl) <= OFF_DESC - OFF_CTL, "control word does not fit");
 static_assert(sizeof(MemberDesc) <= OFF_TS - OFF_DESC, "descriptor does not fit");
+static_assert(OFF_DESC % 16 == 0, "the register sweep takes descriptors to lie on 16 bytes");
 // 2,754,304 bytes (2.63 MiB), the figure the header states
 static_assert(NA_SCRATCH_BYTES == 2754304, "scratch size differs from the documented figure");
 

@@ -135,7 +135,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& a)
     // Every thread looks up its member, step and flags itself (broadcast
     // loads): there is no per-block prologue to wait for.
     const int m = a.n_members == 1 ? 0 : find_member(a.tile_start, a.n_members, blockIdx.x);
-    const MemberDesc* __restrict__ sd = a.members + m;
+    // (16-byte loads of the descriptor, which every thread reads: see MemberDesc)
+    const MemberDesc* __restrict__ sd = static_cast<const MemberDesc*>(__builtin_assume_aligned(a.members + m, 16));
     const int k = __ldcg(&a.ctl->k);
     const int sbase = __ldcg(&a.ctl->slot_base), smod = __ldcg(&a.ctl->slot_mod);
     // a member with an end step of its own (shorter waveform in a batch)
@@ -152,8 +153,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs& a)
     const float2* __restrict__ src = sd->state + (size_t)((k - sbase) % smod) * 7 * P;
     float2* __restrict__ dst = sd->state + (size_t)((k + 1 - sbase) % smod) * 7 * P;
     const uint8_t* __restrict__ mask = sd->mask;
-    const int4 dim = *reinterpret_cast<const int4*>(&sd->nx);   // nx, ny, nz, pitch
-    const int nx = dim.x, ny = dim.y, nz = dim.z;
+    const int nx = sd->nx, ny = sd->ny, nz = sd->nz;
     const int bcx = sd->bc[0], bcy = sd->bc[1], bcz0 = sd->zbc[0], bcz1 = sd->zbc[1];
     const unsigned sxy = (unsigned)nx * ny;
     const unsigned N = (unsigned)sd->N;
